@@ -121,6 +121,9 @@ sbo_status sbo_create_maxkcut(int64_t n, int64_t m, const int32_t* ei, const int
  * CUDA graphs may leave the evaluation of its latest evaluation point pending (it then runs beside
  * the next block's iterations); sbo_sync, sbo_best, sbo_restart_best and sbo_trace complete it
  * first, so every result they report covers all evaluation points up to the current t.
+ * Where the library chooses the sparse form (SBO_OPT_CSR_FORM 0, default schedule) a sparse run of 8
+ * or more iterations may go through a kernel that keeps whole restarts on one SM, up to
+ * SBO_OPT_STEPS_PER_LAUNCH (0: 4,096) iterations per launch; results are identical.
  * sbo_gda: start (x0 = NULL) + run(prm->iters) + synchronise.  A handle may run again:
  * each start begins afresh. */
 sbo_status sbo_gda_start(sbo_problem* p, const sbo_gda_params* prm, const float* x0);

@@ -85,6 +85,7 @@ struct sbo_problem {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int sms = 0;
   int64_t l2_bytes = 0;
+  std::string dev_name;        // device part of the autotuners' keys (filled on first use)
   // dense
   void* A = nullptr;
   int64_t lda = 0;
@@ -97,6 +98,8 @@ struct sbo_problem {
   int64_t nnz = 0;
   int max_deg = 0;             // longest row of A (CSR)
   int res_nnz_max = 0;         // most nonzeros of A in one CTA's rows of the resident sparse form
+  void* rst_buf = nullptr;     // structure of the restart-resident runs (k_csr_restart.cu), null: not laid out
+  CsrRestartDev rst{};         // views into rst_buf
   int kparts = 0;              // Max-k-Cut: parts per vertex (FMT_MAXK)
   // linear term
   float* cp = nullptr;
@@ -116,6 +119,7 @@ struct sbo_problem {
   sbo_gda_params prm{};
   int kernel = KER_AUTO, layout = LAYOUT_RN, op_type = OP_F32, tile_n = 0;
   int csr_form = CSR_FORM_RULE;   // form of the sparse update in this run
+  int rst_R = 0;                  // restarts per CTA of the restart-resident runs (0: not used in this run)
   int B = 0;
   int64_t ld = 0;
   int64_t t = 0;          // iterations completed
@@ -201,6 +205,7 @@ void free_all(sbo_problem* p) {
   dfree(p->rowptr, p->stream);
   dfree(p->col, p->stream);
   dfree(p->val, p->stream);
+  dfree(p->rst_buf, p->stream);
   dfree(p->cp, p->stream);
   dfree(p->cp64, p->stream);
   dfree(p->err, p->stream);
@@ -472,6 +477,58 @@ sbo_status capture_block(sbo_problem* p, int parity, int kind) {
   return SBO_OK;
 }
 
+// Whether the next `iters` iterations run restart by restart (k_csr_restart.cu): the sparse form
+// was left to the library, and the launch's load and write-back of the state are spread over enough
+// iterations.  A request for single launches (graphs off, one iteration per launch) or for a
+// particular evaluation schedule keeps the row-wise kernels.
+constexpr int64_t RESTART_MIN_ITERS = 8;
+bool restart_runs(const sbo_problem* p, int64_t iters) {
+  return p->kernel == KER_CSR && p->rst_R > 0 && !p->single && p->opt_g == G_QUAD && p->opt_graph &&
+         p->opt_eval_mode == 0 && iters >= RESTART_MIN_ITERS &&
+         (p->opt_steps_per_launch == 0 || p->opt_steps_per_launch >= RESTART_MIN_ITERS);
+}
+
+sbo_status run_restart(sbo_problem* p, int64_t iters) {
+  sbo_status st = flush_pending(p);
+  if (st != SBO_OK) return st;
+  const int64_t per = p->opt_steps_per_launch == 0 ? 4096 : p->opt_steps_per_launch;
+  const int64_t K = p->prm.eval_every, T = p->prm.iters;
+  for (int64_t done = 0; done < iters;) {
+    const int64_t chunk = std::min(per, iters - done);
+    const int64_t t0 = p->t, t1 = p->t + chunk;
+    CsrRestartRun r;
+    r.t0 = t0;
+    r.K = K;
+    r.T = T;
+    r.e0 = p->n_evals_host;
+    r.iters = (int)chunk;
+    r.bestF = p->bestF;
+    r.bestT = p->bestT;
+    r.evalF = p->evalF;
+    r.trace = p->trace;
+    r.n_evals = p->n_evals;
+    r.t_last = p->t_last;
+    r.trace_cap = p->trace_cap;
+    r.bestBits = p->bestBits;
+    // evaluation points in (t0, t1]: the multiples of K, and T
+    const bool at_T = T > t0 && T <= t1;
+    r.n_evals_new = p->n_evals_host + t1 / K - t0 / K + (at_T && T % K != 0 ? 1 : 0);
+    r.t_last_new = p->t_last_eval;
+    if (t1 / K > t0 / K) r.t_last_new = t1 / K * K;
+    if (at_T) r.t_last_new = std::max<int64_t>(r.t_last_new, T);
+    void* x = p->Xop[p->cur];
+    cudaError_t e = launch_csr_restart(p->rst, base_args(p), p->op_type,
+                                       p->Xm ? p->Xm : static_cast<const float*>(x), x, r, p->rst_R, p->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "restart-resident launch");
+    ++p->launches;
+    p->t = t1;
+    p->n_evals_host = r.n_evals_new;
+    p->t_last_eval = r.t_last_new;
+    done += chunk;
+  }
+  return SBO_OK;
+}
+
 sbo_status run_tiny(sbo_problem* p, int64_t steps) {
   TinyArgs a;
   a.n = (int)p->n;
@@ -568,15 +625,22 @@ std::string tune_cache_path() {
   return home && *home ? std::string(home) + "/.cache/sbo/tile_tuning.txt" : std::string();
 }
 
-std::string tune_key(const sbo_problem* p) {
+// The device in a decision's key: its name and SM count.
+const std::string& tune_device(sbo_problem* p) {
+  if (!p->dev_name.empty()) return p->dev_name;
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceProp prop;
   std::string name = cudaGetDeviceProperties(&prop, dev) == cudaSuccess ? prop.name : "unknown";
   for (auto& ch : name)
     if (ch == ' ') ch = '_';
+  p->dev_name = name + ":sms" + std::to_string(p->sms);
+  return p->dev_name;
+}
+
+std::string tune_key(sbo_problem* p) {
   std::ostringstream k;
-  k << "v5:" << name << ":sms" << p->sms << ":n" << p->n << ":B" << p->B << ":split" << p->opt_split_k
+  k << "v5:" << tune_device(p) << ":n" << p->n << ":B" << p->B << ":split" << p->opt_split_k
     << (p->opt_steps_per_launch == 1 ? ":one" : "");
   return k.str();
 }
@@ -706,14 +770,8 @@ sbo_status tune_csr_form(sbo_problem* p, int* out) {
   static std::map<std::string, int> cache;
   std::string key;
   {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceProp prop;
-    std::string name = cudaGetDeviceProperties(&prop, dev) == cudaSuccess ? prop.name : "unknown";
-    for (auto& ch : name)
-      if (ch == ' ') ch = '_';
     std::ostringstream k;
-    k << "csr5:" << name << ":sms" << p->sms << ":n" << p->n << ":nnz" << p->nnz << ":deg" << p->max_deg << ":B"
+    k << "csr5:" << tune_device(p) << ":n" << p->n << ":nnz" << p->nnz << ":deg" << p->max_deg << ":B"
       << p->B << ":op" << p->op_type << ":g" << p->opt_g;
     key = k.str();
   }
@@ -800,6 +858,101 @@ sbo_status tune_csr_form(sbo_problem* p, int* out) {
     tune_cache_store(key, best);
   }
   *out = best;
+  return SBO_OK;
+}
+
+// Autotuner of the restart-resident runs: times `update` iterations of the row-wise form in use and of
+// the resident kernel with 1, 2 and 4 restarts per CTA (the difference of a long and a short launch,
+// which leaves out the load and write-back of the state), on this run's buffers before x^0 is
+// written.  *R gets the fastest's restarts per CTA, or 0 for the row-wise kernels.  Kept like the
+// other decisions.
+sbo_status tune_restart(sbo_problem* p, int* R) {
+  static std::mutex mu;
+  static std::map<std::string, int> cache;
+  std::ostringstream k;
+  k << "rst1:" << tune_device(p) << ":n" << p->n << ":nnz" << p->nnz << ":deg" << p->max_deg << ":grp"
+    << p->rst.shape.groups << ":B" << p->B << ":op" << p->op_type;
+  const std::string key = k.str();
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find(key);
+    if (it != cache.end()) { *R = it->second; return SBO_OK; }
+    int t = 0;
+    if (tune_cache_lookup(key, &t, [](int v) { return v == 0 || v == 1 || v == 2 || v == 4; }) &&
+        (t == 0 || csr_restart_fits(p->rst.shape, t))) {
+      cache[key] = t;
+      *R = t;
+      return SBO_OK;
+    }
+  }
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  SBO_CUDA(cudaEventCreate(&e0));
+  SBO_CUDA(cudaEventCreate(&e1));
+  CsrRestartRun r;
+  std::memset(&r, 0, sizeof(r));
+  r.K = r.T = INT64_MAX / 2;   // no evaluation
+  r.bestF = p->bestF;
+  r.bestT = p->bestT;
+  r.evalF = p->evalF;
+  r.trace = p->trace;
+  r.n_evals = p->n_evals;
+  r.t_last = p->t_last;
+  r.trace_cap = p->trace_cap;
+  r.bestBits = p->bestBits;
+  const EpiArgs a = base_args(p);
+  cudaError_t e = cudaSuccess;
+  // device time of launch() in ms, the better of two
+  auto timed = [&](auto&& launch) {
+    float best = 1e30f;
+    for (int round = 0; round < 2 && e == cudaSuccess; ++round) {
+      if (e == cudaSuccess) e = cudaEventRecord(e0, p->stream);
+      if (e == cudaSuccess) e = launch();
+      if (e == cudaSuccess) e = cudaEventRecord(e1, p->stream);
+      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+      float ms = 0.f;
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+      best = std::min(best, ms);
+    }
+    return best;
+  };
+  const int reps = 16;
+  int par = 0;
+  float best_ms = timed([&] {
+                    cudaError_t q = cudaSuccess;
+                    for (int it = 0; it < reps && q == cudaSuccess; ++it, par ^= 1) {
+                      EpiArgs b = a;
+                      b.Xin = p->Xop[par];
+                      b.Xout = p->Xop[par ^ 1];
+                      q = contract(p, b, EPI_UPDATE, par, p->stream);
+                    }
+                    return q;
+                  }) / reps;
+  int best = 0;
+  for (int cand : {1, 2, 4}) {
+    if (e != cudaSuccess || !csr_restart_fits(p->rst.shape, cand)) continue;
+    auto run = [&](int iters) {
+      return timed([&] {
+        r.iters = iters;
+        ++p->launches;
+        return launch_csr_restart(p->rst, a, p->op_type, p->Xm ? p->Xm : static_cast<float*>(p->Xop[0]), p->Xop[0], r,
+                                  cand, p->stream);
+      });
+    };
+    const float lo = run(reps), hi = run(3 * reps);
+    const float ms = (hi - lo) / (2 * reps);
+    if (e == cudaSuccess && ms < best_ms) { best_ms = ms; best = cand; }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (e != cudaSuccess) return cuda_fail(e, "restart autotuner launch");
+  sbo_status st = read_err(p);
+  if (st != SBO_OK) return st;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    cache[key] = best;
+    tune_cache_store(key, best);
+  }
+  *R = best;
   return SBO_OK;
 }
 
@@ -1079,6 +1232,36 @@ sbo_status sbo_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const i
       (e = cudaMemcpy(p->cp, cpf.data(), sizeof(float) * n, cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(p->cp64, cp.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice)) != cudaSuccess)
     return bail(cuda_fail(e, "upload CSR"));
+  CsrRestartHost rh;
+  if (csr_restart_build(n, rp.data(), cc.data(), vv.data(), cp.data(), &rh)) {
+    // one buffer: group streams (16-byte groups), c' exact, then the 4-byte tables and the group counts
+    const size_t b_ent = rh.ent.size() * 4, b_c64 = rh.cpp64.size() * 8, b_ws = rh.wstart.size() * 4,
+                 b_perm = rh.perm.size() * 4, b_cp = rh.cpp.size() * 4, b_w = rh.ngroups.size();
+    std::vector<uint8_t> img(b_ent + b_c64 + b_ws + b_perm + b_cp + b_w);
+    size_t off = 0;
+    auto put = [&](const void* src, size_t bytes) {
+      std::memcpy(img.data() + off, src, bytes);
+      off += bytes;
+      return off - bytes;
+    };
+    const size_t o_ent = put(rh.ent.data(), b_ent), o_c64 = put(rh.cpp64.data(), b_c64),
+                 o_ws = put(rh.wstart.data(), b_ws), o_perm = put(rh.perm.data(), b_perm),
+                 o_cp = put(rh.cpp.data(), b_cp), o_w = put(rh.ngroups.data(), b_w);
+    uint8_t* dev = nullptr;
+    if ((e = dalloc(&dev, img.size(), cs)) != cudaSuccess)
+      return bail(e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation failed") : cuda_fail(e, "cudaMalloc"));
+    p->rst_buf = dev;
+    if ((e = cudaStreamSynchronize(cs)) != cudaSuccess ||
+        (e = cudaMemcpy(dev, img.data(), img.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+      return bail(cuda_fail(e, "upload CSR"));
+    p->rst.shape = rh.shape;
+    p->rst.ent = reinterpret_cast<uint32_t*>(dev + o_ent);
+    p->rst.cpp64 = reinterpret_cast<int64_t*>(dev + o_c64);
+    p->rst.wstart = reinterpret_cast<uint32_t*>(dev + o_ws);
+    p->rst.perm = reinterpret_cast<int32_t*>(dev + o_perm);
+    p->rst.cpp = reinterpret_cast<float*>(dev + o_cp);
+    p->rst.ngroups = dev + o_w;
+  }
   *out = p;
   return SBO_OK;
 }
@@ -1372,7 +1555,9 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
     p->tile_n = 0;
   }
   p->csr_form = CSR_FORM_RULE;
+  p->rst_R = 0;
   if (ker == KER_CSR && !p->single) {
+
     // grid barrier words of the resident form (allocated before the autotuner, which times it)
     if ((e = dalloc(&p->tc_gbar, 3, s)) != cudaSuccess ||
         (e = cudaMemsetAsync(p->tc_gbar, 0, 3 * sizeof(unsigned int), s)) != cudaSuccess) {
@@ -1386,6 +1571,14 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
       sbo_status st2 = tune_csr_form(p, &f);   // on the zeroed state, before x^0 is written
       if (st2 != SBO_OK) { free_run(p); return st2; }
       p->csr_form = f;
+    }
+    if (p->rst_buf && p->opt_csr_form == 0 && p->opt_g == G_QUAD && !p->opt_keep_grad) {
+      if (p->opt_autotune) {
+        sbo_status st2 = tune_restart(p, &p->rst_R);   // on the zeroed state, before x^0 is written
+        if (st2 != SBO_OK) { free_run(p); return st2; }
+      } else {
+        p->rst_R = csr_restart_pick(p->rst.shape, p->B, p->sms);
+      }
     }
     int D, S, rc;
     size_t sm;
@@ -1443,6 +1636,7 @@ sbo_status sbo_gda_run(sbo_problem* p, int64_t iters) {
   if (iters < 0) return fail(SBO_EINVAL, "iters must be >= 0");
   if (iters == 0) return SBO_OK;
   if (p->kernel == KER_TINY) return run_tiny(p, iters);
+  if (restart_runs(p, iters)) return run_restart(p, iters);
   const int64_t K = p->prm.eval_every;
   const int64_t t_end = p->t + iters;
   while (p->t < t_end) {

@@ -1,0 +1,481 @@
+// Sparse runs, restart by restart: a CTA owns R restarts of the whole graph and runs many iterations
+// of Algorithm 1 on them without leaving the SM.
+//
+// The restarts are independent, so the only thing an iteration shares between SMs in the row-wise
+// kernels (k_csr.cu) is an artefact of splitting the rows over them: every iteration there reads
+// and writes all of x and y through L2 or HBM and ends at a kernel boundary.  Here a CTA keeps, for
+// its R restarts, x^t and x^{t+1} of every vertex in shared memory (two FP32 buffers that swap) and
+// y and c' in the registers of the thread that owns the vertex; an iteration gathers neighbours from
+// shared memory and ends at one __syncthreads.  Evaluations (candidate bits, exact integer
+// objective, best record) stay in the CTA too, so a run of T iterations is ceil(T / 4096) launches
+// and no graph replay.  State is read from and written back to global memory once per launch.
+//
+// Same arithmetic in the same order as k_csr: each row's neighbours are summed in ascending column
+// order with FP32 fused multiply-adds, from the FP32 x or (BF16 / E4M3 weights) from x rounded to
+// BF16, so iterates and records are bit-identical to every other form.
+//
+// Structure: vertices are placed by descending degree (stable) at positions 0, 1, ..; 32 consecutive
+// positions form a slice, one lane each.  Warp w owns slices w, w + 32, ... and walks one stream of
+// 16-byte groups: four neighbours of each lane's row, an entry holding the neighbour's position (low
+// 16 bits) and the weight as BF16 (high 16 bits: the float's bits), rows padded to whole
+// groups of the longest of their slice with weight 0.  The stream is read from shared memory when it fits beside x, else
+// through L1 / L2, two groups ahead of its use.
+//
+// What bounds it: shared-memory wavefronts of the gathers (a random graph's 32 4-byte gathers meet
+// about 3.5 bank conflicts deep) and the latency of the streams from L2, not HBM or the launch.
+// Measured per iteration against the row-wise kernels, evaluations every 10 included: Max-Cut ER
+// n = 2,000, B = 256 5.4 -> 2.44 us; 100 x 100 torus, B = 512 16.0 -> 9.4 us; 4-regular n = 20,000,
+// B = 512 38.6 -> 33.4 us.
+#include <algorithm>
+#include <cstring>
+
+#include "sbo_internal.h"
+
+namespace sbo {
+namespace {
+
+constexpr int RST_THREADS = 1024;
+constexpr int RST_SPARE = 2;   // groups a warp reads ahead of their use
+constexpr int RST_WARPS = RST_THREADS / 32;
+constexpr size_t RST_SMEM_MAX = 225 * 1024;   // dynamic; the static arrays take up to 1.2 KB of the 227
+
+struct RestartParams {
+  EpiArgs a;
+  const uint4* ent;              // group streams (global)
+  const uint32_t* wstart;        // [33] first group (of 32 uint4) of each warp's stream, and the end
+  const uint8_t* ngroups;        // [slices] groups of each slice
+  const int32_t* perm;           // [n] vertex at a position
+  const float* cpp;              // [positions] c' by position (0 beyond n)
+  const int64_t* cpp64;
+  const float* xsrc;             // FP32 x^{t0} ([i ld + r])
+  void* xop;                     // operand written at the end (FP32 or BF16), and Xm when set
+  int slices, ent_in_smem;
+  int64_t t0, K, T, e0;          // iterations t0 + 1 .. t0 + iters; evaluate at multiples of K and at T
+  int iters;
+  long long *bestF, *bestT, *evalF, *trace, *n_evals, *t_last;
+  long long trace_cap, t_last_new, n_evals_new;
+  uint8_t* bestBits;
+};
+
+// x of R restarts of one position, as the contraction sees it (BF16: rounded to nearest).
+template <int R, bool BF16>
+__device__ __forceinline__ void gather(const float* __restrict__ xc, uint32_t e, float (&acc)[R]) {
+  const float w = __uint_as_float(e & 0xffff0000u);
+  const float* p = xc + (e & 0xffffu) * R;
+  float v[R];
+  if (R == 1) {
+    v[0] = *p;
+  } else if (R == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(p);
+    v[0] = t.x; v[R - 1] = t.y;
+  } else {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x; v[1 % R] = t.y; v[2 % R] = t.z; v[3 % R] = t.w;
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (BF16) v[r] = __bfloat162float(__float2bfloat16_rn(v[r]));
+    acc[r] = fmaf(w, v[r], acc[r]);
+  }
+}
+
+template <int R>
+__device__ __forceinline__ void add_bits(const uint8_t* bb, uint32_t e, float (&acc)[R]) {
+  const float w = __uint_as_float(e & 0xffff0000u);
+  const uint32_t m = bb[e & 0xffffu];
+#pragma unroll
+  for (int r = 0; r < R; ++r) acc[r] += ((m >> r) & 1u) ? w : 0.0f;
+}
+
+// One iteration's work on one vertex after its neighbour sums: update of R restarts.
+template <int R>
+__device__ __forceinline__ uint32_t update(const EpiArgs& a, const float* xc, float* xn, const float (&acc)[R], float cp,
+                                           float (&y)[R]) {
+  uint32_t m = 0u;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const float x = xc[r];
+    const float gx = g_val(x, G_QUAD);
+    const float d = acc[r] + cp + y[r] * g_der(x, G_QUAD);
+    // pdbo_update (common.cuh) with the projection as a saturation: the same value
+    const bool stagnating = fabsf(x - 0.5f) <= a.delta && fabsf(d) <= a.grad_tol && y[r] <= 0.0f;
+    float xv = __saturatef(x - a.alpha * d);
+    if (stagnating) xv = x <= 0.5f ? 0.5f - a.delta : 0.5f + a.delta;
+    y[r] = y[r] + a.beta * gx;
+    xn[r] = xv;
+    m |= (xv > 0.5f ? 1u : 0u) << r;
+  }
+  return m;
+}
+
+// Q: slices per warp at most (y and c' of a thread's vertices live in registers: Q R + Q, or Q R + Q / 2
+// with c' packed as BF16 pairs when PACK).  R: restarts per CTA.  ONE: every row has at most four
+// neighbours (one group per slice).
+template <int Q, int R, bool BF16, bool ONE, bool PACK>
+__global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_constant__ RestartParams P) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int npos = P.slices * 32;
+  float* xs = reinterpret_cast<float*>(smem);                          // [2][npos][R]
+  uint4* ent_s = reinterpret_cast<uint4*>(xs + 2 * (size_t)npos * R);  // group streams (when they fit)
+  const uint32_t groups = P.wstart[RST_WARPS];
+  const size_t ent_bytes = P.ent_in_smem ? ((size_t)groups + RST_SPARE) * 32 * sizeof(uint4) : 0;
+  uint8_t* bb = reinterpret_cast<uint8_t*>(ent_s) + ent_bytes;         // candidate bits, one per restart
+  uint8_t* best = bb + npos;                                           // bits of the best candidates
+  uint8_t* ngr = best + npos;                                          // groups of each slice
+  __shared__ long long red[RST_WARPS][R];
+  __shared__ long long s_bestF[R], s_bestT[R];
+  __shared__ uint32_t s_improved, s_any;
+
+  const EpiArgs& a = P.a;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = a.n;
+  const int r0 = (int)blockIdx.x * R;
+  const int nlive = min(R, a.B - r0);
+
+  if (P.ent_in_smem)
+    for (uint32_t k = threadIdx.x; k < (groups + RST_SPARE) * 32; k += RST_THREADS) ent_s[k] = P.ent[k];
+  for (int k = threadIdx.x; k < P.slices; k += RST_THREADS) ngr[k] = P.ngroups[k];
+  if (threadIdx.x < R) {
+    const bool live = (int)threadIdx.x < nlive;
+    s_bestF[threadIdx.x] = live ? P.bestF[r0 + threadIdx.x] : 0;
+    s_bestT[threadIdx.x] = live ? P.bestT[r0 + threadIdx.x] : 0;
+  }
+  if (threadIdx.x == 0) s_any = 0u;
+
+  constexpr int NC = PACK ? (Q + 1) / 2 : Q;
+  float y[Q][R], cps[PACK ? 1 : NC];
+  uint32_t cpk[PACK ? NC : 1];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    if (PACK) cpk[PACK ? q : 0] = 0u;
+    else cps[PACK ? 0 : q] = 0.0f;
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int s = warp + q * RST_WARPS;
+#pragma unroll
+    for (int r = 0; r < R; ++r) y[q][r] = 0.0f;
+    if (s < P.slices) {
+      const int p = s * 32 + lane;
+      float x[R], c = 0.0f;
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = 0.0f;
+      if (p < n) {
+        const int64_t idx = (int64_t)P.perm[p] * a.ld + r0;
+        c = P.cpp[p];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (r < nlive) {
+            x[r] = P.xsrc[idx + r];
+            y[q][r] = a.Y[idx + r];
+          }
+      }
+      if (PACK) cpk[PACK ? q / 2 : 0] |= (q & 1) ? (__float_as_uint(c) & 0xffff0000u) : (__float_as_uint(c) >> 16);
+      else cps[PACK ? 0 : q] = c;
+#pragma unroll
+      for (int r = 0; r < R; ++r) xs[(size_t)p * R + r] = x[r];
+    }
+  }
+  __syncthreads();
+
+  const uint4* stream0 = (P.ent_in_smem ? ent_s : P.ent) + (size_t)P.wstart[warp] * 32 + lane;
+  int64_t e_idx = P.e0;
+  int64_t next_eval = (P.t0 / P.K + 1) * P.K;
+  if (P.T > P.t0 && P.T < next_eval) next_eval = P.T;
+  const float* xc = xs;
+  float* xn = xs + (size_t)npos * R;
+  const int p0 = warp * 32 + lane;   // this thread's vertices: positions p0, p0 + RST_THREADS, ..
+  for (int it = 1; it <= P.iters; ++it) {
+    const bool is_eval = P.t0 + it == next_eval;
+    const uint4* st = stream0;
+    uint4 nx[RST_SPARE];   // groups read ahead (the streams end in RST_SPARE spare groups)
+#pragma unroll
+    for (int d = 0; d < RST_SPARE; ++d, st += 32) nx[d] = *st;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      if (warp + q * RST_WARPS < P.slices) {
+        const int p = p0 + q * RST_THREADS;
+        float acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+        const int ng = ONE ? 1 : ngr[warp + q * RST_WARPS];
+        for (int g = 0; g < ng; ++g) {
+          const uint4 c = nx[0];
+#pragma unroll
+          for (int d = 0; d + 1 < RST_SPARE; ++d) nx[d] = nx[d + 1];
+          nx[RST_SPARE - 1] = *st;
+          st += 32;
+          gather<R, BF16>(xc, c.x, acc);
+          gather<R, BF16>(xc, c.y, acc);
+          gather<R, BF16>(xc, c.z, acc);
+          gather<R, BF16>(xc, c.w, acc);
+        }
+        const float cp = !PACK ? cps[PACK ? 0 : q]
+                               : __uint_as_float((q & 1) ? cpk[PACK ? q / 2 : 0] & 0xffff0000u : cpk[PACK ? q / 2 : 0] << 16);
+        const uint32_t m = update<R>(a, xc + (size_t)p * R, xn + (size_t)p * R, acc, cp, y[q]);
+        if (is_eval) bb[p] = (uint8_t)m;
+      }
+    }
+    {
+      float* t = const_cast<float*>(xc);
+      xc = xn;
+      xn = t;
+    }
+    __syncthreads();
+    if (!is_eval) continue;
+
+    // exact objective of the candidates: 2F = sum_i b_i ((A b)_i + 2 c'_i); (A b)_i is an exact
+    // integer in FP32 because every row sum of |A| is below 2^24
+    long long f2[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) f2[r] = 0;
+    st = stream0;
+    for (int s = warp; s < P.slices; s += RST_WARPS) {
+      const int ng = ONE ? 1 : ngr[s];
+      const int p = s * 32 + lane;
+      float acc[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+      for (int g = 0; g < ng; ++g, st += 32) {
+        const uint4 c = *st;   // entries beyond a row's length are padding (weight 0)
+        add_bits<R>(bb, c.x, acc);
+        add_bits<R>(bb, c.y, acc);
+        add_bits<R>(bb, c.z, acc);
+        add_bits<R>(bb, c.w, acc);
+      }
+      if (p < n) {
+        const uint32_t m = bb[p];
+        const long long c2 = 2 * (long long)P.cpp64[p];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if ((m >> r) & 1u) f2[r] += (long long)acc[r] + c2;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) f2[r] += __shfl_xor_sync(0xffffffffu, f2[r], o);
+      if (lane == 0) red[warp][r] = f2[r];
+    }
+    if (threadIdx.x == 0) s_improved = 0u;
+    __syncthreads();
+    if (threadIdx.x < R) {
+      const int r = threadIdx.x;
+      long long sum = 0;
+#pragma unroll 4
+      for (int w = 0; w < RST_WARPS; ++w) sum += red[w][r];
+      if (r < nlive) {
+        const long long F = sum / 2;
+        if (F < s_bestF[r]) {   // strict: equal values keep the earliest t
+          s_bestF[r] = F;
+          s_bestT[r] = P.t0 + it;
+          atomicOr(&s_improved, 1u << r);
+        }
+        P.evalF[r0 + r] = F;
+        if (e_idx < P.trace_cap) atomicMin(&P.trace[e_idx], F);
+      }
+    }
+    __syncthreads();
+    const uint32_t imp = s_improved;
+    if (imp) {
+      for (int s = warp; s < P.slices; s += RST_WARPS) {
+        const int p = s * 32 + lane;
+        best[p] = (uint8_t)((best[p] & ~imp) | (bb[p] & imp));
+      }
+      if (threadIdx.x == 0) s_any |= imp;
+    }
+    ++e_idx;
+    next_eval = ((P.t0 + it) / P.K + 1) * P.K;
+    if (P.T > P.t0 + it && P.T < next_eval) next_eval = P.T;
+  }
+  __syncthreads();
+
+  // write back: x, y and the operand of the next iteration, and the best records that changed
+  const uint32_t any = s_any;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int p = p0 + q * RST_THREADS;
+    if (p >= n) continue;
+    const int64_t idx = (int64_t)P.perm[p] * a.ld + r0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (r >= nlive) continue;
+      const float x = xc[(size_t)p * R + r];
+      a.Y[idx + r] = y[q][r];
+      if (BF16) {
+        a.Xm[idx + r] = x;
+        static_cast<__nv_bfloat16*>(P.xop)[idx + r] = __float2bfloat16_rn(x);
+      } else {
+        static_cast<float*>(P.xop)[idx + r] = x;
+      }
+      if ((any >> r) & 1u) P.bestBits[idx + r] = (best[p] >> r) & 1u;
+    }
+  }
+  if ((int)threadIdx.x < nlive && ((any >> threadIdx.x) & 1u)) {
+    P.bestF[r0 + threadIdx.x] = s_bestF[threadIdx.x];
+    P.bestT[r0 + threadIdx.x] = s_bestT[threadIdx.x];
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *P.n_evals = P.n_evals_new;
+    *P.t_last = P.t_last_new;
+  }
+}
+
+using RestartKernel = void (*)(RestartParams);
+
+template <int Q, int R, bool PACK>
+RestartKernel kernel_of(bool bf16, bool one) {
+  if (one) return bf16 ? (RestartKernel)k_csr_restart<Q, R, true, true, PACK> : (RestartKernel)k_csr_restart<Q, R, false, true, PACK>;
+  return bf16 ? (RestartKernel)k_csr_restart<Q, R, true, false, PACK> : (RestartKernel)k_csr_restart<Q, R, false, false, PACK>;
+}
+
+// Instantiations: slices per warp up to Q with R restarts, in 64 registers per thread.
+RestartKernel pick_kernel(const CsrRestartShape& sh, int R, bool bf16) {
+  const int q = (sh.slices + RST_WARPS - 1) / RST_WARPS;
+  const bool one = sh.max_groups <= 1;
+  switch (R) {
+    case 1:
+      if (q <= 3) return kernel_of<3, 1, false>(bf16, one);
+      if (q <= 10) return kernel_of<10, 1, false>(bf16, one);
+      return q <= 20 && sh.cp_bf16 ? kernel_of<20, 1, true>(bf16, one) : nullptr;
+    case 2: return q <= 3 ? kernel_of<3, 2, false>(bf16, one) : q <= 10 ? kernel_of<10, 2, false>(bf16, one) : nullptr;
+    case 4: return q <= 5 ? kernel_of<5, 4, false>(bf16, one) : nullptr;
+    default: return nullptr;
+  }
+}
+
+size_t smem_bytes(const CsrRestartShape& sh, int R, bool ent) {
+  const size_t npos = (size_t)sh.slices * 32;
+  return 8 * npos * R + 2 * npos + (size_t)sh.slices + 16 + (ent ? ((size_t)sh.groups + RST_SPARE) * 512 : 0);
+}
+
+}  // namespace
+
+bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
+                       CsrRestartHost* out) {
+  if (n < 1 || n > 20 * RST_THREADS) return false;
+  int maxd = 0;
+  for (int64_t i = 0; i < n; ++i) maxd = std::max(maxd, rp[i + 1] - rp[i]);
+  if (maxd > CSR_RESTART_MAX_DEG) return false;
+  for (int64_t e = 0; e < rp[n]; ++e)
+    if (val[e] > 256 || val[e] < -256) return false;   // not exact in BF16
+  // positions by descending degree, equal degrees in vertex order
+  const int slices = (int)((n + 31) / 32);
+  std::vector<int32_t> first((size_t)maxd + 2, 0), perm((size_t)n), pos((size_t)n);
+  for (int64_t i = 0; i < n; ++i) ++first[(size_t)(maxd - (rp[i + 1] - rp[i])) + 1];
+  for (int d = 0; d <= maxd; ++d) first[(size_t)d + 1] += first[(size_t)d];
+  for (int64_t i = 0; i < n; ++i) {
+    const int32_t p = first[(size_t)(maxd - (rp[i + 1] - rp[i]))]++;
+    perm[(size_t)p] = (int32_t)i;
+    pos[(size_t)i] = p;
+  }
+  out->ngroups.assign((size_t)slices, 0);
+  // The first of a slice has its largest degree.  The kernel's ONE form walks exactly one group per
+  // slice, so with no row above four neighbours slices of isolated vertices hold one (padding) too.
+  for (int s = 0; s < slices; ++s) {
+    const int32_t i = perm[(size_t)s * 32];
+    out->ngroups[(size_t)s] = (uint8_t)std::max((rp[i + 1] - rp[i] + 3) / 4, maxd <= 4 ? 1 : 0);
+  }
+  uint32_t groups = 0;
+  out->wstart.assign(RST_WARPS + 1, 0);
+  for (int w = 0; w < RST_WARPS; ++w) {
+    out->wstart[(size_t)w] = groups;
+    for (int s = w; s < slices; s += RST_WARPS) groups += out->ngroups[(size_t)s];
+  }
+  out->wstart[RST_WARPS] = groups;
+  out->ent.assign(((size_t)groups + RST_SPARE) * 128, 0u);
+  for (int w = 0; w < RST_WARPS; ++w) {
+    size_t g = out->wstart[(size_t)w];
+    for (int s = w; s < slices; s += RST_WARPS) {
+      const int gr = out->ngroups[(size_t)s];
+      for (int l = 0; l < 32; ++l) {
+        const int64_t p = (int64_t)s * 32 + l;
+        const int64_t i = p < n ? perm[(size_t)p] : -1;
+        const int deg = i >= 0 ? rp[i + 1] - rp[i] : 0;
+        for (int k = 0; k < 4 * gr; ++k) {
+          uint32_t e = (uint32_t)p;   // padding gathers its own position with weight 0
+          if (k < deg) {
+            const float w32 = (float)val[rp[i] + k];
+            uint32_t bits;
+            std::memcpy(&bits, &w32, 4);
+            e = bits | (uint32_t)pos[(size_t)col[rp[i] + k]];   // |w| <= 256: the low 16 bits are zero
+          }
+          out->ent[(g + (size_t)(k / 4)) * 128 + (size_t)l * 4 + (k & 3)] = e;
+        }
+      }
+      g += (size_t)gr;
+    }
+  }
+  out->perm = std::move(perm);
+  out->cpp.assign((size_t)slices * 32, 0.0f);
+  out->cpp64.assign((size_t)slices * 32, 0);
+  for (int64_t p = 0; p < n; ++p) {
+    out->cpp64[(size_t)p] = cp[out->perm[(size_t)p]];
+    const float c = (float)out->cpp64[(size_t)p];
+    out->cpp[(size_t)p] = c;
+    uint32_t bits;
+    std::memcpy(&bits, &c, 4);
+    if (bits & 0xffffu) out->shape.cp_bf16 = false;
+  }
+  out->shape.slices = slices;
+  out->shape.groups = groups;
+  out->shape.max_groups = std::max(1, (maxd + 3) / 4);
+  return true;
+}
+
+bool csr_restart_fits(const CsrRestartShape& sh, int R) {
+  return pick_kernel(sh, R, false) != nullptr && smem_bytes(sh, R, false) <= RST_SMEM_MAX;
+}
+
+int csr_restart_pick(const CsrRestartShape& sh, int B, int sms) {
+  int best = 0;
+  double best_cost = 0.0;
+  for (int R : {1, 2, 4}) {
+    if (!csr_restart_fits(sh, R)) continue;
+    const int64_t ctas = (B + R - 1) / R;
+    const double cost = (double)((ctas + sms - 1) / sms) * (1.0 + R);
+    if (best == 0 || cost < best_cost) { best = R; best_cost = cost; }
+  }
+  return best;
+}
+
+cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_type, const float* xsrc, void* xop,
+                               const CsrRestartRun& run, int R, cudaStream_t s) {
+  RestartKernel k = pick_kernel(d.shape, R, op_type == OP_BF16);
+  if (!k || run.iters < 1) return cudaErrorInvalidValue;
+  RestartParams P;
+  std::memset(&P, 0, sizeof(P));
+  P.a = a;
+  P.ent = reinterpret_cast<const uint4*>(d.ent);
+  P.wstart = d.wstart;
+  P.ngroups = d.ngroups;
+  P.perm = d.perm;
+  P.cpp = d.cpp;
+  P.cpp64 = d.cpp64;
+  P.xsrc = xsrc;
+  P.xop = xop;
+  P.slices = d.shape.slices;
+  P.ent_in_smem = smem_bytes(d.shape, R, true) <= RST_SMEM_MAX;
+  P.t0 = run.t0;
+  P.K = run.K;
+  P.T = run.T;
+  P.e0 = run.e0;
+  P.iters = run.iters;
+  P.bestF = run.bestF;
+  P.bestT = run.bestT;
+  P.evalF = run.evalF;
+  P.trace = run.trace;
+  P.trace_cap = run.trace_cap;
+  P.n_evals = run.n_evals;
+  P.t_last = run.t_last;
+  P.n_evals_new = run.n_evals_new;
+  P.t_last_new = run.t_last_new;
+  P.bestBits = run.bestBits;
+  const size_t sm = smem_bytes(d.shape, R, P.ent_in_smem != 0);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RST_SMEM_MAX);
+  if (e != cudaSuccess) return e;
+  k<<<(unsigned)((a.B + R - 1) / R), RST_THREADS, sm, s>>>(P);
+  return cudaGetLastError();
+}
+
+}  // namespace sbo

@@ -116,6 +116,47 @@ cudaError_t launch_csr_res(const int32_t* rowptr, const int32_t* col, const void
                            int op_type, int which_x, void* const xop[2], int iters, bool eval_last, int nnz_max,
                            int sms, unsigned int* gbar, uint64_t timeout_ns, cudaStream_t s);
 int csr_partial_rows(int64_t n, int B);
+// k_csr_restart.cu: whole runs with R restarts of the graph per CTA (state on chip between launches).
+// csr_restart_build lays the structure out (false: the graph does not fit the form: more than 20,480
+// vertices, a row longer than CSR_RESTART_MAX_DEG or a weight not exact in BF16); csr_restart_pick
+// gives the restarts per CTA for a run of B restarts.
+constexpr int CSR_RESTART_MAX_DEG = 256;
+struct CsrRestartShape {
+  int slices = 0;
+  uint32_t groups = 0;
+  int max_groups = 0;      // groups of the longest row
+  bool cp_bf16 = true;     // every c' is exact in BF16
+};
+struct CsrRestartHost {
+  CsrRestartShape shape;
+  std::vector<uint32_t> ent, wstart;
+  std::vector<uint8_t> ngroups;
+  std::vector<int32_t> perm;
+  std::vector<float> cpp;
+  std::vector<int64_t> cpp64;
+};
+struct CsrRestartDev {
+  CsrRestartShape shape;
+  uint32_t* ent = nullptr;
+  uint32_t* wstart = nullptr;
+  uint8_t* ngroups = nullptr;
+  int32_t* perm = nullptr;
+  float* cpp = nullptr;
+  int64_t* cpp64 = nullptr;
+};
+struct CsrRestartRun {
+  int64_t t0, K, T, e0;    // iterations t0 + 1 .. t0 + iters; e0: evaluations so far
+  int iters;
+  long long *bestF, *bestT, *evalF, *trace, *n_evals, *t_last;
+  long long trace_cap, n_evals_new, t_last_new;   // counters after the launch
+  uint8_t* bestBits;
+};
+bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
+                       CsrRestartHost* out);
+bool csr_restart_fits(const CsrRestartShape& sh, int R);   // an instantiation exists and x fits on chip
+int csr_restart_pick(const CsrRestartShape& sh, int B, int sms);
+cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_type, const float* xsrc, void* xop,
+                               const CsrRestartRun& run, int R, cudaStream_t s);
 // k_csr_staged.cu: the update with every row's operands staged in shared memory by bulk copies
 // (CSR_FORM_STAGED); max_deg is the largest row length of A.  csr_staged_shape reports its stage
 // layout and false when it does not apply (fewer than four stages fit).

@@ -1,0 +1,84 @@
+"""The restart-resident sparse runs (R restarts of the whole graph per CTA) against the row-wise
+kernels, which the oracle parity tests hold: the same sums in the same order, so iterates, records,
+traces and best candidates are equal bit for bit.  With the autotuner off every run of at least 8
+iterations takes the restart-resident kernel where the graph fits it; SBO_OPT_CSR_FORM = 1 is the
+row-wise side.  Sizes sit at the edges of its layout: slices of 32 vertices, 1,024 vertices per
+register slot (3, 5, 10 and 20 slots), rows of 0, 4, 5 and more neighbours, ragged restarts."""
+import numpy as np
+import pytest
+
+import workloads as W
+from paper_2509_21064_gb300 import sbo as S
+from paper_2509_21064_gb300.build import build as build_lib
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build_lib()
+    S.lib()
+
+
+def _graph(n, deg, seed, wmax=1):
+    """Random CSR QUBO (upper entries only, so A = Q + Q^T) with some isolated vertices, and c."""
+    rng = np.random.default_rng(seed)
+    m = max(1, n * deg // 2)
+    a, b = rng.integers(0, n, m), rng.integers(0, n, m)
+    keep = (a != b) & (a % 11 != 3) & (b % 11 != 3)
+    a, b = a[keep], b[keep]
+    key = np.unique(np.minimum(a, b) * n + np.maximum(a, b))
+    a, b = key // n, key % n
+    w = rng.integers(1, wmax + 1, a.size) * rng.choice([-1, 1], a.size)
+    rowptr = np.concatenate([[0], np.cumsum(np.bincount(a, minlength=n))])
+    return rowptr, b, w, rng.integers(-9, 10, n)
+
+
+def _run(n, csr, prec, prm, chunks, form):
+    rowptr, col, val, c = csr
+    with S.Problem.csr(n, rowptr, col, val, c, precision=prec) as P:
+        P.set_option(S.SBO_OPT_AUTOTUNE, 0)
+        P.set_option(S.SBO_OPT_CSR_FORM, form)
+        P.start(prm)
+        n0 = P.launch_count()
+        for k in chunks:
+            P.run(k)
+        P.sync()
+        launches = P.launch_count() - n0
+        X, Y = P.state()
+        return launches, (X, Y, *P.restart_best(), P.trace(), *P.best())
+
+
+def _same(n, csr, prec, B, K, T, chunks, resident=True):
+    prm = S.params(B, T, 0.025, 0.025, 1.0, eval_every=K, seed=5)
+    la, auto = _run(n, csr, prec, prm, chunks, S.CSR_FORM_AUTO)
+    lr, rows = _run(n, csr, prec, prm, chunks, S.CSR_FORM_ROW1)
+    for a, b in zip(auto, rows):
+        assert np.array_equal(a, b)
+    assert (la < lr) == resident, (la, lr)
+
+
+@pytest.mark.parametrize("prec", [S.SBO_FP32, S.SBO_BF16, S.SBO_FP8_E4M3])
+@pytest.mark.parametrize("n,deg,B", [(1, 1, 3), (31, 3, 1), (33, 8, 7), (1025, 6, 130), (3073, 5, 9), (5121, 3, 301),
+                                     (10240, 6, 305), (10241, 4, 17), (20480, 5, 3)])
+def test_restart_resident_runs_equal_the_row_wise_ones(n, deg, B, prec):
+    # 300 iterations at ybar = 1, beta = 0.025 pass through y = 0, where the perturbation rule acts
+    _same(n, _graph(n, deg, n, wmax=3), prec, B, 10, 303, [303])
+
+
+@pytest.mark.parametrize("K,T,chunks", [(1, 20, [20]), (7, 40, [9, 3, 12, 16]), (10, 25, [60]), (50, 30, [8, 8, 24])])
+def test_evaluation_points_and_split_runs(K, T, chunks):
+    """Evaluations at multiples of K and at T, runs split into calls (short ones on the row-wise
+    kernels, the best record shared between both) and continued past T."""
+    _same(700, _graph(700, 7, 1), S.SBO_FP32, 37, K, T, chunks)
+
+
+def test_degree_and_range_limits_fall_back():
+    n = 11000
+    star = (np.concatenate([[0], np.full(n, 300)]), np.arange(1, 301), np.ones(300, int), np.zeros(n, int))
+    _same(n, star, S.SBO_FP32, 5, 10, 30, [30], resident=False)             # a row of 300
+    heavy = _graph(n, 4, 2)
+    _same(n, (heavy[0], heavy[1], heavy[2] * 300, heavy[3]), S.SBO_FP32, 5, 10, 30, [30], resident=False)   # |A| > 256
+    _same(n, (*heavy[:3], heavy[3] * 1001), S.SBO_FP32, 5, 10, 30, [30], resident=False)   # c' not exact in BF16
+    _same(700, (*_graph(700, 4, 3)[:3], np.full(700, 1001)), S.SBO_FP32, 5, 10, 30, [30])  # small n keeps FP32 c'
+    _same(20481, _graph(20481, 3, 4), S.SBO_FP32, 2, 10, 30, [30], resident=False)
