@@ -351,6 +351,60 @@ size_t smem_bytes(const CsrRestartShape& sh, int R, bool ent) {
 
 }  // namespace
 
+// Lanes within the slices, chosen against bank conflicts.  The 32 gathers of one neighbour slot of a
+// slice fall on the banks of their vertices' lanes (position mod 32); which 32 vertices they are
+// depends on the slices only, so a vertex may move within its slice freely.  One greedy pass over the
+// vertices gives each the free lane of its slice that adds least to the squares of the bank loads of
+// the gathers it takes part in, its own lane where that is as good (a torus in natural order has no
+// conflicts and stays as it is).  Two restarts per CTA (graphs up to 10,240 vertices) gather 8 bytes
+// per lane in two half warps over 16 pairs of banks: there the vertices move within half slices.
+// Random 4-regular graph: 3.51 -> 2.05 wavefronts per 4-byte gather (n = 20,000, 3 ms of host time),
+// 6.15 -> 4.10 per 8-byte gather (n = 10,000, 1 ms).
+static void place_lanes(int64_t n, const int32_t* rp, const int32_t* col, std::vector<int32_t>& perm,
+                 std::vector<int32_t>& pos) {
+  const int BK = n > 10 * RST_THREADS ? 32 : 16;
+  const int64_t slices = (n + 31) / 32;
+  std::vector<int64_t> first((size_t)slices + 1, 0);   // gather sets (neighbour slots) before each slice
+  for (int64_t s = 0; s < slices; ++s) {
+    const int32_t i = perm[(size_t)s * 32];             // by descending degree: the longest row
+    first[(size_t)s + 1] = first[(size_t)s] + (rp[i + 1] - rp[i]);
+  }
+  std::vector<uint8_t> load((size_t)first[(size_t)slices] * 32, 0);   // vertices per (set, half, bank)
+  std::vector<int32_t> at((size_t)n + 1, 0);
+  std::vector<int64_t> occ((size_t)rp[n]);              // sets a vertex is gathered in
+  for (int32_t e = 0; e < rp[n]; ++e) ++at[(size_t)col[e] + 1];
+  for (int64_t i = 0; i < n; ++i) at[(size_t)i + 1] += at[(size_t)i];
+  {
+    std::vector<int32_t> next(at.begin(), at.end() - 1);
+    for (int64_t p = 0; p < n; ++p) {
+      const int32_t i = perm[(size_t)p];
+      const int64_t half = (p % 32) / BK * BK;
+      for (int k = 0; k < rp[i + 1] - rp[i]; ++k)
+        occ[(size_t)next[(size_t)col[rp[i] + k]]++] = (first[(size_t)(p / 32)] + k) * 32 + half;
+    }
+  }
+  for (int64_t p0 = 0; p0 < n; p0 += BK) {
+    const int cnt = (int)std::min<int64_t>(BK, n - p0);
+    int32_t v[32];
+    for (int l = 0; l < cnt; ++l) v[l] = perm[(size_t)(p0 + l)];
+    uint32_t free_lanes = cnt == 32 ? 0xffffffffu : (1u << cnt) - 1u;
+    for (int l = 0; l < cnt; ++l) {
+      uint32_t cost[32] = {};
+      for (int32_t o = at[(size_t)v[l]]; o < at[(size_t)v[l] + 1]; ++o) {
+        const uint8_t* L = &load[(size_t)occ[(size_t)o]];
+        for (int b = 0; b < BK; ++b) cost[b] += (uint32_t)L[b] * L[b];
+      }
+      int best = (free_lanes >> l) & 1u ? l : -1;
+      for (int b = 0; b < cnt; ++b)
+        if (((free_lanes >> b) & 1u) && (best < 0 || cost[b] < cost[best])) best = b;
+      free_lanes &= ~(1u << best);
+      perm[(size_t)(p0 + best)] = v[l];
+      pos[(size_t)v[l]] = (int32_t)(p0 + best);
+      for (int32_t o = at[(size_t)v[l]]; o < at[(size_t)v[l] + 1]; ++o) ++load[(size_t)occ[(size_t)o] + best];
+    }
+  }
+}
+
 bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
                        CsrRestartHost* out) {
   if (n < 1 || n > 20 * RST_THREADS) return false;
@@ -369,12 +423,14 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
     perm[(size_t)p] = (int32_t)i;
     pos[(size_t)i] = p;
   }
+  place_lanes(n, rp, col, perm, pos);
   out->ngroups.assign((size_t)slices, 0);
-  // The first of a slice has its largest degree.  The kernel's ONE form walks exactly one group per
-  // slice, so with no row above four neighbours slices of isolated vertices hold one (padding) too.
+  // The kernel's ONE form walks exactly one group per slice, so with no row above four neighbours slices of isolated vertices hold one (padding) too.
   for (int s = 0; s < slices; ++s) {
-    const int32_t i = perm[(size_t)s * 32];
-    out->ngroups[(size_t)s] = (uint8_t)std::max((rp[i + 1] - rp[i] + 3) / 4, maxd <= 4 ? 1 : 0);
+    int width = 0;
+    for (int64_t p = (int64_t)s * 32; p < std::min<int64_t>(n, (int64_t)(s + 1) * 32); ++p)
+      width = std::max(width, rp[perm[(size_t)p] + 1] - rp[perm[(size_t)p]]);
+    out->ngroups[(size_t)s] = (uint8_t)std::max((width + 3) / 4, maxd <= 4 ? 1 : 0);
   }
   uint32_t groups = 0;
   out->wstart.assign(RST_WARPS + 1, 0);
