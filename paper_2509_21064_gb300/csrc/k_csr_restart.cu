@@ -16,8 +16,8 @@
 //
 // Structure: vertices are placed by descending degree (stable) at positions 0, 1, ..; 32 consecutive
 // positions form a slice, one lane each.  Warp w owns slices w, w + 32, ... and walks one stream of
-// 16-byte groups: four neighbours of each lane's row, an entry holding the neighbour's position (low
-// 16 bits) and the weight as BF16 (high 16 bits: the float's bits), rows padded to whole
+// 16-byte groups: four neighbours of each lane's row, an entry holding the neighbour's place and its
+// weight (see ENT_W), rows padded to whole
 // groups of the longest of their slice with weight 0.  The stream is read from shared memory when it fits beside x, else
 // through L1 / L2, two groups ahead of its use.
 //
@@ -57,55 +57,88 @@ struct RestartParams {
   uint8_t* bestBits;
 };
 
-// x of R restarts of one position, as the contraction sees it (BF16: rounded to nearest).
-template <int R, bool BF16>
-__device__ __forceinline__ void gather(const float* __restrict__ xc, uint32_t e, float (&acc)[R]) {
-  const float w = __uint_as_float(e & 0xffff0000u);
-  const float* p = xc + (e & 0xffffu) * R;
-  float v[R];
-  if (R == 1) {
-    v[0] = *p;
-  } else if (R == 2) {
-    const float2 t = *reinterpret_cast<const float2*>(p);
-    v[0] = t.x; v[R - 1] = t.y;
-  } else {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x; v[1 % R] = t.y; v[2 % R] = t.z; v[3 % R] = t.w;
+// An entry of the streams: the neighbour's position, shifted so that masking gives the byte offset of
+// its x in a buffer of `base` restarts per position, and the weight's top 15 bits (sign, exponent and 6
+// bits of mantissa: every |w| <= 127, even ones to 254, and so on).
+constexpr uint32_t ENT_W = 0xfffe0000u;
+template <int R>
+__device__ __forceinline__ uint32_t entry_offset(uint32_t e, int base) {   // byte offset for R restarts
+  const uint32_t o = e & ~ENT_W;
+  if (R == 1) return base == 1 ? o : o >> 1;
+  return R == 2 ? o : o << 1;
+}
+
+// The four neighbours of one group: their x as the contraction sees it (BF16: rounded to nearest, two
+// values per conversion), added in order.
+template <int R, bool BF16, int BASE>
+__device__ __forceinline__ void gather4(const float* xc, const uint4& c, float (&acc)[R]) {
+  const uint32_t e[4] = {c.x, c.y, c.z, c.w};
+  float v[4][R];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const char* p = reinterpret_cast<const char*>(xc) + entry_offset<R>(e[k], BASE);
+    if (R == 1) {
+      v[k][0] = *reinterpret_cast<const float*>(p);
+    } else if (R == 2) {
+      const float2 t = *reinterpret_cast<const float2*>(p);
+      v[k][0] = t.x; v[k][R - 1] = t.y;
+    } else {
+      const float4 t = *reinterpret_cast<const float4*>(p);
+      v[k][0] = t.x; v[k][1 % R] = t.y; v[k][2 % R] = t.z; v[k][3 % R] = t.w;
+    }
+  }
+  if (BF16) {
+#pragma unroll
+    for (int j = 0; j < 4 * R; j += 2) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(v[j / R][j % R], v[(j + 1) / R][(j + 1) % R]);
+      v[j / R][j % R] = __low2float(h);
+      v[(j + 1) / R][(j + 1) % R] = __high2float(h);
+    }
   }
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    if (BF16) v[r] = __bfloat162float(__float2bfloat16_rn(v[r]));
-    acc[r] = fmaf(w, v[r], acc[r]);
+  for (int k = 0; k < 4; ++k) {
+    const float w = __uint_as_float(e[k] & ENT_W);
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = fmaf(w, v[k][r], acc[r]);
   }
 }
 
 template <int R>
-__device__ __forceinline__ void add_bits(const uint8_t* bb, uint32_t e, float (&acc)[R]) {
-  const float w = __uint_as_float(e & 0xffff0000u);
-  const uint32_t m = bb[e & 0xffffu];
+__device__ __forceinline__ void add_bits(const uint8_t* bb, uint32_t e, int shift, float (&acc)[R]) {
+  const float w = __uint_as_float(e & ENT_W);
+  const uint32_t m = bb[(e & ~ENT_W) >> shift];
 #pragma unroll
   for (int r = 0; r < R; ++r) acc[r] += ((m >> r) & 1u) ? w : 0.0f;
 }
 
 // One iteration's work on one vertex after its neighbour sums: update of R restarts.
 template <int R>
-__device__ __forceinline__ uint32_t update(const EpiArgs& a, const float* xc, float* xn, const float (&acc)[R], float cp,
-                                           float (&y)[R]) {
-  uint32_t m = 0u;
+__device__ __forceinline__ void update(const EpiArgs& a, const float* xc, float* xn, const float (&acc)[R], float cp,
+                                       float (&y)[R]) {
+  float xo[R], xv[R];
+  if (R == 1) {
+    xo[0] = *xc;
+  } else if (R == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(xc);
+    xo[0] = t.x; xo[R - 1] = t.y;
+  } else {
+    const float4 t = *reinterpret_cast<const float4*>(xc);
+    xo[0] = t.x; xo[1 % R] = t.y; xo[2 % R] = t.z; xo[3 % R] = t.w;
+  }
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const float x = xc[r];
+    const float x = xo[r];
     const float gx = g_val(x, G_QUAD);
     const float d = acc[r] + cp + y[r] * g_der(x, G_QUAD);
     // pdbo_update (common.cuh) with the projection as a saturation: the same value
     const bool stagnating = fabsf(x - 0.5f) <= a.delta && fabsf(d) <= a.grad_tol && y[r] <= 0.0f;
-    float xv = __saturatef(x - a.alpha * d);
-    if (stagnating) xv = x <= 0.5f ? 0.5f - a.delta : 0.5f + a.delta;
+    xv[r] = __saturatef(x - a.alpha * d);
+    if (stagnating) xv[r] = x <= 0.5f ? 0.5f - a.delta : 0.5f + a.delta;
     y[r] = y[r] + a.beta * gx;
-    xn[r] = xv;
-    m |= (xv > 0.5f ? 1u : 0u) << r;
   }
-  return m;
+  if (R == 1) *xn = xv[0];
+  else if (R == 2) *reinterpret_cast<float2*>(xn) = make_float2(xv[0], xv[R - 1]);
+  else *reinterpret_cast<float4*>(xn) = make_float4(xv[0], xv[1 % R], xv[2 % R], xv[3 % R]);
 }
 
 // Q: slices per warp at most (y and c' of a thread's vertices live in registers: Q R + Q, or Q R + Q / 2
@@ -177,6 +210,8 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
     }
   }
   __syncthreads();
+  constexpr int BASE = Q > 10 ? 1 : 2;            // restarts per position the entries are scaled for
+  const int shift = BASE == 1 ? 2 : 3;            // entry offset -> position
 
   const uint4* stream0 = (P.ent_in_smem ? ent_s : P.ent) + (size_t)P.wstart[warp] * 32 + lane;
   int64_t e_idx = P.e0;
@@ -193,7 +228,8 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
     for (int d = 0; d < RST_SPARE; ++d, st += 32) nx[d] = *st;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-      if (warp + q * RST_WARPS < P.slices) {
+      if (warp + q * RST_WARPS >= P.slices) break;   // no later slice either
+      {
         const int p = p0 + q * RST_THREADS;
         float acc[R];
 #pragma unroll
@@ -205,15 +241,11 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
           for (int d = 0; d + 1 < RST_SPARE; ++d) nx[d] = nx[d + 1];
           nx[RST_SPARE - 1] = *st;
           st += 32;
-          gather<R, BF16>(xc, c.x, acc);
-          gather<R, BF16>(xc, c.y, acc);
-          gather<R, BF16>(xc, c.z, acc);
-          gather<R, BF16>(xc, c.w, acc);
+          gather4<R, BF16, BASE>(xc, c, acc);
         }
         const float cp = !PACK ? cps[PACK ? 0 : q]
                                : __uint_as_float((q & 1) ? cpk[PACK ? q / 2 : 0] & 0xffff0000u : cpk[PACK ? q / 2 : 0] << 16);
-        const uint32_t m = update<R>(a, xc + (size_t)p * R, xn + (size_t)p * R, acc, cp, y[q]);
-        if (is_eval) bb[p] = (uint8_t)m;
+        update<R>(a, xc + p * R, xn + p * R, acc, cp, y[q]);
       }
     }
     {
@@ -224,6 +256,14 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
     __syncthreads();
     if (!is_eval) continue;
 
+    // candidates b = [x > 1/2]
+    for (int p = p0; p < npos; p += RST_THREADS) {
+      uint32_t m = 0u;
+#pragma unroll
+      for (int r = 0; r < R; ++r) m |= (xc[p * R + r] > 0.5f ? 1u : 0u) << r;
+      bb[p] = (uint8_t)m;
+    }
+    __syncthreads();
     // exact objective of the candidates: 2F = sum_i b_i ((A b)_i + 2 c'_i); (A b)_i is an exact
     // integer in FP32 because every row sum of |A| is below 2^24
     long long f2[R];
@@ -238,10 +278,10 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
       for (int r = 0; r < R; ++r) acc[r] = 0.0f;
       for (int g = 0; g < ng; ++g, st += 32) {
         const uint4 c = *st;   // entries beyond a row's length are padding (weight 0)
-        add_bits<R>(bb, c.x, acc);
-        add_bits<R>(bb, c.y, acc);
-        add_bits<R>(bb, c.z, acc);
-        add_bits<R>(bb, c.w, acc);
+        add_bits<R>(bb, c.x, shift, acc);
+        add_bits<R>(bb, c.y, shift, acc);
+        add_bits<R>(bb, c.z, shift, acc);
+        add_bits<R>(bb, c.w, shift, acc);
       }
       if (p < n) {
         const uint32_t m = bb[p];
@@ -411,10 +451,15 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
   int maxd = 0;
   for (int64_t i = 0; i < n; ++i) maxd = std::max(maxd, rp[i + 1] - rp[i]);
   if (maxd > CSR_RESTART_MAX_DEG) return false;
-  for (int64_t e = 0; e < rp[n]; ++e)
-    if (val[e] > 256 || val[e] < -256) return false;   // not exact in BF16
+  for (int64_t e = 0; e < rp[n]; ++e) {   // the weight must fit an entry's top 15 bits exactly
+    const float w = (float)val[e];
+    uint32_t bits;
+    std::memcpy(&bits, &w, 4);
+    if ((int64_t)w != val[e] || (bits & ~ENT_W)) return false;
+  }
   // positions by descending degree, equal degrees in vertex order
   const int slices = (int)((n + 31) / 32);
+  const int shift = n > 10 * RST_THREADS ? 2 : 3;   // see k_csr_restart: BASE
   std::vector<int32_t> first((size_t)maxd + 2, 0), perm((size_t)n), pos((size_t)n);
   for (int64_t i = 0; i < n; ++i) ++first[(size_t)(maxd - (rp[i + 1] - rp[i])) + 1];
   for (int d = 0; d <= maxd; ++d) first[(size_t)d + 1] += first[(size_t)d];
@@ -449,12 +494,12 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
         const int64_t i = p < n ? perm[(size_t)p] : -1;
         const int deg = i >= 0 ? rp[i + 1] - rp[i] : 0;
         for (int k = 0; k < 4 * gr; ++k) {
-          uint32_t e = (uint32_t)p;   // padding gathers its own position with weight 0
+          uint32_t e = (uint32_t)p << shift;   // padding gathers its own position with weight 0
           if (k < deg) {
             const float w32 = (float)val[rp[i] + k];
             uint32_t bits;
             std::memcpy(&bits, &w32, 4);
-            e = bits | (uint32_t)pos[(size_t)col[rp[i] + k]];   // |w| <= 256: the low 16 bits are zero
+            e = bits | (uint32_t)pos[(size_t)col[rp[i] + k]] << shift;
           }
           out->ent[(g + (size_t)(k / 4)) * 128 + (size_t)l * 4 + (k & 3)] = e;
         }

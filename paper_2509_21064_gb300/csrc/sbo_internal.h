@@ -118,7 +118,8 @@ cudaError_t launch_csr_res(const int32_t* rowptr, const int32_t* col, const void
 int csr_partial_rows(int64_t n, int B);
 // k_csr_restart.cu: whole runs with R restarts of the graph per CTA (state on chip between launches).
 // csr_restart_build lays the structure out (false: the graph does not fit the form: more than 20,480
-// vertices, a row longer than CSR_RESTART_MAX_DEG or a weight not exact in BF16); csr_restart_pick
+// vertices, a row longer than CSR_RESTART_MAX_DEG or a weight of more than 7
+// significant bits); csr_restart_pick
 // gives the restarts per CTA for a run of B restarts.
 constexpr int CSR_RESTART_MAX_DEG = 256;
 struct CsrRestartShape {

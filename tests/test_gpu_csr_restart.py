@@ -78,7 +78,9 @@ def test_degree_and_range_limits_fall_back():
     star = (np.concatenate([[0], np.full(n, 300)]), np.arange(1, 301), np.ones(300, int), np.zeros(n, int))
     _same(n, star, S.SBO_FP32, 5, 10, 30, [30], resident=False)             # a row of 300
     heavy = _graph(n, 4, 2)
-    _same(n, (heavy[0], heavy[1], heavy[2] * 300, heavy[3]), S.SBO_FP32, 5, 10, 30, [30], resident=False)   # |A| > 256
+    _same(n, (heavy[0], heavy[1], heavy[2] * 129, heavy[3]), S.SBO_FP32, 5, 10, 30, [30], resident=False)   # 8 bits
+    _same(n, (heavy[0], heavy[1], heavy[2] * 4064, heavy[3]), S.SBO_FP32, 5, 10, 30, [30])   # 127 * 32: 7 bits
+    _same(700, _graph(700, 6, 2, wmax=127), S.SBO_BF16, 5, 10, 30, [30])
     _same(n, (*heavy[:3], heavy[3] * 1001), S.SBO_FP32, 5, 10, 30, [30], resident=False)   # c' not exact in BF16
     _same(700, (*_graph(700, 4, 3)[:3], np.full(700, 1001)), S.SBO_FP32, 5, 10, 30, [30])  # small n keeps FP32 c'
     _same(20481, _graph(20481, 3, 4), S.SBO_FP32, 2, 10, 30, [30], resident=False)
