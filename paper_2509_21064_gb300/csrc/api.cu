@@ -120,6 +120,12 @@ struct sbo_problem {
   int kernel = KER_AUTO, layout = LAYOUT_RN, op_type = OP_F32, tile_n = 0;
   int csr_form = CSR_FORM_RULE;   // form of the sparse update in this run
   int rst_R = 0;                  // restarts per CTA of the restart-resident runs (0: not used in this run)
+  // State of the restart-resident runs.  rst_home: it is current and the row-wise arrays (Xm, Y, Xop, bits,
+  // bestBits) are stale or not allocated; to_rows / to_units convert.
+  bool rst_home = false;
+  float *rX = nullptr, *rY = nullptr;
+  uint8_t* rBest = nullptr;
+  unsigned int* rst_sched = nullptr;
   int B = 0;
   int64_t ld = 0;
   int64_t t = 0;          // iterations completed
@@ -196,6 +202,11 @@ void free_run(sbo_problem* p) {
   dfree(p->tc_ctr, p->stream);
   dfree(p->tc_gbar, p->stream);
   dfree(p->csk_ws, p->stream);
+  dfree(p->rX, p->stream);
+  dfree(p->rY, p->stream);
+  dfree(p->rBest, p->stream);
+  dfree(p->rst_sched, p->stream);
+  p->rst_home = false;
   p->started = false;
 }
 
@@ -477,48 +488,131 @@ sbo_status capture_block(sbo_problem* p, int parity, int kind) {
   return SBO_OK;
 }
 
-// Whether the next `iters` iterations run restart by restart (k_csr_restart.cu): the sparse form
-// was left to the library, and the launch's load and write-back of the state are spread over enough
-// iterations.  A request for single launches (graphs off, one iteration per launch) or for a
-// particular evaluation schedule keeps the row-wise kernels.
+// Whether a run may go restart by restart (k_csr_restart.cu): the sparse form was left to the library.  A
+// request for single launches (graphs off, one iteration per launch) or for a particular evaluation
+// schedule keeps the row-wise kernels, and so do calls of fewer than RESTART_MIN_ITERS iterations,
+// over which the launch's load and write-back of the state would not be spread.
 constexpr int64_t RESTART_MIN_ITERS = 8;
-bool restart_runs(const sbo_problem* p, int64_t iters) {
-  return p->kernel == KER_CSR && p->rst_R > 0 && !p->single && p->opt_g == G_QUAD && p->opt_graph &&
-         p->opt_eval_mode == 0 && iters >= RESTART_MIN_ITERS &&
+bool restart_wanted(const sbo_problem* p) {
+  return p->rst_buf && p->opt_g == G_QUAD && p->opt_graph && p->opt_eval_mode == 0 &&
          (p->opt_steps_per_launch == 0 || p->opt_steps_per_launch >= RESTART_MIN_ITERS);
+}
+bool restart_runs(const sbo_problem* p, int64_t iters) {
+  return p->kernel == KER_CSR && p->rst_R > 0 && iters >= RESTART_MIN_ITERS && restart_wanted(p);
+}
+
+// Buffers of the restart-resident runs, for any number of restarts per CTA.
+cudaError_t alloc_units(sbo_problem* p) {
+  if (p->rst_sched) return cudaSuccess;   // the last one allocated
+  const size_t npos = csr_restart_positions(p->rst.shape), rows = (size_t)p->B + CSR_RESTART_MAX_R - 1;
+  cudaError_t e = cudaSuccess;
+  if (!p->rX) e = dalloc(&p->rX, rows * npos, p->stream);
+  if (e == cudaSuccess && !p->rY) e = dalloc(&p->rY, rows * npos, p->stream);
+  if (e == cudaSuccess && !p->rBest) e = dalloc(&p->rBest, (size_t)p->B * npos, p->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(p->rBest, 0, (size_t)p->B * npos, p->stream);
+  if (e == cudaSuccess) e = dalloc(&p->rst_sched, (size_t)p->B + 2, p->stream);
+  return e;
+}
+
+// The row-wise kernels' state arrays of a sparse run, zeroed (padding never holds stale values).
+cudaError_t alloc_rows(sbo_problem* p) {
+  if (p->bestBits) return cudaSuccess;   // the last one allocated
+  cudaStream_t s = p->stream;
+  const size_t elems = (size_t)p->n * p->ld, op = elems * (p->op_type == OP_F32 ? 4 : 2);
+  cudaError_t e = cudaSuccess;
+  auto al = [&](void** q, size_t bytes) {
+    if (e == cudaSuccess && !*q) e = cudaMallocAsync(q, bytes, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(*q, 0, bytes, s);
+  };
+  if (p->op_type != OP_F32) al((void**)&p->Xm, elems * 4);
+  al((void**)&p->Y, elems * 4);
+  al(&p->Xop[0], op);
+  al(&p->Xop[1], op);
+  al(&p->bits, elems);
+  al((void**)&p->bestBits, elems);
+  return e;
+}
+
+cudaError_t convert_units(sbo_problem* p, bool to_rows) {
+  RestartLayout L;
+  std::memset(&L, 0, sizeof(L));
+  L.n = (int)p->n;
+  L.B = p->B;
+  L.R = p->rst_R;
+  L.op_type = p->op_type;
+  L.ld = p->ld;
+  L.X = p->rX;
+  L.Y = p->rY;
+  L.best = p->rBest;
+  L.Xm = p->Xm;
+  L.Yrows = p->Y;
+  L.Xop = p->Xop[p->cur];
+  L.bestBits = p->bestBits;
+  ++p->launches;
+  return launch_restart_convert(p->rst, L, to_rows, p->stream);
+}
+sbo_status to_rows(sbo_problem* p) {
+  if (!p->rst_home) return SBO_OK;
+  cudaError_t e = alloc_rows(p);
+  if (e == cudaSuccess) e = convert_units(p, true);
+  if (e != cudaSuccess)
+    return e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation of the run state failed")
+                                          : cuda_fail(e, "state layout");
+  p->rst_home = false;
+  return SBO_OK;
+}
+sbo_status to_units(sbo_problem* p) {
+  if (p->rst_home) return SBO_OK;
+  sbo_status st = flush_pending(p);
+  if (st != SBO_OK) return st;
+  cudaError_t e = alloc_units(p);
+  if (e == cudaSuccess) e = convert_units(p, false);
+  if (e != cudaSuccess)
+    return e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation of the run state failed")
+                                          : cuda_fail(e, "state layout");
+  p->rst_home = true;
+  return SBO_OK;
+}
+
+CsrRestartRun restart_run_args(const sbo_problem* p) {
+  CsrRestartRun r;
+  std::memset(&r, 0, sizeof(r));
+  r.bestF = p->bestF;
+  r.bestT = p->bestT;
+  r.evalF = p->evalF;
+  r.trace = p->trace;
+  r.n_evals = p->n_evals;
+  r.t_last = p->t_last;
+  r.trace_cap = p->trace_cap;
+  r.X = p->rX;
+  r.Y = p->rY;
+  r.best = p->rBest;
+  r.sched = p->rst_sched;
+  r.timeout_ns = timeout_ns(p);
+  return r;
 }
 
 sbo_status run_restart(sbo_problem* p, int64_t iters) {
-  sbo_status st = flush_pending(p);
+  sbo_status st = to_units(p);
   if (st != SBO_OK) return st;
   const int64_t per = p->opt_steps_per_launch == 0 ? 4096 : p->opt_steps_per_launch;
   const int64_t K = p->prm.eval_every, T = p->prm.iters;
   for (int64_t done = 0; done < iters;) {
     const int64_t chunk = std::min(per, iters - done);
     const int64_t t0 = p->t, t1 = p->t + chunk;
-    CsrRestartRun r;
+    CsrRestartRun r = restart_run_args(p);
     r.t0 = t0;
     r.K = K;
     r.T = T;
     r.e0 = p->n_evals_host;
     r.iters = (int)chunk;
-    r.bestF = p->bestF;
-    r.bestT = p->bestT;
-    r.evalF = p->evalF;
-    r.trace = p->trace;
-    r.n_evals = p->n_evals;
-    r.t_last = p->t_last;
-    r.trace_cap = p->trace_cap;
-    r.bestBits = p->bestBits;
     // evaluation points in (t0, t1]: the multiples of K, and T
     const bool at_T = T > t0 && T <= t1;
     r.n_evals_new = p->n_evals_host + t1 / K - t0 / K + (at_T && T % K != 0 ? 1 : 0);
     r.t_last_new = p->t_last_eval;
     if (t1 / K > t0 / K) r.t_last_new = t1 / K * K;
     if (at_T) r.t_last_new = std::max<int64_t>(r.t_last_new, T);
-    void* x = p->Xop[p->cur];
-    cudaError_t e = launch_csr_restart(p->rst, base_args(p), p->op_type,
-                                       p->Xm ? p->Xm : static_cast<const float*>(x), x, r, p->rst_R, p->stream);
+    cudaError_t e = launch_csr_restart(p->rst, base_args(p), p->op_type, r, p->rst_R, p->sms, p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "restart-resident launch");
     ++p->launches;
     p->t = t1;
@@ -527,6 +621,13 @@ sbo_status run_restart(sbo_problem* p, int64_t iters) {
     done += chunk;
   }
   return SBO_OK;
+}
+
+// FP32 copy of the current x as [B][n] on the device.
+cudaError_t gather_x(sbo_problem* p, float* dst, cudaStream_t s) {
+  if (p->rst_home) return launch_restart_gather(p->rst, p->rX, (int)p->n, p->B, p->rst_R, dst, s);
+  const float* xsrc = p->Xm ? p->Xm : static_cast<const float*>(p->Xop[p->cur]);
+  return launch_gather_state(xsrc, (int)p->n, p->B, p->ld, p->layout, dst, s);
 }
 
 sbo_status run_tiny(sbo_problem* p, int64_t steps) {
@@ -765,7 +866,7 @@ sbo_status tune_tile(sbo_problem* p, int* out) {
 // with 128 or 256 restarts, pipelined rows of 256, each with and without the L2 eviction
 // priorities) on this run's own buffers, before x^0 is written, and keeps the fastest.  Kept per (device, graph
 // size, restarts, precision, g) for the process and in the persistent record of tune_tile.
-sbo_status tune_csr_form(sbo_problem* p, int* out) {
+sbo_status tune_csr_form(sbo_problem* p, int* out, bool lookup_only) {
   static std::mutex mu;
   static std::map<std::string, int> cache;
   std::string key;
@@ -786,6 +887,7 @@ sbo_status tune_csr_form(sbo_problem* p, int* out) {
       return SBO_OK;
     }
   }
+  if (lookup_only) return SBO_OK;   // *out keeps the rule
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   SBO_CUDA(cudaEventCreate(&e0));
   SBO_CUDA(cudaEventCreate(&e1));
@@ -861,46 +963,42 @@ sbo_status tune_csr_form(sbo_problem* p, int* out) {
   return SBO_OK;
 }
 
-// Autotuner of the restart-resident runs: times `update` iterations of the row-wise form in use and of
-// the resident kernel with 1, 2 and 4 restarts per CTA (the difference of a long and a short launch,
-// which leaves out the load and write-back of the state), on this run's buffers before x^0 is
-// written.  *R gets the fastest's restarts per CTA, or 0 for the row-wise kernels.  Kept like the
-// other decisions.
-sbo_status tune_restart(sbo_problem* p, int* R) {
+// Autotuner of the restart-resident runs: times iterations of the row-wise form in use and of the
+// resident kernel with 1, 2 and 4 restarts per CTA (the difference of a long and a short launch, which
+// leaves out the load and write-back of the state), on this run's buffers before x^0 is written.  *R
+// gets the fastest's restarts per CTA, or 0 for the row-wise kernels.  Kept like the other decisions;
+// lookup_only: true only when a decision is on record.
+bool tune_restart_known(sbo_problem* p, const std::string& key, std::mutex& mu, std::map<std::string, int>& cache, int* R) {
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = cache.find(key);
+  if (it != cache.end()) { *R = it->second; return true; }
+  int t = 0;
+  if (tune_cache_lookup(key, &t, [](int v) { return v == 0 || v == 1 || v == 2 || v == 4; }) &&
+      (t == 0 || csr_restart_fits(p->rst.shape, t))) {
+    cache[key] = t;
+    *R = t;
+    return true;
+  }
+  return false;
+}
+sbo_status tune_restart(sbo_problem* p, int* R, bool lookup_only, bool* known) {
   static std::mutex mu;
   static std::map<std::string, int> cache;
   std::ostringstream k;
-  k << "rst1:" << tune_device(p) << ":n" << p->n << ":nnz" << p->nnz << ":deg" << p->max_deg << ":grp"
+  k << "rst2:" << tune_device(p) << ":n" << p->n << ":nnz" << p->nnz << ":deg" << p->max_deg << ":grp"
     << p->rst.shape.groups << ":B" << p->B << ":op" << p->op_type;
   const std::string key = k.str();
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = cache.find(key);
-    if (it != cache.end()) { *R = it->second; return SBO_OK; }
-    int t = 0;
-    if (tune_cache_lookup(key, &t, [](int v) { return v == 0 || v == 1 || v == 2 || v == 4; }) &&
-        (t == 0 || csr_restart_fits(p->rst.shape, t))) {
-      cache[key] = t;
-      *R = t;
-      return SBO_OK;
-    }
-  }
+  *known = tune_restart_known(p, key, mu, cache, R);
+  if (*known || lookup_only) return SBO_OK;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   SBO_CUDA(cudaEventCreate(&e0));
   SBO_CUDA(cudaEventCreate(&e1));
-  CsrRestartRun r;
-  std::memset(&r, 0, sizeof(r));
+  CsrRestartRun r = restart_run_args(p);
   r.K = r.T = INT64_MAX / 2;   // no evaluation
-  r.bestF = p->bestF;
-  r.bestT = p->bestT;
-  r.evalF = p->evalF;
-  r.trace = p->trace;
-  r.n_evals = p->n_evals;
-  r.t_last = p->t_last;
-  r.trace_cap = p->trace_cap;
-  r.bestBits = p->bestBits;
   const EpiArgs a = base_args(p);
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(p->rX, 0, ((size_t)p->B + CSR_RESTART_MAX_R - 1) * csr_restart_positions(p->rst.shape) * 4, p->stream);
+  if (e == cudaSuccess)
+    e = cudaMemsetAsync(p->rY, 0, ((size_t)p->B + CSR_RESTART_MAX_R - 1) * csr_restart_positions(p->rst.shape) * 4, p->stream);
   // device time of launch() in ms, the better of two
   auto timed = [&](auto&& launch) {
     float best = 1e30f;
@@ -934,12 +1032,11 @@ sbo_status tune_restart(sbo_problem* p, int* R) {
       return timed([&] {
         r.iters = iters;
         ++p->launches;
-        return launch_csr_restart(p->rst, a, p->op_type, p->Xm ? p->Xm : static_cast<float*>(p->Xop[0]), p->Xop[0], r,
-                                  cand, p->stream);
+        return launch_csr_restart(p->rst, a, p->op_type, r, cand, p->sms, p->stream);
       });
     };
-    const float lo = run(reps), hi = run(3 * reps);
-    const float ms = (hi - lo) / (2 * reps);
+    const float lo = run(4 * reps), hi = run(12 * reps);   // long enough to be cut into chunks like a run
+    const float ms = (hi - lo) / (8 * reps);
     if (e == cudaSuccess && ms < best_ms) { best_ms = ms; best = cand; }
   }
   cudaEventDestroy(e0);
@@ -953,6 +1050,7 @@ sbo_status tune_restart(sbo_problem* p, int* R) {
     tune_cache_store(key, best);
   }
   *R = best;
+  *known = true;
   return SBO_OK;
 }
 
@@ -1236,8 +1334,8 @@ sbo_status sbo_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const i
   if (csr_restart_build(n, rp.data(), cc.data(), vv.data(), cp.data(), &rh)) {
     // one buffer: group streams (16-byte groups), c' exact, then the 4-byte tables and the group counts
     const size_t b_ent = rh.ent.size() * 4, b_c64 = rh.cpp64.size() * 8, b_ws = rh.wstart.size() * 4,
-                 b_perm = rh.perm.size() * 4, b_cp = rh.cpp.size() * 4, b_w = rh.ngroups.size();
-    std::vector<uint8_t> img(b_ent + b_c64 + b_ws + b_perm + b_cp + b_w);
+                 b_perm = rh.perm.size() * 4, b_pos = rh.pos.size() * 4, b_cp = rh.cpp.size() * 4, b_w = rh.ngroups.size();
+    std::vector<uint8_t> img(b_ent + b_c64 + b_ws + b_perm + b_pos + b_cp + b_w);
     size_t off = 0;
     auto put = [&](const void* src, size_t bytes) {
       std::memcpy(img.data() + off, src, bytes);
@@ -1245,7 +1343,7 @@ sbo_status sbo_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const i
       return off - bytes;
     };
     const size_t o_ent = put(rh.ent.data(), b_ent), o_c64 = put(rh.cpp64.data(), b_c64),
-                 o_ws = put(rh.wstart.data(), b_ws), o_perm = put(rh.perm.data(), b_perm),
+                 o_ws = put(rh.wstart.data(), b_ws), o_perm = put(rh.perm.data(), b_perm), o_pos = put(rh.pos.data(), b_pos),
                  o_cp = put(rh.cpp.data(), b_cp), o_w = put(rh.ngroups.data(), b_w);
     uint8_t* dev = nullptr;
     if ((e = dalloc(&dev, img.size(), cs)) != cudaSuccess)
@@ -1259,6 +1357,7 @@ sbo_status sbo_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const i
     p->rst.cpp64 = reinterpret_cast<int64_t*>(dev + o_c64);
     p->rst.wstart = reinterpret_cast<uint32_t*>(dev + o_ws);
     p->rst.perm = reinterpret_cast<int32_t*>(dev + o_perm);
+    p->rst.pos = reinterpret_cast<int32_t*>(dev + o_pos);
     p->rst.cpp = reinterpret_cast<float*>(dev + o_cp);
     p->rst.ngroups = dev + o_w;
   }
@@ -1446,20 +1545,39 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   auto al = [&](void** q, size_t bytes) {
     if (e == cudaSuccess) e = cudaMallocAsync(q, bytes ? bytes : 1, p->stream);
   };
-  if (need_master) al((void**)&p->Xm, xelems * 4);
-  al((void**)&p->Y, elems * 4);
-  if (p->opt_keep_grad) al((void**)&p->Gd, elems * 4);
-  if (ker != KER_TINY) {
-    al(&p->Xop[0], xelems * op_elt);
-    al(&p->Xop[1], xelems * op_elt);
-    al(&p->bits, elems * (ker == KER_CSR ? 1 : op_elt));   // the sparse path keeps candidates as bytes
+  // A sparse run that is known to go restart by restart starts in that layout: the row-wise arrays
+  // are allocated only if a later call needs them.
+  p->rst_R = 0;
+  p->single = p->opt_dual == 1;
+  const bool try_restart =
+      ker == KER_CSR && !p->single && p->opt_csr_form == 0 && !p->opt_keep_grad && restart_wanted(p);
+  bool restart_known = true;   // (without the autotuner: the fixed rule)
+  if (try_restart) {
+    if (!p->opt_autotune) {
+      p->rst_R = csr_restart_pick(p->rst.shape, p->B, p->sms);
+    } else {
+      sbo_status st2 = tune_restart(p, &p->rst_R, true, &restart_known);
+      if (st2 != SBO_OK) return st2;
+    }
   }
+  bool home = p->rst_R > 0;
+  if (!home) {
+    if (need_master) al((void**)&p->Xm, xelems * 4);
+    al((void**)&p->Y, elems * 4);
+    if (p->opt_keep_grad) al((void**)&p->Gd, elems * 4);
+    if (ker != KER_TINY) {
+      al(&p->Xop[0], xelems * op_elt);
+      al(&p->Xop[1], xelems * op_elt);
+      al(&p->bits, elems * (ker == KER_CSR ? 1 : op_elt));   // the sparse path keeps candidates as bytes
+    }
+    al((void**)&p->bestBits, elems);
+  }
+  if (e == cudaSuccess && (home || !restart_known)) e = alloc_units(p);
   al((void**)&p->bestF, sizeof(long long) * p->B);
   al((void**)&p->bestT, sizeof(long long) * p->B);
   al((void**)&p->evalF, sizeof(long long) * p->B);
   al((void**)&p->F2, sizeof(unsigned long long) * p->B);
   al((void**)&p->commit_ctr, sizeof(unsigned int));
-  p->single = p->opt_dual == 1;
   if (p->single) {
     // rows of partial sums the update kernel writes: 4 per 128 variables (tcgen05 kernels; CTA
     // pairs round up to 256), 1 per 64 variables (SIMT), 1 per block along the rows (CSR)
@@ -1469,7 +1587,6 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
     al((void**)&p->mu, sizeof(float) * p->gpart_ld);
     al((void**)&p->gpart, sizeof(float) * p->gpart_rows * p->gpart_ld);
   }
-  al((void**)&p->bestBits, elems);
   al((void**)&p->trace, sizeof(long long) * p->trace_cap);
   al((void**)&p->n_evals, sizeof(long long));
   al((void**)&p->t_last, sizeof(long long));
@@ -1482,7 +1599,7 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   cudaStream_t s = p->stream;
   // zero every buffer so padding never holds stale values; sentinels for bests and trace
   if (p->Xm) cudaMemsetAsync(p->Xm, 0, xelems * 4, s);
-  cudaMemsetAsync(p->Y, 0, elems * 4, s);
+  if (p->Y) cudaMemsetAsync(p->Y, 0, elems * 4, s);
   if (p->Gd) cudaMemsetAsync(p->Gd, 0, elems * 4, s);
   for (void* b : {p->Xop[0], p->Xop[1]})
     if (b) cudaMemsetAsync(b, 0, xelems * op_elt, s);
@@ -1493,7 +1610,7 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   p->launches += 3;
   cudaMemsetAsync(p->F2, 0, sizeof(unsigned long long) * p->B, s);
   cudaMemsetAsync(p->commit_ctr, 0, sizeof(unsigned int), s);
-  cudaMemsetAsync(p->bestBits, 0, elems, s);
+  if (p->bestBits) cudaMemsetAsync(p->bestBits, 0, elems, s);
   cudaMemsetAsync(p->n_evals, 0, sizeof(long long), s);
   cudaMemsetAsync(p->t_last, 0, sizeof(long long), s);
   if (ker == KER_TC) {
@@ -1555,7 +1672,6 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
     p->tile_n = 0;
   }
   p->csr_form = CSR_FORM_RULE;
-  p->rst_R = 0;
   if (ker == KER_CSR && !p->single) {
 
     // grid barrier words of the resident form (allocated before the autotuner, which times it)
@@ -1568,17 +1684,14 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
       p->csr_form = p->opt_csr_form;
     } else if (p->opt_autotune) {
       int f = CSR_FORM_RULE;
-      sbo_status st2 = tune_csr_form(p, &f);   // on the zeroed state, before x^0 is written
+      sbo_status st2 = tune_csr_form(p, &f, home);   // on the zeroed state, before x^0 is written
       if (st2 != SBO_OK) { free_run(p); return st2; }
       p->csr_form = f;
     }
-    if (p->rst_buf && p->opt_csr_form == 0 && p->opt_g == G_QUAD && !p->opt_keep_grad) {
-      if (p->opt_autotune) {
-        sbo_status st2 = tune_restart(p, &p->rst_R);   // on the zeroed state, before x^0 is written
-        if (st2 != SBO_OK) { free_run(p); return st2; }
-      } else {
-        p->rst_R = csr_restart_pick(p->rst.shape, p->B, p->sms);
-      }
+    if (!restart_known) {
+      sbo_status st2 = tune_restart(p, &p->rst_R, false, &restart_known);   // on the zeroed state too
+      if (st2 != SBO_OK) { free_run(p); return st2; }
+      home = p->rst_R > 0;   // the row-wise arrays stay allocated for calls that need them
     }
     int D, S, rc;
     size_t sm;
@@ -1615,7 +1728,10 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
       dfree(x0d, s); dfree(y0d, s); free_run(p); return cuda_fail(e, "single-constraint dual set-up");
     }
   }
-  if (ker == KER_MAXK)
+  if (home)
+    e = launch_restart_init(p->rst, (int)p->n, p->B, p->rst_R, prm->seed, (float)prm->ybar, x0d, y0d, p->rX, p->rY,
+                            p->err, s);
+  else if (ker == KER_MAXK)
     e = launch_maxk_init((int)p->n, p->B, p->ld, p->kparts, prm->seed, (float)prm->ybar, p->Xm, p->Y,
                          static_cast<float*>(p->Xop[0]), s);
   else
@@ -1625,6 +1741,7 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   ++p->launches;
   if (x0d || y0d) { cudaStreamSynchronize(s); dfree(x0d, s); dfree(y0d, s); }
   if (e != cudaSuccess) { free_run(p); return cuda_fail(e, "init launch"); }
+  p->rst_home = home;
   p->started = true;
   return SBO_OK;
 }
@@ -1637,6 +1754,10 @@ sbo_status sbo_gda_run(sbo_problem* p, int64_t iters) {
   if (iters == 0) return SBO_OK;
   if (p->kernel == KER_TINY) return run_tiny(p, iters);
   if (restart_runs(p, iters)) return run_restart(p, iters);
+  {
+    sbo_status st = to_rows(p);
+    if (st != SBO_OK) return st;
+  }
   const int64_t K = p->prm.eval_every;
   const int64_t t_end = p->t + iters;
   while (p->t < t_end) {
@@ -1796,7 +1917,16 @@ sbo_status sbo_best(sbo_problem* p, uint8_t* x_out, int64_t* F_out, int64_t* ite
   if (restart_out) *restart_out = (int32_t)h[2];
   if (x_out) {
     const int64_t r = h[2];
-    if (p->layout == LAYOUT_RN) {
+    if (p->rst_home) {
+      uint8_t* row = nullptr;
+      SBO_CUDA(dalloc(&row, (size_t)p->n, s));
+      e = launch_restart_best_row(p->rst, p->rBest, (int)p->n, p->rst_R, r, row, s);
+      ++p->launches;
+      if (e == cudaSuccess) e = cudaMemcpyAsync(x_out, row, (size_t)p->n, cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      dfree(row, s);
+      if (e != cudaSuccess) return cuda_fail(e, "best candidate read-back");
+    } else if (p->layout == LAYOUT_RN) {
       SBO_CUDA(cudaMemcpy(x_out, p->bestBits + r * p->ld, (size_t)p->n, cudaMemcpyDeviceToHost));
     } else {
       SBO_CUDA(cudaMemcpy2D(x_out, 1, p->bestBits + r, (size_t)p->ld, 1, (size_t)p->n, cudaMemcpyDeviceToHost));
@@ -1825,13 +1955,12 @@ sbo_status sbo_state(sbo_problem* p, float* X, float* Y) {
   float* tmp = nullptr;
   const int kx = p->kernel == KER_MAXK ? p->kparts : 1;   // Max-k-Cut: X_:,i has k entries
   SBO_CUDA(dalloc(&tmp, (size_t)p->B * p->n * kx, s));
-  const float* xsrc = p->Xm ? p->Xm : static_cast<const float*>(p->Xop[p->cur]);
   cudaError_t e = cudaSuccess;
   if (X) {
     if (p->kernel == KER_MAXK)
       e = launch_maxk_gather(static_cast<const float*>(p->Xop[p->cur]), (int)p->n, kx, p->B, p->ld, tmp, s);
     else
-      e = launch_gather_state(xsrc, (int)p->n, p->B, p->ld, p->layout, tmp, s);
+      e = gather_x(p, tmp, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(X, tmp, sizeof(float) * p->B * p->n * kx, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
@@ -1842,7 +1971,8 @@ sbo_status sbo_state(sbo_problem* p, float* X, float* Y) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     for (int64_t r = 0; r < p->B && e == cudaSuccess; ++r) std::fill(Y + r * p->n, Y + (r + 1) * p->n, mu[r]);
   } else if (Y && e == cudaSuccess) {
-    e = launch_gather_state(p->Y, (int)p->n, p->B, p->ld, p->layout, tmp, s);
+    e = p->rst_home ? launch_restart_gather(p->rst, p->rY, (int)p->n, p->B, p->rst_R, tmp, s)
+                    : launch_gather_state(p->Y, (int)p->n, p->B, p->ld, p->layout, tmp, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(Y, tmp, sizeof(float) * p->B * p->n, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
@@ -1996,8 +2126,7 @@ sbo_status sbo_dual_bound(sbo_problem* p, double ybar, double alpha, int64_t ite
     dfree(tmp, s); dfree(xdev, s); dfree(gdev, s);
     return cuda_fail(e, "cudaMalloc (dual bound)");
   }
-  const float* xsrc = p->Xm ? p->Xm : static_cast<const float*>(p->Xop[p->cur]);
-  e = launch_gather_state(xsrc, (int)n, 1, p->ld, p->layout, tmp, s);
+  e = gather_x(p, tmp, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(xf.data(), tmp, sizeof(float) * n, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(cp.data(), p->cp64, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -44,18 +44,43 @@ struct RestartParams {
   const uint4* ent;              // group streams (global)
   const uint32_t* wstart;        // [33] first group (of 32 uint4) of each warp's stream, and the end
   const uint8_t* ngroups;        // [slices] groups of each slice
-  const int32_t* perm;           // [n] vertex at a position
   const float* cpp;              // [positions] c' by position (0 beyond n)
   const int64_t* cpp64;
-  const float* xsrc;             // FP32 x^{t0} ([i ld + r])
-  void* xop;                     // operand written at the end (FP32 or BF16), and Xm when set
-  int slices, ent_in_smem;
+  float *X, *Y;                  // state [unit][position][R] (unit: R restarts)
+  uint8_t* best;                 // bits of the best candidates [unit][position], bit r of a byte: restart r
+  unsigned int* sched;           // chunks > 1: [ticket, abort, chunks finished per unit]
+  int slices, ent_in_smem, units, chunks, chunk_len;
   int64_t t0, K, T, e0;          // iterations t0 + 1 .. t0 + iters; evaluate at multiples of K and at T
   int iters;
   long long *bestF, *bestT, *evalF, *trace, *n_evals, *t_last;
   long long trace_cap, t_last_new, n_evals_new;
-  uint8_t* bestBits;
+  uint64_t timeout_ns;
 };
+
+// Evaluation points among iterations 1 .. t (multiples of K, and T).
+__device__ __forceinline__ int64_t evals_upto(int64_t t, int64_t K, int64_t T) {
+  return t / K + (T > 0 && T <= t && T % K != 0 ? 1 : 0);
+}
+
+// State vectors of one position: R consecutive floats, through L2 (another SM may have written them).
+template <int R>
+__device__ __forceinline__ void ld_state(const float* p, float (&v)[R]) {
+  if (R == 1) {
+    v[0] = __ldcg(p);
+  } else if (R == 2) {
+    const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
+    v[0] = t.x; v[R - 1] = t.y;
+  } else {
+    const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
+    v[0] = t.x; v[1 % R] = t.y; v[2 % R] = t.z; v[3 % R] = t.w;
+  }
+}
+template <int R>
+__device__ __forceinline__ void st_vec(float* p, const float (&v)[R]) {
+  if (R == 1) *p = v[0];
+  else if (R == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[R - 1]);
+  else *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1 % R], v[2 % R], v[3 % R]);
+}
 
 // An entry of the streams: the neighbour's position, shifted so that masking gives the byte offset of
 // its x in a buffer of `base` restarts per position, and the weight's top 15 bits (sign, exponent and 6
@@ -136,9 +161,7 @@ __device__ __forceinline__ void update(const EpiArgs& a, const float* xc, float*
     if (stagnating) xv[r] = x <= 0.5f ? 0.5f - a.delta : 0.5f + a.delta;
     y[r] = y[r] + a.beta * gx;
   }
-  if (R == 1) *xn = xv[0];
-  else if (R == 2) *reinterpret_cast<float2*>(xn) = make_float2(xv[0], xv[R - 1]);
-  else *reinterpret_cast<float4*>(xn) = make_float4(xv[0], xv[1 % R], xv[2 % R], xv[3 % R]);
+  st_vec<R>(xn, xv);
 }
 
 // Q: slices per warp at most (y and c' of a thread's vertices live in registers: Q R + Q, or Q R + Q / 2
@@ -158,206 +181,335 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
   __shared__ long long red[RST_WARPS][R];
   __shared__ long long s_bestF[R], s_bestT[R];
   __shared__ uint32_t s_improved, s_any;
+  __shared__ int s_ticket;
 
   const EpiArgs& a = P.a;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = a.n;
-  const int r0 = (int)blockIdx.x * R;
-  const int nlive = min(R, a.B - r0);
+  const int p0 = warp * 32 + lane;   // this thread's vertices: positions p0, p0 + RST_THREADS, ..
+  constexpr int BASE = Q > 10 ? 1 : 2;            // restarts per position the entries are scaled for
+  const int shift = BASE == 1 ? 2 : 3;            // entry offset -> position
 
   if (P.ent_in_smem)
     for (uint32_t k = threadIdx.x; k < (groups + RST_SPARE) * 32; k += RST_THREADS) ent_s[k] = P.ent[k];
   for (int k = threadIdx.x; k < P.slices; k += RST_THREADS) ngr[k] = P.ngroups[k];
-  if (threadIdx.x < R) {
-    const bool live = (int)threadIdx.x < nlive;
-    s_bestF[threadIdx.x] = live ? P.bestF[r0 + threadIdx.x] : 0;
-    s_bestT[threadIdx.x] = live ? P.bestT[r0 + threadIdx.x] : 0;
-  }
-  if (threadIdx.x == 0) s_any = 0u;
-
+  constexpr int AHEAD = ONE ? RST_SPARE : 1;      // groups in flight per warp
+  const uint32_t stream0 = P.wstart[warp] * 32 + lane;
   constexpr int NC = PACK ? (Q + 1) / 2 : Q;
-  float y[Q][R], cps[PACK ? 1 : NC];
+  float cps[PACK ? 1 : NC];
   uint32_t cpk[PACK ? NC : 1];
 #pragma unroll
-  for (int q = 0; q < NC; ++q) {
-    if (PACK) cpk[PACK ? q : 0] = 0u;
-    else cps[PACK ? 0 : q] = 0.0f;
-  }
-#pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const int s = warp + q * RST_WARPS;
-#pragma unroll
-    for (int r = 0; r < R; ++r) y[q][r] = 0.0f;
-    if (s < P.slices) {
-      const int p = s * 32 + lane;
-      float x[R], c = 0.0f;
-#pragma unroll
-      for (int r = 0; r < R; ++r) x[r] = 0.0f;
-      if (p < n) {
-        const int64_t idx = (int64_t)P.perm[p] * a.ld + r0;
-        c = P.cpp[p];
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-          if (r < nlive) {
-            x[r] = P.xsrc[idx + r];
-            y[q][r] = a.Y[idx + r];
-          }
-      }
-      if (PACK) cpk[PACK ? q / 2 : 0] |= (q & 1) ? (__float_as_uint(c) & 0xffff0000u) : (__float_as_uint(c) >> 16);
-      else cps[PACK ? 0 : q] = c;
-#pragma unroll
-      for (int r = 0; r < R; ++r) xs[(size_t)p * R + r] = x[r];
-    }
+    const float c = warp + q * RST_WARPS < P.slices ? P.cpp[p0 + q * RST_THREADS] : 0.0f;
+    if (!PACK) cps[PACK ? 0 : q] = c;
+    else if (q & 1) cpk[PACK ? q / 2 : 0] |= __float_as_uint(c) & 0xffff0000u;
+    else cpk[PACK ? q / 2 : 0] = __float_as_uint(c) >> 16;
   }
-  __syncthreads();
-  constexpr int BASE = Q > 10 ? 1 : 2;            // restarts per position the entries are scaled for
-  const int shift = BASE == 1 ? 2 : 3;            // entry offset -> position
 
-  const uint4* stream0 = (P.ent_in_smem ? ent_s : P.ent) + (size_t)P.wstart[warp] * 32 + lane;
-  int64_t e_idx = P.e0;
-  int64_t next_eval = (P.t0 / P.K + 1) * P.K;
-  if (P.T > P.t0 && P.T < next_eval) next_eval = P.T;
-  const float* xc = xs;
-  float* xn = xs + (size_t)npos * R;
-  const int p0 = warp * 32 + lane;   // this thread's vertices: positions p0, p0 + RST_THREADS, ..
-  for (int it = 1; it <= P.iters; ++it) {
-    const bool is_eval = P.t0 + it == next_eval;
-    const uint4* st = stream0;
-    uint4 nx[RST_SPARE];   // groups read ahead (the streams end in RST_SPARE spare groups)
-#pragma unroll
-    for (int d = 0; d < RST_SPARE; ++d, st += 32) nx[d] = *st;
+  // Work: (chunk of iterations, unit) pairs.  With one chunk a CTA runs its unit; with more, CTAs
+  // take tickets in order (all units' first chunk, then all second ones, ..) and a chunk starts once
+  // its unit's previous one is finished, which a CTA with an earlier ticket is running or has done.
+  for (;;) {
+    int u = (int)blockIdx.x, c = 0;
+    if (P.chunks > 1) {
+      if (threadIdx.x == 0) {
+        int t = (int)atomicAdd(P.sched, 1u);
+        if (t >= P.units * P.chunks) {
+          t = -1;
+        } else if (t >= P.units) {
+          const uint64_t deadline = globaltimer_ns() + P.timeout_ns;
+          const unsigned int* done = P.sched + 2 + t % P.units;
+          while (ld_acquire_gpu(done) < (unsigned)(t / P.units)) {
+            if (ld_acquire_gpu(P.sched + 1) != 0u || globaltimer_ns() > deadline) {
+              atomicOr(a.err, ERR_TIMEOUT);
+              atomicExch(P.sched + 1, 1u);   // ends every other CTA's waits too
+              t = -1;
+              break;
+            }
+            __nanosleep(200);
+          }
+        }
+        s_ticket = t;
+      }
+      __syncthreads();
+      const int t = s_ticket;
+      if (t < 0) return;
+      u = t % P.units;
+      c = t / P.units;
+    }
+    const int r0 = u * R;
+    const int nlive = min(R, a.B - r0);
+    const int64_t t0 = P.t0 + (int64_t)c * P.chunk_len;
+    const int iters = min(P.chunk_len, P.iters - c * P.chunk_len);
+    float* Xu = P.X + (size_t)u * npos * R;
+    float* Yu = P.Y + (size_t)u * npos * R;
+
+    if (threadIdx.x < R) {
+      const bool live = (int)threadIdx.x < nlive;
+      s_bestF[threadIdx.x] = live ? __ldcg(&P.bestF[r0 + threadIdx.x]) : 0;
+      s_bestT[threadIdx.x] = live ? __ldcg(&P.bestT[r0 + threadIdx.x]) : 0;
+    }
+    if (threadIdx.x == 0) s_any = 0u;
+    float y[Q][R];
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-      if (warp + q * RST_WARPS >= P.slices) break;   // no later slice either
-      {
+#pragma unroll
+      for (int r = 0; r < R; ++r) y[q][r] = 0.0f;
+      if (warp + q * RST_WARPS < P.slices) {
+        const int p = p0 + q * RST_THREADS;
+        float x[R];
+        ld_state<R>(Xu + (size_t)p * R, x);
+        ld_state<R>(Yu + (size_t)p * R, y[q]);
+        st_vec<R>(xs + p * R, x);
+      }
+    }
+    __syncthreads();
+
+    // iterations to the next evaluation point
+    auto until_eval = [&](int64_t t) {
+      int64_t next = (t / P.K + 1) * P.K;
+      if (P.T > t && P.T < next) next = P.T;
+      return (int)min(next - t, (int64_t)1 << 30);
+    };
+    int left = until_eval(t0);
+    const float* xc = xs;
+    float* xn = xs + (size_t)npos * R;
+    for (int it = 1; it <= iters; ++it) {
+      const uint4* st = (P.ent_in_smem ? ent_s : P.ent) + stream0;
+      uint4 nx[AHEAD];   // groups read ahead (the streams end in RST_SPARE spare groups)
+#pragma unroll
+      for (int d = 0; d < AHEAD; ++d, st += 32) nx[d] = *st;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        if (warp + q * RST_WARPS >= P.slices) break;   // no later slice either
         const int p = p0 + q * RST_THREADS;
         float acc[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) acc[r] = 0.0f;
         const int ng = ONE ? 1 : ngr[warp + q * RST_WARPS];
         for (int g = 0; g < ng; ++g) {
-          const uint4 c = nx[0];
+          const uint4 e = nx[0];
 #pragma unroll
-          for (int d = 0; d + 1 < RST_SPARE; ++d) nx[d] = nx[d + 1];
-          nx[RST_SPARE - 1] = *st;
+          for (int d = 0; d + 1 < AHEAD; ++d) nx[d] = nx[d + 1];
+          nx[AHEAD - 1] = *st;
           st += 32;
-          gather4<R, BF16, BASE>(xc, c, acc);
+          gather4<R, BF16, BASE>(xc, e, acc);
         }
         const float cp = !PACK ? cps[PACK ? 0 : q]
                                : __uint_as_float((q & 1) ? cpk[PACK ? q / 2 : 0] & 0xffff0000u : cpk[PACK ? q / 2 : 0] << 16);
         update<R>(a, xc + p * R, xn + p * R, acc, cp, y[q]);
       }
-    }
-    {
-      float* t = const_cast<float*>(xc);
-      xc = xn;
-      xn = t;
-    }
-    __syncthreads();
-    if (!is_eval) continue;
+      {
+        float* t = const_cast<float*>(xc);
+        xc = xn;
+        xn = t;
+      }
+      __syncthreads();
+      if (--left != 0) continue;
 
-    // candidates b = [x > 1/2]
-    for (int p = p0; p < npos; p += RST_THREADS) {
-      uint32_t m = 0u;
+      // candidates b = [x > 1/2]
+      for (int p = p0; p < npos; p += RST_THREADS) {
+        uint32_t m = 0u;
 #pragma unroll
-      for (int r = 0; r < R; ++r) m |= (xc[p * R + r] > 0.5f ? 1u : 0u) << r;
-      bb[p] = (uint8_t)m;
-    }
-    __syncthreads();
-    // exact objective of the candidates: 2F = sum_i b_i ((A b)_i + 2 c'_i); (A b)_i is an exact
-    // integer in FP32 because every row sum of |A| is below 2^24
-    long long f2[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) f2[r] = 0;
-    st = stream0;
-    for (int s = warp; s < P.slices; s += RST_WARPS) {
-      const int ng = ONE ? 1 : ngr[s];
-      const int p = s * 32 + lane;
-      float acc[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) acc[r] = 0.0f;
-      for (int g = 0; g < ng; ++g, st += 32) {
-        const uint4 c = *st;   // entries beyond a row's length are padding (weight 0)
-        add_bits<R>(bb, c.x, shift, acc);
-        add_bits<R>(bb, c.y, shift, acc);
-        add_bits<R>(bb, c.z, shift, acc);
-        add_bits<R>(bb, c.w, shift, acc);
+        for (int r = 0; r < R; ++r) m |= (xc[p * R + r] > 0.5f ? 1u : 0u) << r;
+        bb[p] = (uint8_t)m;
       }
-      if (p < n) {
-        const uint32_t m = bb[p];
-        const long long c2 = 2 * (long long)P.cpp64[p];
+      __syncthreads();
+      // exact objective of the candidates: 2F = sum_i b_i ((A b)_i + 2 c'_i); (A b)_i is an exact
+      // integer in FP32 because every row sum of |A| is below 2^24
+      long long f2[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-          if ((m >> r) & 1u) f2[r] += (long long)acc[r] + c2;
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) f2[r] += __shfl_xor_sync(0xffffffffu, f2[r], o);
-      if (lane == 0) red[warp][r] = f2[r];
-    }
-    if (threadIdx.x == 0) s_improved = 0u;
-    __syncthreads();
-    if (threadIdx.x < R) {
-      const int r = threadIdx.x;
-      long long sum = 0;
-#pragma unroll 4
-      for (int w = 0; w < RST_WARPS; ++w) sum += red[w][r];
-      if (r < nlive) {
-        const long long F = sum / 2;
-        if (F < s_bestF[r]) {   // strict: equal values keep the earliest t
-          s_bestF[r] = F;
-          s_bestT[r] = P.t0 + it;
-          atomicOr(&s_improved, 1u << r);
-        }
-        P.evalF[r0 + r] = F;
-        if (e_idx < P.trace_cap) atomicMin(&P.trace[e_idx], F);
-      }
-    }
-    __syncthreads();
-    const uint32_t imp = s_improved;
-    if (imp) {
+      for (int r = 0; r < R; ++r) f2[r] = 0;
+      const int64_t t = t0 + it;
+      left = until_eval(t);
+      st = (P.ent_in_smem ? ent_s : P.ent) + stream0;
       for (int s = warp; s < P.slices; s += RST_WARPS) {
+        const int ng = ONE ? 1 : ngr[s];
         const int p = s * 32 + lane;
-        best[p] = (uint8_t)((best[p] & ~imp) | (bb[p] & imp));
+        float acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+        for (int g = 0; g < ng; ++g, st += 32) {
+          const uint4 e = *st;   // entries beyond a row's length are padding (weight 0)
+          add_bits<R>(bb, e.x, shift, acc);
+          add_bits<R>(bb, e.y, shift, acc);
+          add_bits<R>(bb, e.z, shift, acc);
+          add_bits<R>(bb, e.w, shift, acc);
+        }
+        if (p < n) {
+          const uint32_t m = bb[p];
+          const long long c2 = 2 * (long long)P.cpp64[p];
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+            if ((m >> r) & 1u) f2[r] += (long long)acc[r] + c2;
+        }
       }
-      if (threadIdx.x == 0) s_any |= imp;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) f2[r] += __shfl_xor_sync(0xffffffffu, f2[r], o);
+        if (lane == 0) red[warp][r] = f2[r];
+      }
+      if (threadIdx.x == 0) s_improved = 0u;
+      __syncthreads();
+      if (threadIdx.x < R) {
+        const int r = threadIdx.x;
+        long long sum = 0;
+#pragma unroll 4
+        for (int w = 0; w < RST_WARPS; ++w) sum += red[w][r];
+        if (r < nlive) {
+          const long long F = sum / 2;
+          if (F < s_bestF[r]) {   // strict: equal values keep the earliest t
+            s_bestF[r] = F;
+            s_bestT[r] = t;
+            atomicOr(&s_improved, 1u << r);
+          }
+          P.evalF[r0 + r] = F;
+          const int64_t e_idx = P.e0 + evals_upto(t, P.K, P.T) - evals_upto(P.t0, P.K, P.T) - 1;
+          if (e_idx < P.trace_cap) atomicMin(&P.trace[e_idx], F);
+        }
+      }
+      __syncthreads();
+      const uint32_t imp = s_improved;
+      if (imp) {
+        for (int p = p0; p < npos; p += RST_THREADS) best[p] = (uint8_t)((best[p] & ~imp) | (bb[p] & imp));
+        if (threadIdx.x == 0) s_any |= imp;
+      }
     }
-    ++e_idx;
-    next_eval = ((P.t0 + it) / P.K + 1) * P.K;
-    if (P.T > P.t0 + it && P.T < next_eval) next_eval = P.T;
-  }
-  __syncthreads();
+    __syncthreads();
 
-  // write back: x, y and the operand of the next iteration, and the best records that changed
-  const uint32_t any = s_any;
+    // write back: x and y, and the best records that changed
+    const uint32_t any = s_any;
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int p = p0 + q * RST_THREADS;
-    if (p >= n) continue;
-    const int64_t idx = (int64_t)P.perm[p] * a.ld + r0;
+    for (int q = 0; q < Q; ++q) {
+      if (warp + q * RST_WARPS >= P.slices) break;
+      const int p = p0 + q * RST_THREADS;
+      float x[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (r >= nlive) continue;
-      const float x = xc[(size_t)p * R + r];
-      a.Y[idx + r] = y[q][r];
-      if (BF16) {
-        a.Xm[idx + r] = x;
-        static_cast<__nv_bfloat16*>(P.xop)[idx + r] = __float2bfloat16_rn(x);
-      } else {
-        static_cast<float*>(P.xop)[idx + r] = x;
-      }
-      if ((any >> r) & 1u) P.bestBits[idx + r] = (best[p] >> r) & 1u;
+      for (int r = 0; r < R; ++r) x[r] = xc[p * R + r];
+      st_vec<R>(Xu + (size_t)p * R, x);
+      st_vec<R>(Yu + (size_t)p * R, y[q]);
     }
+    if (any) {
+      uint8_t* bu = P.best + (size_t)u * npos;
+      for (int p = p0; p < npos; p += RST_THREADS) bu[p] = (uint8_t)((__ldcg(bu + p) & ~any) | (best[p] & any));
+    }
+    if ((int)threadIdx.x < nlive && ((any >> threadIdx.x) & 1u)) {
+      P.bestF[r0 + threadIdx.x] = s_bestF[threadIdx.x];
+      P.bestT[r0 + threadIdx.x] = s_bestT[threadIdx.x];
+    }
+    if (u == 0 && c == P.chunks - 1 && threadIdx.x == 0) {
+      *P.n_evals = P.n_evals_new;
+      *P.t_last = P.t_last_new;
+    }
+    if (P.chunks == 1) return;
+    __threadfence();
+    __syncthreads();   // every thread's stores before the count that publishes them
+    if (threadIdx.x == 0) red_release_gpu_add(P.sched + 2 + u, 1u);
   }
-  if ((int)threadIdx.x < nlive && ((any >> threadIdx.x) & 1u)) {
-    P.bestF[r0 + threadIdx.x] = s_bestF[threadIdx.x];
-    P.bestT[r0 + threadIdx.x] = s_bestT[threadIdx.x];
+}
+
+// x^0 and y^0 in the unit layout: from the caller ([r][i], values checked as in k_init_state) or from
+// SplitMix64 and ybar; positions and restarts beyond the problem are zero.
+__global__ void k_restart_init(int n, int npos, int B, int R, const int32_t* __restrict__ perm, uint64_t seed,
+                               float ybar, const float* __restrict__ x0, const float* __restrict__ y0, float* X,
+                               float* Y, uint32_t* err) {
+  const int64_t per = (int64_t)npos * R, total = per * ((B + R - 1) / R);
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = e / per * R + e % R;
+    const int p = (int)(e % per / R);
+    float x = 0.0f, y = 0.0f;
+    if (p < n && r < B) {
+      const int64_t i = perm[p];
+      x = x0 ? x0[r * n + i] : uniform24(seed, (uint64_t)r, (uint64_t)i);
+      if (!(x >= 0.0f && x <= 1.0f)) {  // also rejects NaN
+        atomicOr(err, ERR_BOUNDS);
+        x = 0.5f;
+      }
+      y = y0 ? y0[r * n + i] : ybar;
+    }
+    X[e] = x;
+    Y[e] = y;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *P.n_evals = P.n_evals_new;
-    *P.t_last = P.t_last_new;
+}
+
+// [B][n] copy of a state array in the unit layout (read-back); pos: position of a vertex.
+__global__ void k_restart_gather(const float* __restrict__ src, const int32_t* __restrict__ pos, int n, int npos, int B,
+                                 int R, float* dst) {
+  for (int64_t r = blockIdx.y; r < B; r += gridDim.y) {
+    const float* s = src + (r / R) * npos * R + r % R;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+      dst[r * n + i] = s[(int64_t)pos[i] * R];
+  }
+}
+__global__ void k_restart_best_row(const uint8_t* __restrict__ best, const int32_t* __restrict__ pos, int n, int npos,
+                                   int R, int64_t r, uint8_t* dst) {
+  const uint8_t* b = best + (r / R) * npos;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    dst[i] = (b[pos[i]] >> (r % R)) & 1u;
+}
+
+// Between the unit layout and the row-wise kernels' variable-major one ([i ld + r]), 32 positions x 32
+// restarts at a time through shared memory.  to_rows: x into the operand (and the FP32 master), y, and
+// the best bits as bytes; else back.
+template <bool TO_ROWS>
+__global__ void __launch_bounds__(256) k_restart_convert(RestartLayout L) {
+  __shared__ float tx[32][33], ty[32][33];
+  __shared__ uint8_t tb[32][33];
+  const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
+  const int64_t r0 = (int64_t)blockIdx.y * 32;
+  for (int p0 = (int)blockIdx.x * 32; p0 < L.npos; p0 += (int)gridDim.x * 32) {
+    __syncthreads();
+    for (int k = ly; k < 32; k += 8) {
+      if (TO_ROWS) {   // lanes along positions
+        const int64_t r = r0 + k;
+        const int p = p0 + lx;
+        if (r < L.B && p < L.n) {
+          const size_t at = ((size_t)(r / L.R) * L.npos + p) * L.R + r % L.R;
+          tx[k][lx] = L.X[at];
+          ty[k][lx] = L.Y[at];
+          tb[k][lx] = (L.best[(size_t)(r / L.R) * L.npos + p] >> (r % L.R)) & 1u;
+        }
+      } else {         // lanes along restarts
+        const int64_t r = r0 + lx;
+        const int p = p0 + k;
+        tx[lx][k] = ty[lx][k] = 0.0f;
+        tb[lx][k] = 0;
+        if (r < L.B && p < L.n) {
+          const int64_t idx = (int64_t)L.perm[p] * L.ld + r;
+          tx[lx][k] = L.Xm ? L.Xm[idx] : static_cast<const float*>(L.Xop)[idx];
+          ty[lx][k] = L.Yrows[idx];
+          tb[lx][k] = L.bestBits[idx];
+        }
+      }
+    }
+    __syncthreads();
+    for (int k = ly; k < 32; k += 8) {
+      if (TO_ROWS) {
+        const int64_t r = r0 + lx;
+        const int p = p0 + k;
+        if (r < L.B && p < L.n) {
+          const int64_t idx = (int64_t)L.perm[p] * L.ld + r;
+          op_store(L.Xop, idx, tx[lx][k], L.op_type);
+          if (L.Xm) L.Xm[idx] = tx[lx][k];
+          L.Yrows[idx] = ty[lx][k];
+          L.bestBits[idx] = tb[lx][k];
+        }
+      } else {
+        const int64_t r = r0 + k;
+        const int p = p0 + lx;
+        if (r < (int64_t)(L.B + L.R - 1) / L.R * L.R && p < L.npos) {
+          const size_t at = ((size_t)(r / L.R) * L.npos + p) * L.R + r % L.R;
+          L.X[at] = tx[k][lx];
+          L.Y[at] = ty[k][lx];
+          if (r % L.R == 0) {
+            uint32_t m = 0u;
+            for (int q = 0; q < L.R; ++q) m |= (uint32_t)tb[k + q][lx] << q;   // R divides 32
+            L.best[(size_t)(r / L.R) * L.npos + p] = (uint8_t)m;
+          }
+        }
+      }
+    }
   }
 }
 
@@ -508,6 +660,7 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
     }
   }
   out->perm = std::move(perm);
+  out->pos = std::move(pos);
   out->cpp.assign((size_t)slices * 32, 0.0f);
   out->cpp64.assign((size_t)slices * 32, 0);
   for (int64_t p = 0; p < n; ++p) {
@@ -528,20 +681,37 @@ bool csr_restart_fits(const CsrRestartShape& sh, int R) {
   return pick_kernel(sh, R, false) != nullptr && smem_bytes(sh, R, false) <= RST_SMEM_MAX;
 }
 
+// Units (CTAs' worth of restarts) run side by side at once, and how many chunks the iterations are cut
+// into so that the last round of units leaves no SM idle: with u units on c CTAs, k chunks take
+// ceil(u k / c) chunk times, each a chunk's iterations and about one iteration's time for the load and
+// write-back of the state (4-regular graph n = 20,000, B = 512: 4 rounds -> 3.4).
+static int chunks_for(int units, int ctas, int iters) {
+  if (units <= ctas || units % ctas == 0) return 1;
+  int best = 1;
+  double best_cost = 0.0;
+  for (int k = 1; k <= 16 && iters / k >= 16; ++k) {
+    const double cost = (double)(((int64_t)units * k + ctas - 1) / ctas) * ((iters + k - 1) / k + 1.0);
+    if (k == 1 || cost < best_cost) { best = k; best_cost = cost; }
+  }
+  return best;
+}
+
 int csr_restart_pick(const CsrRestartShape& sh, int B, int sms) {
   int best = 0;
   double best_cost = 0.0;
   for (int R : {1, 2, 4}) {
     if (!csr_restart_fits(sh, R)) continue;
-    const int64_t ctas = (B + R - 1) / R;
-    const double cost = (double)((ctas + sms - 1) / sms) * (1.0 + R);
+    const int units = (B + R - 1) / R;
+    const double cost = std::max(1.0, (double)units / sms) * (1.0 + R);
     if (best == 0 || cost < best_cost) { best = R; best_cost = cost; }
   }
   return best;
 }
 
-cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_type, const float* xsrc, void* xop,
-                               const CsrRestartRun& run, int R, cudaStream_t s) {
+size_t csr_restart_positions(const CsrRestartShape& sh) { return (size_t)sh.slices * 32; }
+
+cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_type, const CsrRestartRun& run, int R,
+                               int sms, cudaStream_t s) {
   RestartKernel k = pick_kernel(d.shape, R, op_type == OP_BF16);
   if (!k || run.iters < 1) return cudaErrorInvalidValue;
   RestartParams P;
@@ -550,13 +720,15 @@ cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_
   P.ent = reinterpret_cast<const uint4*>(d.ent);
   P.wstart = d.wstart;
   P.ngroups = d.ngroups;
-  P.perm = d.perm;
   P.cpp = d.cpp;
   P.cpp64 = d.cpp64;
-  P.xsrc = xsrc;
-  P.xop = xop;
+  P.X = run.X;
+  P.Y = run.Y;
+  P.best = run.best;
+  P.sched = run.sched;
   P.slices = d.shape.slices;
   P.ent_in_smem = smem_bytes(d.shape, R, true) <= RST_SMEM_MAX;
+  P.units = (a.B + R - 1) / R;
   P.t0 = run.t0;
   P.K = run.K;
   P.T = run.T;
@@ -571,11 +743,47 @@ cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_
   P.t_last = run.t_last;
   P.n_evals_new = run.n_evals_new;
   P.t_last_new = run.t_last_new;
-  P.bestBits = run.bestBits;
+  P.timeout_ns = run.timeout_ns;
+  P.chunks = chunks_for(P.units, sms, run.iters);   // one CTA per SM: 1,024 threads of 64 registers
+  P.chunk_len = (run.iters + P.chunks - 1) / P.chunks;
+  P.chunks = (run.iters + P.chunk_len - 1) / P.chunk_len;   // none empty
   const size_t sm = smem_bytes(d.shape, R, P.ent_in_smem != 0);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RST_SMEM_MAX);
   if (e != cudaSuccess) return e;
-  k<<<(unsigned)((a.B + R - 1) / R), RST_THREADS, sm, s>>>(P);
+  if (P.chunks > 1 && (e = cudaMemsetAsync(run.sched, 0, sizeof(unsigned int) * (2 + P.units), s)) != cudaSuccess) return e;
+  k<<<(unsigned)(P.chunks > 1 ? std::min(P.units, sms) : P.units), RST_THREADS, sm, s>>>(P);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_restart_init(const CsrRestartDev& d, int n, int B, int R, uint64_t seed, float ybar, const float* x0,
+                                const float* y0, float* X, float* Y, uint32_t* err, cudaStream_t s) {
+  const int npos = d.shape.slices * 32;
+  const int64_t total = (int64_t)npos * R * ((B + R - 1) / R);
+  k_restart_init<<<(unsigned)std::min<int64_t>((total + 255) / 256, 152 * 32), 256, 0, s>>>(n, npos, B, R, d.perm, seed,
+                                                                                            ybar, x0, y0, X, Y, err);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_restart_gather(const CsrRestartDev& d, const float* src, int n, int B, int R, float* dst,
+                                  cudaStream_t s) {
+  const dim3 grid((unsigned)std::min((n + 255) / 256, 64), (unsigned)std::min(B, 65535));
+  k_restart_gather<<<grid, 256, 0, s>>>(src, d.pos, n, d.shape.slices * 32, B, R, dst);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_restart_best_row(const CsrRestartDev& d, const uint8_t* best, int n, int R, int64_t r, uint8_t* dst,
+                                    cudaStream_t s) {
+  k_restart_best_row<<<(unsigned)std::min((n + 255) / 256, 304), 256, 0, s>>>(best, d.pos, n, d.shape.slices * 32, R, r,
+                                                                              dst);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_restart_convert(const CsrRestartDev& d, RestartLayout L, bool to_rows, cudaStream_t s) {
+  L.npos = d.shape.slices * 32;
+  L.perm = d.perm;
+  const dim3 grid((unsigned)std::min(d.shape.slices, 1024), (unsigned)((L.B + 31) / 32));
+  if (to_rows) k_restart_convert<true><<<grid, 256, 0, s>>>(L);
+  else k_restart_convert<false><<<grid, 256, 0, s>>>(L);
   return cudaGetLastError();
 }
 

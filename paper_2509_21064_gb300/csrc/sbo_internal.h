@@ -122,6 +122,7 @@ int csr_partial_rows(int64_t n, int B);
 // significant bits); csr_restart_pick
 // gives the restarts per CTA for a run of B restarts.
 constexpr int CSR_RESTART_MAX_DEG = 256;
+constexpr int CSR_RESTART_MAX_R = 4;   // restarts per CTA: 1, 2 or 4
 struct CsrRestartShape {
   int slices = 0;
   uint32_t groups = 0;
@@ -132,7 +133,7 @@ struct CsrRestartHost {
   CsrRestartShape shape;
   std::vector<uint32_t> ent, wstart;
   std::vector<uint8_t> ngroups;
-  std::vector<int32_t> perm;
+  std::vector<int32_t> perm, pos;   // vertex at a position, position of a vertex
   std::vector<float> cpp;
   std::vector<int64_t> cpp64;
 };
@@ -142,6 +143,7 @@ struct CsrRestartDev {
   uint32_t* wstart = nullptr;
   uint8_t* ngroups = nullptr;
   int32_t* perm = nullptr;
+  int32_t* pos = nullptr;
   float* cpp = nullptr;
   int64_t* cpp64 = nullptr;
 };
@@ -150,14 +152,36 @@ struct CsrRestartRun {
   int iters;
   long long *bestF, *bestT, *evalF, *trace, *n_evals, *t_last;
   long long trace_cap, n_evals_new, t_last_new;   // counters after the launch
+  float *X, *Y;            // state in the unit layout: [unit of R restarts][position][R]
+  uint8_t* best;           // best candidates' bits [unit][position], bit r of a byte: restart r of the unit
+  unsigned int* sched;     // 2 + units words
+  uint64_t timeout_ns;
+};
+// Unit layout <-> the row-wise kernels' arrays (npos and perm are filled in by the launcher).
+struct RestartLayout {
+  int n, npos, B, R, op_type;
+  int64_t ld;
+  const int32_t* perm;
+  float *X, *Y;
+  uint8_t* best;
+  float *Xm, *Yrows;
+  void* Xop;
   uint8_t* bestBits;
 };
 bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
                        CsrRestartHost* out);
 bool csr_restart_fits(const CsrRestartShape& sh, int R);   // an instantiation exists and x fits on chip
 int csr_restart_pick(const CsrRestartShape& sh, int B, int sms);
-cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_type, const float* xsrc, void* xop,
-                               const CsrRestartRun& run, int R, cudaStream_t s);
+size_t csr_restart_positions(const CsrRestartShape& sh);
+cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_type, const CsrRestartRun& run, int R,
+                               int sms, cudaStream_t s);
+cudaError_t launch_restart_init(const CsrRestartDev& d, int n, int B, int R, uint64_t seed, float ybar, const float* x0,
+                                const float* y0, float* X, float* Y, uint32_t* err, cudaStream_t s);
+cudaError_t launch_restart_gather(const CsrRestartDev& d, const float* src, int n, int B, int R, float* dst,
+                                  cudaStream_t s);
+cudaError_t launch_restart_best_row(const CsrRestartDev& d, const uint8_t* best, int n, int R, int64_t r, uint8_t* dst,
+                                    cudaStream_t s);
+cudaError_t launch_restart_convert(const CsrRestartDev& d, RestartLayout L, bool to_rows, cudaStream_t s);
 // k_csr_staged.cu: the update with every row's operands staged in shared memory by bulk copies
 // (CSR_FORM_STAGED); max_deg is the largest row length of A.  csr_staged_shape reports its stage
 // layout and false when it does not apply (fewer than four stages fit).
