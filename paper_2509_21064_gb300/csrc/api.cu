@@ -963,97 +963,6 @@ sbo_status tune_csr_form(sbo_problem* p, int* out, bool lookup_only) {
   return SBO_OK;
 }
 
-// Autotuner of the restart-resident runs: times iterations of the row-wise form in use and of the
-// resident kernel with 1, 2 and 4 restarts per CTA (the difference of a long and a short launch, which
-// leaves out the load and write-back of the state), on this run's buffers before x^0 is written.  *R
-// gets the fastest's restarts per CTA, or 0 for the row-wise kernels.  Kept like the other decisions;
-// lookup_only: true only when a decision is on record.
-bool tune_restart_known(sbo_problem* p, const std::string& key, std::mutex& mu, std::map<std::string, int>& cache, int* R) {
-  std::lock_guard<std::mutex> lock(mu);
-  auto it = cache.find(key);
-  if (it != cache.end()) { *R = it->second; return true; }
-  int t = 0;
-  if (tune_cache_lookup(key, &t, [](int v) { return v == 0 || v == 1 || v == 2 || v == 4; }) &&
-      (t == 0 || csr_restart_fits(p->rst.shape, t))) {
-    cache[key] = t;
-    *R = t;
-    return true;
-  }
-  return false;
-}
-sbo_status tune_restart(sbo_problem* p, int* R, bool lookup_only, bool* known) {
-  static std::mutex mu;
-  static std::map<std::string, int> cache;
-  std::ostringstream k;
-  k << "rst2:" << tune_device(p) << ":n" << p->n << ":nnz" << p->nnz << ":deg" << p->max_deg << ":grp"
-    << p->rst.shape.groups << ":B" << p->B << ":op" << p->op_type;
-  const std::string key = k.str();
-  *known = tune_restart_known(p, key, mu, cache, R);
-  if (*known || lookup_only) return SBO_OK;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  SBO_CUDA(cudaEventCreate(&e0));
-  SBO_CUDA(cudaEventCreate(&e1));
-  CsrRestartRun r = restart_run_args(p);
-  r.K = r.T = INT64_MAX / 2;   // no evaluation
-  const EpiArgs a = base_args(p);
-  cudaError_t e = cudaMemsetAsync(p->rX, 0, ((size_t)p->B + CSR_RESTART_MAX_R - 1) * csr_restart_positions(p->rst.shape) * 4, p->stream);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(p->rY, 0, ((size_t)p->B + CSR_RESTART_MAX_R - 1) * csr_restart_positions(p->rst.shape) * 4, p->stream);
-  // device time of launch() in ms, the better of two
-  auto timed = [&](auto&& launch) {
-    float best = 1e30f;
-    for (int round = 0; round < 2 && e == cudaSuccess; ++round) {
-      if (e == cudaSuccess) e = cudaEventRecord(e0, p->stream);
-      if (e == cudaSuccess) e = launch();
-      if (e == cudaSuccess) e = cudaEventRecord(e1, p->stream);
-      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-      float ms = 0.f;
-      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-      best = std::min(best, ms);
-    }
-    return best;
-  };
-  const int reps = 16;
-  int par = 0;
-  float best_ms = timed([&] {
-                    cudaError_t q = cudaSuccess;
-                    for (int it = 0; it < reps && q == cudaSuccess; ++it, par ^= 1) {
-                      EpiArgs b = a;
-                      b.Xin = p->Xop[par];
-                      b.Xout = p->Xop[par ^ 1];
-                      q = contract(p, b, EPI_UPDATE, par, p->stream);
-                    }
-                    return q;
-                  }) / reps;
-  int best = 0;
-  for (int cand : {1, 2, 4}) {
-    if (e != cudaSuccess || !csr_restart_fits(p->rst.shape, cand)) continue;
-    auto run = [&](int iters) {
-      return timed([&] {
-        r.iters = iters;
-        ++p->launches;
-        return launch_csr_restart(p->rst, a, p->op_type, r, cand, p->sms, p->stream);
-      });
-    };
-    const float lo = run(4 * reps), hi = run(12 * reps);   // long enough to be cut into chunks like a run
-    const float ms = (hi - lo) / (8 * reps);
-    if (e == cudaSuccess && ms < best_ms) { best_ms = ms; best = cand; }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  if (e != cudaSuccess) return cuda_fail(e, "restart autotuner launch");
-  sbo_status st = read_err(p);
-  if (st != SBO_OK) return st;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    cache[key] = best;
-    tune_cache_store(key, best);
-  }
-  *R = best;
-  *known = true;
-  return SBO_OK;
-}
-
 sbo_status check_params(const sbo_gda_params* q) {
   if (!q) return fail(SBO_EINVAL, "params is NULL");
   if (q->restarts < 1) return fail(SBO_EINVAL, "restarts must be >= 1");
@@ -1545,22 +1454,14 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   auto al = [&](void** q, size_t bytes) {
     if (e == cudaSuccess) e = cudaMallocAsync(q, bytes ? bytes : 1, p->stream);
   };
-  // A sparse run that is known to go restart by restart starts in that layout: the row-wise arrays
-  // are allocated only if a later call needs them.
+  // A sparse run that goes restart by restart starts in that layout: the row-wise arrays are allocated
+  // (and the row-wise form left to its rule or an earlier decision) only if a later call needs them.
   p->rst_R = 0;
   p->single = p->opt_dual == 1;
   const bool try_restart =
       ker == KER_CSR && !p->single && p->opt_csr_form == 0 && !p->opt_keep_grad && restart_wanted(p);
-  bool restart_known = true;   // (without the autotuner: the fixed rule)
-  if (try_restart) {
-    if (!p->opt_autotune) {
-      p->rst_R = csr_restart_pick(p->rst.shape, p->B, p->sms);
-    } else {
-      sbo_status st2 = tune_restart(p, &p->rst_R, true, &restart_known);
-      if (st2 != SBO_OK) return st2;
-    }
-  }
-  bool home = p->rst_R > 0;
+  if (try_restart) p->rst_R = csr_restart_pick(p->rst.shape, p->n, p->nnz, p->B, p->sms);
+  const bool home = p->rst_R > 0;
   if (!home) {
     if (need_master) al((void**)&p->Xm, xelems * 4);
     al((void**)&p->Y, elems * 4);
@@ -1572,7 +1473,7 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
     }
     al((void**)&p->bestBits, elems);
   }
-  if (e == cudaSuccess && (home || !restart_known)) e = alloc_units(p);
+  if (e == cudaSuccess && home) e = alloc_units(p);
   al((void**)&p->bestF, sizeof(long long) * p->B);
   al((void**)&p->bestT, sizeof(long long) * p->B);
   al((void**)&p->evalF, sizeof(long long) * p->B);
@@ -1687,11 +1588,6 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
       sbo_status st2 = tune_csr_form(p, &f, home);   // on the zeroed state, before x^0 is written
       if (st2 != SBO_OK) { free_run(p); return st2; }
       p->csr_form = f;
-    }
-    if (!restart_known) {
-      sbo_status st2 = tune_restart(p, &p->rst_R, false, &restart_known);   // on the zeroed state too
-      if (st2 != SBO_OK) { free_run(p); return st2; }
-      home = p->rst_R > 0;   // the row-wise arrays stay allocated for calls that need them
     }
     int D, S, rc;
     size_t sm;

@@ -1,0 +1,484 @@
+// Sparse runs, restart by restart: a CTA owns R restarts of the whole graph and runs many iterations
+// of Algorithm 1 on them without leaving the SM.
+//
+// The restarts are independent, so the only thing an iteration shares between SMs in the row-wise
+// kernels (k_csr.cu) is an artefact of splitting the rows over them: every iteration there reads
+// and writes all of x and y through L2 or HBM and ends at a kernel boundary.  Here a CTA keeps, for
+// its R restarts, x^t and x^{t+1} of every vertex in shared memory (two FP32 buffers that swap) and
+// y and c' in the registers of the thread that owns the vertex; an iteration gathers neighbours from
+// shared memory and ends at one __syncthreads.  Evaluations (candidate bits, exact integer
+// objective, best record) stay in the CTA too, so a run of T iterations is ceil(T / 4096) launches
+// and no graph replay.  State is read from and written back to global memory once per launch.
+//
+// Same arithmetic in the same order as k_csr: each row's neighbours are summed in ascending column
+// order with FP32 fused multiply-adds, from the FP32 x or (BF16 / E4M3 weights) from x rounded to
+// BF16, so iterates and records are bit-identical to every other form.
+//
+// Structure: vertices are placed by descending degree (stable) at positions 0, 1, ..; 32 consecutive
+// positions form a slice, one lane each.  Warp w owns slices w, w + 32, ... and walks one stream of
+// 16-byte groups: four neighbours of each lane's row, an entry holding the neighbour's place and its
+// weight (see ENT_W), rows padded to whole
+// groups of the longest of their slice with weight 0.  The stream is read from shared memory when it fits beside x, else
+// through L1 / L2, two groups ahead of its use.
+//
+// What bounds it: with the structure in shared memory (small graphs) instruction issue (70-80 % of the
+// slots) and the shared-memory wavefronts of the gathers; on larger graphs also the streams from L2
+// (n = 20,000, 4-regular, 32-bit entries: 320 KB per CTA and iteration, 7.4 TB/s over the GPU; 16-bit
+// entries halve that, 23.9 -> 20.4 us per iteration at B = 512).
+// Measured per iteration against the row-wise kernels, evaluations every 10 included: Max-Cut ER
+// n = 2,000, B = 256 5.5 -> 1.9 us; 100 x 100 torus, E4M3, B = 512 16.5 -> 8.2 us; 4-regular n = 20,000,
+// B = 512 38.6 -> 20.4 us.
+#pragma once
+#include "sbo_internal.h"
+
+namespace sbo {
+
+constexpr int RST_THREADS = 1024;
+constexpr int RST_SPARE = 2;   // groups a warp reads ahead of their use
+constexpr int RST_WARPS = RST_THREADS / 32;
+constexpr int RST_PAD = 32;     // positions after the last one whose x is 0
+constexpr size_t RST_SMEM_MAX = 225 * 1024;   // dynamic; the static arrays take up to 1.2 KB of the 227
+
+struct RestartParams {
+  EpiArgs a;
+  const void* ent;               // group streams (global)
+  uint32_t wbits;                // narrow entries: the weights' magnitude
+  const uint32_t* wstart;        // [33] first group (32 lanes) of each warp's stream, and the end
+  const uint8_t* ngroups;        // [slices] groups of each slice
+  const float* cpp;              // [positions] c' by position (0 beyond n)
+  const int64_t* cpp64;
+  float *X, *Y;                  // state [unit][position][R] (unit: R restarts)
+  uint8_t* best;                 // bits of the best candidates [unit][position], bit r of a byte: restart r
+  unsigned int* sched;           // chunks > 1: [ticket, abort, chunks finished per unit]
+  int slices, ent_in_smem, units, chunks, chunk_len;
+  int64_t t0, K, T, e0;          // iterations t0 + 1 .. t0 + iters; evaluate at multiples of K and at T
+  int iters;
+  long long *bestF, *bestT, *evalF, *trace, *n_evals, *t_last;
+  long long trace_cap, t_last_new, n_evals_new;
+  uint64_t timeout_ns;
+};
+
+using RestartKernel = void (*)(RestartParams);
+RestartKernel pick_wide(const CsrRestartShape& sh, int R, bool bf16);
+RestartKernel pick_narrow(const CsrRestartShape& sh, int R, bool bf16);
+
+namespace {
+
+// Evaluation points among iterations 1 .. t (multiples of K, and T).
+__device__ __forceinline__ int64_t evals_upto(int64_t t, int64_t K, int64_t T) {
+  return t / K + (T > 0 && T <= t && T % K != 0 ? 1 : 0);
+}
+
+// State vectors of one position: R consecutive floats, through L2 (another SM may have written them).
+template <int R>
+__device__ __forceinline__ void ld_state(const float* p, float (&v)[R]) {
+  if (R == 1) {
+    v[0] = __ldcg(p);
+  } else if (R == 2) {
+    const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
+    v[0] = t.x; v[R - 1] = t.y;
+  } else {
+    const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
+    v[0] = t.x; v[1 % R] = t.y; v[2 % R] = t.z; v[3 % R] = t.w;
+  }
+}
+template <int R>
+__device__ __forceinline__ void st_vec(float* p, const float (&v)[R]) {
+  if (R == 1) *p = v[0];
+  else if (R == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[R - 1]);
+  else *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1 % R], v[2 % R], v[3 % R]);
+}
+
+// Entries of the streams, four per lane and group.
+//   Wide (32 bits): the neighbour's position, shifted so that masking gives the byte offset of its x in a
+//   buffer of BASE restarts per position, and the weight's top 15 bits (sign, exponent and 6 bits of
+//   mantissa: every |w| <= 127, even ones to 254, and so on).  Padding: the lane's own position, weight 0.
+//   Narrow (16 bits): position and sign, for graphs whose weights share one magnitude (unit and +-1
+//   graphs): half the bytes of the streams.  Padding: the position after the last, whose x stays 0.
+constexpr uint32_t ENT_W = 0xfffe0000u;
+template <bool NARROW> struct Group { using T = uint4; };
+template <> struct Group<true> { using T = uint2; };
+
+// Byte offset for R restarts of a position's x, from its offset for BASE restarts.
+template <int R, int BASE>
+__device__ __forceinline__ uint32_t scale_offset(uint32_t o) {
+  return R == BASE ? o : R < BASE ? o >> 1 : R == 2 * BASE ? o << 1 : o << 2;
+}
+// The k-th entry of a group: byte offset of the neighbour's x for R restarts, and its weight.
+template <int R, int BASE>
+__device__ __forceinline__ void entry(const uint4& c, int k, uint32_t, uint32_t& off, float& w) {
+  const uint32_t e = k == 0 ? c.x : k == 1 ? c.y : k == 2 ? c.z : c.w;
+  off = scale_offset<R, BASE>(e & ~ENT_W);
+  w = __uint_as_float(e & ENT_W);
+}
+template <int R, int BASE>
+__device__ __forceinline__ void entry(const uint2& c, int k, uint32_t wbits, uint32_t& off, float& w) {
+  const uint32_t e = k < 2 ? c.x : c.y;
+  constexpr int S = R == 1 ? 2 : R == 2 ? 3 : 4;
+  if (k & 1) {
+    off = (e >> (16 - S)) & (0x7fffu << S);
+    w = __uint_as_float((e & 0x80000000u) ^ wbits);
+  } else {
+    off = (e << S) & (0x7fffu << S);
+    w = __uint_as_float(((e << 16) & 0x80000000u) ^ wbits);
+  }
+}
+
+// The four neighbours of one group: their x as the contraction sees it (BF16: rounded to nearest, two
+// values per conversion), added in order.
+template <int R, bool BF16, int BASE, class G>
+__device__ __forceinline__ void gather4(const float* xc, const G& c, uint32_t wbits, float (&acc)[R]) {
+  float v[4][R], w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    uint32_t off;
+    entry<R, BASE>(c, k, wbits, off, w[k]);
+    const char* p = reinterpret_cast<const char*>(xc) + off;
+    if (R == 1) {
+      v[k][0] = *reinterpret_cast<const float*>(p);
+    } else if (R == 2) {
+      const float2 t = *reinterpret_cast<const float2*>(p);
+      v[k][0] = t.x; v[k][R - 1] = t.y;
+    } else {
+      const float4 t = *reinterpret_cast<const float4*>(p);
+      v[k][0] = t.x; v[k][1 % R] = t.y; v[k][2 % R] = t.z; v[k][3 % R] = t.w;
+    }
+  }
+  if (BF16) {
+#pragma unroll
+    for (int j = 0; j < 4 * R; j += 2) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(v[j / R][j % R], v[(j + 1) / R][(j + 1) % R]);
+      v[j / R][j % R] = __low2float(h);
+      v[(j + 1) / R][(j + 1) % R] = __high2float(h);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = fmaf(w[k], v[k][r], acc[r]);
+}
+
+// The same sums over candidate bits.
+template <int R, class G>
+__device__ __forceinline__ void add_bits4(const uint8_t* bb, const G& c, uint32_t wbits, int shift, float (&acc)[R]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    uint32_t off;
+    float w;
+    if (sizeof(G) == 16) {
+      entry<1, 1>(c, k, wbits, off, w);   // wide: the offset as stored
+      off >>= shift;
+    } else {
+      entry<1, 1>(c, k, wbits, off, w);
+      off >>= 2;
+    }
+    const uint32_t m = bb[off];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] += ((m >> r) & 1u) ? w : 0.0f;
+  }
+}
+
+// One iteration's work on one vertex after its neighbour sums: update of R restarts.
+template <int R>
+__device__ __forceinline__ void update(const EpiArgs& a, const float* xc, float* xn, const float (&acc)[R], float cp,
+                                       float (&y)[R]) {
+  float xo[R], xv[R];
+  if (R == 1) {
+    xo[0] = *xc;
+  } else if (R == 2) {
+    const float2 t = *reinterpret_cast<const float2*>(xc);
+    xo[0] = t.x; xo[R - 1] = t.y;
+  } else {
+    const float4 t = *reinterpret_cast<const float4*>(xc);
+    xo[0] = t.x; xo[1 % R] = t.y; xo[2 % R] = t.z; xo[3 % R] = t.w;
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const float x = xo[r];
+    const float gx = g_val(x, G_QUAD);
+    const float d = acc[r] + cp + y[r] * g_der(x, G_QUAD);
+    // pdbo_update (common.cuh) with the projection as a saturation: the same value
+    const bool stagnating = fabsf(x - 0.5f) <= a.delta && fabsf(d) <= a.grad_tol && y[r] <= 0.0f;
+    xv[r] = __saturatef(x - a.alpha * d);
+    if (stagnating) xv[r] = x <= 0.5f ? 0.5f - a.delta : 0.5f + a.delta;
+    y[r] = y[r] + a.beta * gx;
+  }
+  st_vec<R>(xn, xv);
+}
+
+// Q: slices per warp at most (y and c' of a thread's vertices live in registers: Q R + Q, or Q R + Q / 2
+// with c' packed as BF16 pairs when PACK).  R: restarts per CTA.  ONE: every row has at most four
+// neighbours (one group per slice).
+template <int Q, int R, bool BF16, bool ONE, bool PACK, bool NARROW>
+__global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_constant__ RestartParams P) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int npos = P.slices * 32;
+  using G = typename Group<NARROW>::T;
+  const int nx_pos = npos + RST_PAD;                                   // positions of a buffer, the zero ones too
+  float* xs = reinterpret_cast<float*>(smem);                          // [2][nx_pos][R]
+  G* ent_s = reinterpret_cast<G*>(xs + 2 * (size_t)nx_pos * R);        // group streams (when they fit)
+  const G* ent_g = static_cast<const G*>(P.ent);
+  const uint32_t groups = P.wstart[RST_WARPS];
+  const size_t ent_bytes = P.ent_in_smem ? ((size_t)groups + RST_SPARE) * 32 * sizeof(G) : 0;
+  uint8_t* bb = reinterpret_cast<uint8_t*>(ent_s) + ent_bytes;         // candidate bits, one per restart
+  uint8_t* best = bb + nx_pos;                                         // bits of the best candidates
+  uint8_t* ngr = best + npos;                                          // groups of each slice
+  __shared__ long long red[RST_WARPS][R];
+  __shared__ long long s_bestF[R], s_bestT[R];
+  __shared__ uint32_t s_improved, s_any;
+  __shared__ int s_ticket;
+  // progress of the chunk, kept here and not in registers, which the state needs: t done and t at its end
+  __shared__ volatile int64_t s_t, s_end;
+
+  const EpiArgs& a = P.a;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = a.n;
+  const int p0 = threadIdx.x;   // this thread's vertices: positions p0, p0 + RST_THREADS, ..
+  constexpr int BASE = Q > 10 ? 1 : 2;            // restarts per position the entries are scaled for
+  const int shift = BASE == 1 ? 2 : 3;            // entry offset -> position
+
+  if (P.ent_in_smem)
+    for (uint32_t k = threadIdx.x; k < (groups + RST_SPARE) * 32; k += RST_THREADS) ent_s[k] = ent_g[k];
+  for (int k = threadIdx.x; k < RST_PAD * R; k += RST_THREADS)   // x of the zero positions, in both buffers
+    xs[npos * R + k] = xs[(nx_pos + npos) * R + k] = 0.0f;
+  if (threadIdx.x < RST_PAD) bb[npos + threadIdx.x] = 0;
+  for (int k = threadIdx.x; k < P.slices; k += RST_THREADS) ngr[k] = P.ngroups[k];
+  constexpr int AHEAD = ONE || (NARROW && Q <= 10) ? RST_SPARE : 1;   // groups in flight per warp (registers allowing)
+  const uint32_t stream0 = P.wstart[warp] * 32 + lane;
+  constexpr int NC = PACK ? (Q + 1) / 2 : Q;
+  float cps[PACK ? 1 : NC];
+  uint32_t cpk[PACK ? NC : 1];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const float c = warp + q * RST_WARPS < P.slices ? P.cpp[p0 + q * RST_THREADS] : 0.0f;
+    if (!PACK) cps[PACK ? 0 : q] = c;
+    else if (q & 1) cpk[PACK ? q / 2 : 0] |= __float_as_uint(c) & 0xffff0000u;
+    else cpk[PACK ? q / 2 : 0] = __float_as_uint(c) >> 16;
+  }
+
+  // Work: (chunk of iterations, unit) pairs.  With one chunk a CTA runs its unit; with more, CTAs
+  // take tickets in order (all units' first chunk, then all second ones, ..) and a chunk starts once
+  // its unit's previous one is finished, which a CTA with an earlier ticket is running or has done.
+  for (;;) {
+    int u = (int)blockIdx.x, c = 0;
+    if (P.chunks > 1) {
+      if (threadIdx.x == 0) {
+        int t = (int)atomicAdd(P.sched, 1u);
+        if (t >= P.units * P.chunks) {
+          t = -1;
+        } else if (t >= P.units) {
+          const uint64_t deadline = globaltimer_ns() + P.timeout_ns;
+          const unsigned int* done = P.sched + 2 + t % P.units;
+          while (ld_acquire_gpu(done) < (unsigned)(t / P.units)) {
+            if (ld_acquire_gpu(P.sched + 1) != 0u || globaltimer_ns() > deadline) {
+              atomicOr(a.err, ERR_TIMEOUT);
+              atomicExch(P.sched + 1, 1u);   // ends every other CTA's waits too
+              t = -1;
+              break;
+            }
+            __nanosleep(200);
+          }
+        }
+        s_ticket = t;
+      }
+      __syncthreads();
+      const int t = s_ticket;
+      if (t < 0) return;
+      u = t % P.units;
+      c = t / P.units;
+    }
+    if (threadIdx.x < R) {
+      const int r = u * R + (int)threadIdx.x;
+      s_bestF[threadIdx.x] = r < a.B ? __ldcg(&P.bestF[r]) : 0;
+      s_bestT[threadIdx.x] = r < a.B ? __ldcg(&P.bestT[r]) : 0;
+    }
+    if (threadIdx.x == 0) {
+      s_any = 0u;
+      s_ticket = c * P.units + u;
+      s_t = P.t0 + (int64_t)c * P.chunk_len;
+      s_end = P.t0 + min((int64_t)(c + 1) * P.chunk_len, (int64_t)P.iters);
+    }
+    float y[Q][R];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) y[q][r] = 0.0f;
+      if (warp + q * RST_WARPS < P.slices) {
+        const int p = p0 + q * RST_THREADS;
+        float x[R];
+        ld_state<R>(P.X + ((size_t)u * npos + p) * R, x);
+        ld_state<R>(P.Y + ((size_t)u * npos + p) * R, y[q]);
+        st_vec<R>(xs + p * R, x);
+      }
+    }
+    __syncthreads();
+
+    // iterations from t to the next evaluation point
+    auto until_eval = [&](int64_t t) -> int64_t {
+      int64_t next = (t / P.K + 1) * P.K;
+      if (P.T > t && P.T < next) next = P.T;
+      return next - t;
+    };
+    const float* xc = xs;
+    float* xn = xs + nx_pos * R;
+    while (s_t < s_end) {   // stretches of iterations that end at an evaluation point or with the chunk
+      for (int left = (int)min(until_eval(s_t), (int64_t)(s_end - s_t)); left > 0; --left) {
+        const G* st = (P.ent_in_smem ? ent_s : ent_g) + stream0;
+        G nx[AHEAD];   // groups read ahead (the streams end in RST_SPARE spare groups)
+#pragma unroll
+        for (int d = 0; d < AHEAD; ++d, st += 32) nx[d] = *st;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          if (warp + q * RST_WARPS >= P.slices) break;   // no later slice either
+          const int p = p0 + q * RST_THREADS;
+          float acc[R];
+#pragma unroll
+          for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+          const int ng = ONE ? 1 : ngr[warp + q * RST_WARPS];
+          for (int g = 0; g < ng; ++g) {
+            const G e = nx[0];
+#pragma unroll
+            for (int d = 0; d + 1 < AHEAD; ++d) nx[d] = nx[d + 1];
+            nx[AHEAD - 1] = *st;
+            st += 32;
+            gather4<R, BF16, BASE>(xc, e, P.wbits, acc);
+          }
+          const float cp = !PACK ? cps[PACK ? 0 : q]
+                                 : __uint_as_float((q & 1) ? cpk[PACK ? q / 2 : 0] & 0xffff0000u : cpk[PACK ? q / 2 : 0] << 16);
+          update<R>(a, xc + p * R, xn + p * R, acc, cp, y[q]);
+        }
+        {
+          float* t = const_cast<float*>(xc);
+          xc = xn;
+          xn = t;
+        }
+        __syncthreads();
+      }
+      const int64_t t = min(s_t + until_eval(s_t), (int64_t)s_end);
+      const bool is_eval = t - s_t == until_eval(s_t);
+      __syncthreads();   // every thread has read s_t
+      if (threadIdx.x == 0) s_t = t;
+      if (!is_eval) break;   // the chunk's end
+      // candidates b = [x > 1/2]
+      for (int p = p0; p < npos; p += RST_THREADS) {
+        uint32_t m = 0u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) m |= (xc[p * R + r] > 0.5f ? 1u : 0u) << r;
+        bb[p] = (uint8_t)m;
+      }
+      __syncthreads();
+      // exact objective of the candidates: 2F = sum_i b_i ((A b)_i + 2 c'_i); (A b)_i is an exact
+      // integer in FP32 because every row sum of |A| is below 2^24
+      long long f2[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) f2[r] = 0;
+      const G* st = (P.ent_in_smem ? ent_s : ent_g) + stream0;
+      for (int s = warp; s < P.slices; s += RST_WARPS) {
+        const int ng = ONE ? 1 : ngr[s];
+        const int p = s * 32 + lane;
+        float acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+        for (int g = 0; g < ng; ++g, st += 32) add_bits4<R>(bb, *st, P.wbits, shift, acc);
+        if (p < n) {
+          const uint32_t m = bb[p];
+          const long long c2 = 2 * (long long)P.cpp64[p];
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+            if ((m >> r) & 1u) f2[r] += (long long)acc[r] + c2;
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) f2[r] += __shfl_xor_sync(0xffffffffu, f2[r], o);
+        if (lane == 0) red[warp][r] = f2[r];
+      }
+      if (threadIdx.x == 0) s_improved = 0u;
+      __syncthreads();
+      if (threadIdx.x < R) {
+        const int r = threadIdx.x;
+        long long sum = 0;
+#pragma unroll 4
+        for (int w = 0; w < RST_WARPS; ++w) sum += red[w][r];
+        const int rg = s_ticket % P.units * R + r;   // the restart
+        if (rg < a.B) {
+          const long long F = sum / 2;
+          if (F < s_bestF[r]) {   // strict: equal values keep the earliest t
+            s_bestF[r] = F;
+            s_bestT[r] = t;
+            atomicOr(&s_improved, 1u << r);
+          }
+          P.evalF[rg] = F;
+          const int64_t e_idx = P.e0 + evals_upto(t, P.K, P.T) - evals_upto(P.t0, P.K, P.T) - 1;
+          if (e_idx < P.trace_cap) atomicMin(&P.trace[e_idx], F);
+        }
+      }
+      __syncthreads();
+      const uint32_t imp = s_improved;
+      if (imp) {
+        for (int p = p0; p < npos; p += RST_THREADS) best[p] = (uint8_t)((best[p] & ~imp) | (bb[p] & imp));
+        if (threadIdx.x == 0) s_any |= imp;
+      }
+    }
+    __syncthreads();
+
+    // write back: x and y, and the best records that changed
+    const uint32_t any = s_any;
+    u = s_ticket % P.units;
+    c = s_ticket / P.units;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      if (warp + q * RST_WARPS >= P.slices) break;
+      const int p = p0 + q * RST_THREADS;
+      float x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = xc[p * R + r];
+      st_vec<R>(P.X + ((size_t)u * npos + p) * R, x);
+      st_vec<R>(P.Y + ((size_t)u * npos + p) * R, y[q]);
+    }
+    if (any) {
+      uint8_t* bu = P.best + (size_t)u * npos;
+      for (int p = p0; p < npos; p += RST_THREADS) bu[p] = (uint8_t)((__ldcg(bu + p) & ~any) | (best[p] & any));
+    }
+    if (threadIdx.x < R && ((any >> threadIdx.x) & 1u)) {   // (restarts beyond the run never improve)
+      P.bestF[u * R + threadIdx.x] = s_bestF[threadIdx.x];
+      P.bestT[u * R + threadIdx.x] = s_bestT[threadIdx.x];
+    }
+    if (u == 0 && c == P.chunks - 1 && threadIdx.x == 0) {
+      *P.n_evals = P.n_evals_new;
+      *P.t_last = P.t_last_new;
+    }
+    if (P.chunks == 1) return;
+    __threadfence();
+    __syncthreads();   // every thread's stores before the count that publishes them
+    if (threadIdx.x == 0) red_release_gpu_add(P.sched + 2 + u, 1u);
+  }
+}
+
+template <int Q, int R, bool PACK>
+RestartKernel kernel_of(bool bf16, bool one) {
+  constexpr bool N = RST_NARROW;
+  if (one) return bf16 ? (RestartKernel)k_csr_restart<Q, R, true, true, PACK, N> : (RestartKernel)k_csr_restart<Q, R, false, true, PACK, N>;
+  return bf16 ? (RestartKernel)k_csr_restart<Q, R, true, false, PACK, N> : (RestartKernel)k_csr_restart<Q, R, false, false, PACK, N>;
+}
+
+}  // namespace
+
+// Instantiations of this translation unit's entry width: slices per warp up to Q with R restarts, in 64
+// registers per thread.
+RestartKernel RST_PICK(const CsrRestartShape& sh, int R, bool bf16) {
+  const int q = (sh.slices + RST_WARPS - 1) / RST_WARPS;
+  const bool one = sh.max_groups <= 1;
+  switch (R) {
+    case 1:
+      if (q <= 3) return kernel_of<3, 1, false>(bf16, one);
+      if (q <= 10) return kernel_of<10, 1, false>(bf16, one);
+      return q <= 20 && sh.cp_bf16 ? kernel_of<20, 1, true>(bf16, one) : nullptr;
+    case 2: return q <= 3 ? kernel_of<3, 2, false>(bf16, one) : q <= 10 ? kernel_of<10, 2, false>(bf16, one) : nullptr;
+    case 4: return q <= 5 ? kernel_of<5, 4, false>(bf16, one) : nullptr;
+    default: return nullptr;
+  }
+}
+
+}  // namespace sbo

@@ -1,413 +1,14 @@
-// Sparse runs, restart by restart: a CTA owns R restarts of the whole graph and runs many iterations
-// of Algorithm 1 on them without leaving the SM.
-//
-// The restarts are independent, so the only thing an iteration shares between SMs in the row-wise
-// kernels (k_csr.cu) is an artefact of splitting the rows over them: every iteration there reads
-// and writes all of x and y through L2 or HBM and ends at a kernel boundary.  Here a CTA keeps, for
-// its R restarts, x^t and x^{t+1} of every vertex in shared memory (two FP32 buffers that swap) and
-// y and c' in the registers of the thread that owns the vertex; an iteration gathers neighbours from
-// shared memory and ends at one __syncthreads.  Evaluations (candidate bits, exact integer
-// objective, best record) stay in the CTA too, so a run of T iterations is ceil(T / 4096) launches
-// and no graph replay.  State is read from and written back to global memory once per launch.
-//
-// Same arithmetic in the same order as k_csr: each row's neighbours are summed in ascending column
-// order with FP32 fused multiply-adds, from the FP32 x or (BF16 / E4M3 weights) from x rounded to
-// BF16, so iterates and records are bit-identical to every other form.
-//
-// Structure: vertices are placed by descending degree (stable) at positions 0, 1, ..; 32 consecutive
-// positions form a slice, one lane each.  Warp w owns slices w, w + 32, ... and walks one stream of
-// 16-byte groups: four neighbours of each lane's row, an entry holding the neighbour's place and its
-// weight (see ENT_W), rows padded to whole
-// groups of the longest of their slice with weight 0.  The stream is read from shared memory when it fits beside x, else
-// through L1 / L2, two groups ahead of its use.
-//
-// What bounds it: shared-memory wavefronts of the gathers (a random graph's 32 4-byte gathers meet
-// about 3.5 bank conflicts deep) and the latency of the streams from L2, not HBM or the launch.
-// Measured per iteration against the row-wise kernels, evaluations every 10 included: Max-Cut ER
-// n = 2,000, B = 256 5.4 -> 2.44 us; 100 x 100 torus, B = 512 16.0 -> 9.4 us; 4-regular n = 20,000,
-// B = 512 38.6 -> 33.4 us.
+// Restart-resident sparse runs (csr_restart.cuh): the kernels with 32-bit entries, the host side (layout
+// of the structure, the rule, the launch) and the kernels around the state's unit layout.
+#define RST_NARROW false
+#define RST_PICK pick_wide
+#include "csr_restart.cuh"
+
 #include <algorithm>
 #include <cstring>
 
-#include "sbo_internal.h"
-
 namespace sbo {
 namespace {
-
-constexpr int RST_THREADS = 1024;
-constexpr int RST_SPARE = 2;   // groups a warp reads ahead of their use
-constexpr int RST_WARPS = RST_THREADS / 32;
-constexpr size_t RST_SMEM_MAX = 225 * 1024;   // dynamic; the static arrays take up to 1.2 KB of the 227
-
-struct RestartParams {
-  EpiArgs a;
-  const uint4* ent;              // group streams (global)
-  const uint32_t* wstart;        // [33] first group (of 32 uint4) of each warp's stream, and the end
-  const uint8_t* ngroups;        // [slices] groups of each slice
-  const float* cpp;              // [positions] c' by position (0 beyond n)
-  const int64_t* cpp64;
-  float *X, *Y;                  // state [unit][position][R] (unit: R restarts)
-  uint8_t* best;                 // bits of the best candidates [unit][position], bit r of a byte: restart r
-  unsigned int* sched;           // chunks > 1: [ticket, abort, chunks finished per unit]
-  int slices, ent_in_smem, units, chunks, chunk_len;
-  int64_t t0, K, T, e0;          // iterations t0 + 1 .. t0 + iters; evaluate at multiples of K and at T
-  int iters;
-  long long *bestF, *bestT, *evalF, *trace, *n_evals, *t_last;
-  long long trace_cap, t_last_new, n_evals_new;
-  uint64_t timeout_ns;
-};
-
-// Evaluation points among iterations 1 .. t (multiples of K, and T).
-__device__ __forceinline__ int64_t evals_upto(int64_t t, int64_t K, int64_t T) {
-  return t / K + (T > 0 && T <= t && T % K != 0 ? 1 : 0);
-}
-
-// State vectors of one position: R consecutive floats, through L2 (another SM may have written them).
-template <int R>
-__device__ __forceinline__ void ld_state(const float* p, float (&v)[R]) {
-  if (R == 1) {
-    v[0] = __ldcg(p);
-  } else if (R == 2) {
-    const float2 t = __ldcg(reinterpret_cast<const float2*>(p));
-    v[0] = t.x; v[R - 1] = t.y;
-  } else {
-    const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
-    v[0] = t.x; v[1 % R] = t.y; v[2 % R] = t.z; v[3 % R] = t.w;
-  }
-}
-template <int R>
-__device__ __forceinline__ void st_vec(float* p, const float (&v)[R]) {
-  if (R == 1) *p = v[0];
-  else if (R == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[R - 1]);
-  else *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1 % R], v[2 % R], v[3 % R]);
-}
-
-// An entry of the streams: the neighbour's position, shifted so that masking gives the byte offset of
-// its x in a buffer of `base` restarts per position, and the weight's top 15 bits (sign, exponent and 6
-// bits of mantissa: every |w| <= 127, even ones to 254, and so on).
-constexpr uint32_t ENT_W = 0xfffe0000u;
-template <int R>
-__device__ __forceinline__ uint32_t entry_offset(uint32_t e, int base) {   // byte offset for R restarts
-  const uint32_t o = e & ~ENT_W;
-  if (R == 1) return base == 1 ? o : o >> 1;
-  return R == 2 ? o : o << 1;
-}
-
-// The four neighbours of one group: their x as the contraction sees it (BF16: rounded to nearest, two
-// values per conversion), added in order.
-template <int R, bool BF16, int BASE>
-__device__ __forceinline__ void gather4(const float* xc, const uint4& c, float (&acc)[R]) {
-  const uint32_t e[4] = {c.x, c.y, c.z, c.w};
-  float v[4][R];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const char* p = reinterpret_cast<const char*>(xc) + entry_offset<R>(e[k], BASE);
-    if (R == 1) {
-      v[k][0] = *reinterpret_cast<const float*>(p);
-    } else if (R == 2) {
-      const float2 t = *reinterpret_cast<const float2*>(p);
-      v[k][0] = t.x; v[k][R - 1] = t.y;
-    } else {
-      const float4 t = *reinterpret_cast<const float4*>(p);
-      v[k][0] = t.x; v[k][1 % R] = t.y; v[k][2 % R] = t.z; v[k][3 % R] = t.w;
-    }
-  }
-  if (BF16) {
-#pragma unroll
-    for (int j = 0; j < 4 * R; j += 2) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(v[j / R][j % R], v[(j + 1) / R][(j + 1) % R]);
-      v[j / R][j % R] = __low2float(h);
-      v[(j + 1) / R][(j + 1) % R] = __high2float(h);
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float w = __uint_as_float(e[k] & ENT_W);
-#pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = fmaf(w, v[k][r], acc[r]);
-  }
-}
-
-template <int R>
-__device__ __forceinline__ void add_bits(const uint8_t* bb, uint32_t e, int shift, float (&acc)[R]) {
-  const float w = __uint_as_float(e & ENT_W);
-  const uint32_t m = bb[(e & ~ENT_W) >> shift];
-#pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] += ((m >> r) & 1u) ? w : 0.0f;
-}
-
-// One iteration's work on one vertex after its neighbour sums: update of R restarts.
-template <int R>
-__device__ __forceinline__ void update(const EpiArgs& a, const float* xc, float* xn, const float (&acc)[R], float cp,
-                                       float (&y)[R]) {
-  float xo[R], xv[R];
-  if (R == 1) {
-    xo[0] = *xc;
-  } else if (R == 2) {
-    const float2 t = *reinterpret_cast<const float2*>(xc);
-    xo[0] = t.x; xo[R - 1] = t.y;
-  } else {
-    const float4 t = *reinterpret_cast<const float4*>(xc);
-    xo[0] = t.x; xo[1 % R] = t.y; xo[2 % R] = t.z; xo[3 % R] = t.w;
-  }
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const float x = xo[r];
-    const float gx = g_val(x, G_QUAD);
-    const float d = acc[r] + cp + y[r] * g_der(x, G_QUAD);
-    // pdbo_update (common.cuh) with the projection as a saturation: the same value
-    const bool stagnating = fabsf(x - 0.5f) <= a.delta && fabsf(d) <= a.grad_tol && y[r] <= 0.0f;
-    xv[r] = __saturatef(x - a.alpha * d);
-    if (stagnating) xv[r] = x <= 0.5f ? 0.5f - a.delta : 0.5f + a.delta;
-    y[r] = y[r] + a.beta * gx;
-  }
-  st_vec<R>(xn, xv);
-}
-
-// Q: slices per warp at most (y and c' of a thread's vertices live in registers: Q R + Q, or Q R + Q / 2
-// with c' packed as BF16 pairs when PACK).  R: restarts per CTA.  ONE: every row has at most four
-// neighbours (one group per slice).
-template <int Q, int R, bool BF16, bool ONE, bool PACK>
-__global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_constant__ RestartParams P) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  const int npos = P.slices * 32;
-  float* xs = reinterpret_cast<float*>(smem);                          // [2][npos][R]
-  uint4* ent_s = reinterpret_cast<uint4*>(xs + 2 * (size_t)npos * R);  // group streams (when they fit)
-  const uint32_t groups = P.wstart[RST_WARPS];
-  const size_t ent_bytes = P.ent_in_smem ? ((size_t)groups + RST_SPARE) * 32 * sizeof(uint4) : 0;
-  uint8_t* bb = reinterpret_cast<uint8_t*>(ent_s) + ent_bytes;         // candidate bits, one per restart
-  uint8_t* best = bb + npos;                                           // bits of the best candidates
-  uint8_t* ngr = best + npos;                                          // groups of each slice
-  __shared__ long long red[RST_WARPS][R];
-  __shared__ long long s_bestF[R], s_bestT[R];
-  __shared__ uint32_t s_improved, s_any;
-  __shared__ int s_ticket;
-
-  const EpiArgs& a = P.a;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int n = a.n;
-  const int p0 = warp * 32 + lane;   // this thread's vertices: positions p0, p0 + RST_THREADS, ..
-  constexpr int BASE = Q > 10 ? 1 : 2;            // restarts per position the entries are scaled for
-  const int shift = BASE == 1 ? 2 : 3;            // entry offset -> position
-
-  if (P.ent_in_smem)
-    for (uint32_t k = threadIdx.x; k < (groups + RST_SPARE) * 32; k += RST_THREADS) ent_s[k] = P.ent[k];
-  for (int k = threadIdx.x; k < P.slices; k += RST_THREADS) ngr[k] = P.ngroups[k];
-  constexpr int AHEAD = ONE ? RST_SPARE : 1;      // groups in flight per warp
-  const uint32_t stream0 = P.wstart[warp] * 32 + lane;
-  constexpr int NC = PACK ? (Q + 1) / 2 : Q;
-  float cps[PACK ? 1 : NC];
-  uint32_t cpk[PACK ? NC : 1];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const float c = warp + q * RST_WARPS < P.slices ? P.cpp[p0 + q * RST_THREADS] : 0.0f;
-    if (!PACK) cps[PACK ? 0 : q] = c;
-    else if (q & 1) cpk[PACK ? q / 2 : 0] |= __float_as_uint(c) & 0xffff0000u;
-    else cpk[PACK ? q / 2 : 0] = __float_as_uint(c) >> 16;
-  }
-
-  // Work: (chunk of iterations, unit) pairs.  With one chunk a CTA runs its unit; with more, CTAs
-  // take tickets in order (all units' first chunk, then all second ones, ..) and a chunk starts once
-  // its unit's previous one is finished, which a CTA with an earlier ticket is running or has done.
-  for (;;) {
-    int u = (int)blockIdx.x, c = 0;
-    if (P.chunks > 1) {
-      if (threadIdx.x == 0) {
-        int t = (int)atomicAdd(P.sched, 1u);
-        if (t >= P.units * P.chunks) {
-          t = -1;
-        } else if (t >= P.units) {
-          const uint64_t deadline = globaltimer_ns() + P.timeout_ns;
-          const unsigned int* done = P.sched + 2 + t % P.units;
-          while (ld_acquire_gpu(done) < (unsigned)(t / P.units)) {
-            if (ld_acquire_gpu(P.sched + 1) != 0u || globaltimer_ns() > deadline) {
-              atomicOr(a.err, ERR_TIMEOUT);
-              atomicExch(P.sched + 1, 1u);   // ends every other CTA's waits too
-              t = -1;
-              break;
-            }
-            __nanosleep(200);
-          }
-        }
-        s_ticket = t;
-      }
-      __syncthreads();
-      const int t = s_ticket;
-      if (t < 0) return;
-      u = t % P.units;
-      c = t / P.units;
-    }
-    const int r0 = u * R;
-    const int nlive = min(R, a.B - r0);
-    const int64_t t0 = P.t0 + (int64_t)c * P.chunk_len;
-    const int iters = min(P.chunk_len, P.iters - c * P.chunk_len);
-    float* Xu = P.X + (size_t)u * npos * R;
-    float* Yu = P.Y + (size_t)u * npos * R;
-
-    if (threadIdx.x < R) {
-      const bool live = (int)threadIdx.x < nlive;
-      s_bestF[threadIdx.x] = live ? __ldcg(&P.bestF[r0 + threadIdx.x]) : 0;
-      s_bestT[threadIdx.x] = live ? __ldcg(&P.bestT[r0 + threadIdx.x]) : 0;
-    }
-    if (threadIdx.x == 0) s_any = 0u;
-    float y[Q][R];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) y[q][r] = 0.0f;
-      if (warp + q * RST_WARPS < P.slices) {
-        const int p = p0 + q * RST_THREADS;
-        float x[R];
-        ld_state<R>(Xu + (size_t)p * R, x);
-        ld_state<R>(Yu + (size_t)p * R, y[q]);
-        st_vec<R>(xs + p * R, x);
-      }
-    }
-    __syncthreads();
-
-    // iterations to the next evaluation point
-    auto until_eval = [&](int64_t t) {
-      int64_t next = (t / P.K + 1) * P.K;
-      if (P.T > t && P.T < next) next = P.T;
-      return (int)min(next - t, (int64_t)1 << 30);
-    };
-    int left = until_eval(t0);
-    const float* xc = xs;
-    float* xn = xs + (size_t)npos * R;
-    for (int it = 1; it <= iters; ++it) {
-      const uint4* st = (P.ent_in_smem ? ent_s : P.ent) + stream0;
-      uint4 nx[AHEAD];   // groups read ahead (the streams end in RST_SPARE spare groups)
-#pragma unroll
-      for (int d = 0; d < AHEAD; ++d, st += 32) nx[d] = *st;
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        if (warp + q * RST_WARPS >= P.slices) break;   // no later slice either
-        const int p = p0 + q * RST_THREADS;
-        float acc[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = 0.0f;
-        const int ng = ONE ? 1 : ngr[warp + q * RST_WARPS];
-        for (int g = 0; g < ng; ++g) {
-          const uint4 e = nx[0];
-#pragma unroll
-          for (int d = 0; d + 1 < AHEAD; ++d) nx[d] = nx[d + 1];
-          nx[AHEAD - 1] = *st;
-          st += 32;
-          gather4<R, BF16, BASE>(xc, e, acc);
-        }
-        const float cp = !PACK ? cps[PACK ? 0 : q]
-                               : __uint_as_float((q & 1) ? cpk[PACK ? q / 2 : 0] & 0xffff0000u : cpk[PACK ? q / 2 : 0] << 16);
-        update<R>(a, xc + p * R, xn + p * R, acc, cp, y[q]);
-      }
-      {
-        float* t = const_cast<float*>(xc);
-        xc = xn;
-        xn = t;
-      }
-      __syncthreads();
-      if (--left != 0) continue;
-
-      // candidates b = [x > 1/2]
-      for (int p = p0; p < npos; p += RST_THREADS) {
-        uint32_t m = 0u;
-#pragma unroll
-        for (int r = 0; r < R; ++r) m |= (xc[p * R + r] > 0.5f ? 1u : 0u) << r;
-        bb[p] = (uint8_t)m;
-      }
-      __syncthreads();
-      // exact objective of the candidates: 2F = sum_i b_i ((A b)_i + 2 c'_i); (A b)_i is an exact
-      // integer in FP32 because every row sum of |A| is below 2^24
-      long long f2[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) f2[r] = 0;
-      const int64_t t = t0 + it;
-      left = until_eval(t);
-      st = (P.ent_in_smem ? ent_s : P.ent) + stream0;
-      for (int s = warp; s < P.slices; s += RST_WARPS) {
-        const int ng = ONE ? 1 : ngr[s];
-        const int p = s * 32 + lane;
-        float acc[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = 0.0f;
-        for (int g = 0; g < ng; ++g, st += 32) {
-          const uint4 e = *st;   // entries beyond a row's length are padding (weight 0)
-          add_bits<R>(bb, e.x, shift, acc);
-          add_bits<R>(bb, e.y, shift, acc);
-          add_bits<R>(bb, e.z, shift, acc);
-          add_bits<R>(bb, e.w, shift, acc);
-        }
-        if (p < n) {
-          const uint32_t m = bb[p];
-          const long long c2 = 2 * (long long)P.cpp64[p];
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-            if ((m >> r) & 1u) f2[r] += (long long)acc[r] + c2;
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) f2[r] += __shfl_xor_sync(0xffffffffu, f2[r], o);
-        if (lane == 0) red[warp][r] = f2[r];
-      }
-      if (threadIdx.x == 0) s_improved = 0u;
-      __syncthreads();
-      if (threadIdx.x < R) {
-        const int r = threadIdx.x;
-        long long sum = 0;
-#pragma unroll 4
-        for (int w = 0; w < RST_WARPS; ++w) sum += red[w][r];
-        if (r < nlive) {
-          const long long F = sum / 2;
-          if (F < s_bestF[r]) {   // strict: equal values keep the earliest t
-            s_bestF[r] = F;
-            s_bestT[r] = t;
-            atomicOr(&s_improved, 1u << r);
-          }
-          P.evalF[r0 + r] = F;
-          const int64_t e_idx = P.e0 + evals_upto(t, P.K, P.T) - evals_upto(P.t0, P.K, P.T) - 1;
-          if (e_idx < P.trace_cap) atomicMin(&P.trace[e_idx], F);
-        }
-      }
-      __syncthreads();
-      const uint32_t imp = s_improved;
-      if (imp) {
-        for (int p = p0; p < npos; p += RST_THREADS) best[p] = (uint8_t)((best[p] & ~imp) | (bb[p] & imp));
-        if (threadIdx.x == 0) s_any |= imp;
-      }
-    }
-    __syncthreads();
-
-    // write back: x and y, and the best records that changed
-    const uint32_t any = s_any;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      if (warp + q * RST_WARPS >= P.slices) break;
-      const int p = p0 + q * RST_THREADS;
-      float x[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) x[r] = xc[p * R + r];
-      st_vec<R>(Xu + (size_t)p * R, x);
-      st_vec<R>(Yu + (size_t)p * R, y[q]);
-    }
-    if (any) {
-      uint8_t* bu = P.best + (size_t)u * npos;
-      for (int p = p0; p < npos; p += RST_THREADS) bu[p] = (uint8_t)((__ldcg(bu + p) & ~any) | (best[p] & any));
-    }
-    if ((int)threadIdx.x < nlive && ((any >> threadIdx.x) & 1u)) {
-      P.bestF[r0 + threadIdx.x] = s_bestF[threadIdx.x];
-      P.bestT[r0 + threadIdx.x] = s_bestT[threadIdx.x];
-    }
-    if (u == 0 && c == P.chunks - 1 && threadIdx.x == 0) {
-      *P.n_evals = P.n_evals_new;
-      *P.t_last = P.t_last_new;
-    }
-    if (P.chunks == 1) return;
-    __threadfence();
-    __syncthreads();   // every thread's stores before the count that publishes them
-    if (threadIdx.x == 0) red_release_gpu_add(P.sched + 2 + u, 1u);
-  }
-}
 
 // x^0 and y^0 in the unit layout: from the caller ([r][i], values checked as in k_init_state) or from
 // SplitMix64 and ybar; positions and restarts beyond the problem are zero.
@@ -513,32 +114,14 @@ __global__ void __launch_bounds__(256) k_restart_convert(RestartLayout L) {
   }
 }
 
-using RestartKernel = void (*)(RestartParams);
-
-template <int Q, int R, bool PACK>
-RestartKernel kernel_of(bool bf16, bool one) {
-  if (one) return bf16 ? (RestartKernel)k_csr_restart<Q, R, true, true, PACK> : (RestartKernel)k_csr_restart<Q, R, false, true, PACK>;
-  return bf16 ? (RestartKernel)k_csr_restart<Q, R, true, false, PACK> : (RestartKernel)k_csr_restart<Q, R, false, false, PACK>;
-}
-
-// Instantiations: slices per warp up to Q with R restarts, in 64 registers per thread.
-RestartKernel pick_kernel(const CsrRestartShape& sh, int R, bool bf16) {
-  const int q = (sh.slices + RST_WARPS - 1) / RST_WARPS;
-  const bool one = sh.max_groups <= 1;
-  switch (R) {
-    case 1:
-      if (q <= 3) return kernel_of<3, 1, false>(bf16, one);
-      if (q <= 10) return kernel_of<10, 1, false>(bf16, one);
-      return q <= 20 && sh.cp_bf16 ? kernel_of<20, 1, true>(bf16, one) : nullptr;
-    case 2: return q <= 3 ? kernel_of<3, 2, false>(bf16, one) : q <= 10 ? kernel_of<10, 2, false>(bf16, one) : nullptr;
-    case 4: return q <= 5 ? kernel_of<5, 4, false>(bf16, one) : nullptr;
-    default: return nullptr;
-  }
-}
-
 size_t smem_bytes(const CsrRestartShape& sh, int R, bool ent) {
   const size_t npos = (size_t)sh.slices * 32;
-  return 8 * npos * R + 2 * npos + (size_t)sh.slices + 16 + (ent ? ((size_t)sh.groups + RST_SPARE) * 512 : 0);
+  return 8 * (npos + RST_PAD) * R + 2 * npos + RST_PAD + (size_t)sh.slices + 16 +
+         (ent ? ((size_t)sh.groups + RST_SPARE) * (sh.narrow ? 256 : 512) : 0);
+}
+
+RestartKernel pick_kernel(const CsrRestartShape& sh, int R, bool bf16) {
+  return sh.narrow ? pick_narrow(sh, R, bf16) : pick_wide(sh, R, bf16);
 }
 
 }  // namespace
@@ -603,12 +186,19 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
   int maxd = 0;
   for (int64_t i = 0; i < n; ++i) maxd = std::max(maxd, rp[i + 1] - rp[i]);
   if (maxd > CSR_RESTART_MAX_DEG) return false;
-  for (int64_t e = 0; e < rp[n]; ++e) {   // the weight must fit an entry's top 15 bits exactly
-    const float w = (float)val[e];
-    uint32_t bits;
-    std::memcpy(&bits, &w, 4);
-    if ((int64_t)w != val[e] || (bits & ~ENT_W)) return false;
-  }
+  // narrow entries where the weights share one magnitude, else each must fit an entry's top 15 bits
+  auto bits_of = [](float w) {
+    uint32_t b;
+    std::memcpy(&b, &w, 4);
+    return b;
+  };
+  out->shape.narrow = rp[n] > 0;
+  for (int64_t e = 1; e < rp[n] && out->shape.narrow; ++e)
+    out->shape.narrow = val[e] == val[0] || val[e] == -val[0];
+  const bool narrow = out->shape.narrow;
+  out->shape.wbits = narrow ? bits_of((float)val[0]) & 0x7fffffffu : 0u;
+  for (int64_t e = 0; e < rp[n] && !narrow; ++e)
+    if (bits_of((float)val[e]) & ~ENT_W) return false;
   // positions by descending degree, equal degrees in vertex order
   const int slices = (int)((n + 31) / 32);
   const int shift = n > 10 * RST_THREADS ? 2 : 3;   // see k_csr_restart: BASE
@@ -636,7 +226,8 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
     for (int s = w; s < slices; s += RST_WARPS) groups += out->ngroups[(size_t)s];
   }
   out->wstart[RST_WARPS] = groups;
-  out->ent.assign(((size_t)groups + RST_SPARE) * 128, 0u);
+  const size_t words = narrow ? 64 : 128;   // of a group
+  out->ent.assign(((size_t)groups + RST_SPARE) * words, narrow ? (uint32_t)slices * 32u * 0x10001u : 0u);
   for (int w = 0; w < RST_WARPS; ++w) {
     size_t g = out->wstart[(size_t)w];
     for (int s = w; s < slices; s += RST_WARPS) {
@@ -646,14 +237,17 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
         const int64_t i = p < n ? perm[(size_t)p] : -1;
         const int deg = i >= 0 ? rp[i + 1] - rp[i] : 0;
         for (int k = 0; k < 4 * gr; ++k) {
-          uint32_t e = (uint32_t)p << shift;   // padding gathers its own position with weight 0
-          if (k < deg) {
-            const float w32 = (float)val[rp[i] + k];
-            uint32_t bits;
-            std::memcpy(&bits, &w32, 4);
-            e = bits | (uint32_t)pos[(size_t)col[rp[i] + k]] << shift;
+          const size_t at = (g + (size_t)(k / 4)) * words;
+          if (narrow) {   // assign() above filled in the padding
+            if (k >= deg) break;
+            const uint32_t e = (uint32_t)pos[(size_t)col[rp[i] + k]] | (val[rp[i] + k] < 0 ? 0x8000u : 0u);
+            uint32_t& w = out->ent[at + (size_t)l * 2 + (k & 3) / 2];
+            w = (k & 1) ? (w & 0xffffu) | (e << 16) : (w & 0xffff0000u) | e;
+          } else {        // padding gathers its own position with weight 0
+            out->ent[at + (size_t)l * 4 + (k & 3)] =
+                k < deg ? bits_of((float)val[rp[i] + k]) | (uint32_t)pos[(size_t)col[rp[i] + k]] << shift
+                        : (uint32_t)p << shift;
           }
-          out->ent[(g + (size_t)(k / 4)) * 128 + (size_t)l * 4 + (k & 3)] = e;
         }
       }
       g += (size_t)gr;
@@ -667,9 +261,7 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
     out->cpp64[(size_t)p] = cp[out->perm[(size_t)p]];
     const float c = (float)out->cpp64[(size_t)p];
     out->cpp[(size_t)p] = c;
-    uint32_t bits;
-    std::memcpy(&bits, &c, 4);
-    if (bits & 0xffffu) out->shape.cp_bf16 = false;
+    if (bits_of(c) & 0xffffu) out->shape.cp_bf16 = false;
   }
   out->shape.slices = slices;
   out->shape.groups = groups;
@@ -696,14 +288,23 @@ static int chunks_for(int units, int ctas, int iters) {
   return best;
 }
 
-int csr_restart_pick(const CsrRestartShape& sh, int B, int sms) {
+// Restarts per CTA of a run, 0: the row-wise kernels.  Both sides' time per iteration (us) from fits to
+// measurements on GB300 (random graphs, n 300-20,000, mean degree 3-50, B 4-512; within about 20 %):
+//   here, rounds of units on the SMs x a unit's time, which grows with its groups, restarts and slices
+//   (n = 20,000, 4-regular, R = 1: 6.0 us; n = 10,000, degree 6, R = 2: 7.9; n = 4,000, degree 50: 13.6,
+//   20.2 and 35 with R = 1, 2, 4);
+//   row-wise, the kernel boundary, and per 128 restarts the rows and their gathers (n = 10,000, degree
+//   6: 8.6 us with B = 100, 21.5 with B = 512; n = 20,000, degree 16: 22 and 69).
+// The line lies near B = 152, degree 10-20 for n = 20,000 (degree 16, B = 512: 72 here, 69 row-wise).
+int csr_restart_pick(const CsrRestartShape& sh, int64_t n, int64_t nnz, int B, int sms) {
+  const int chunks = (B + 127) / 128;
+  double best_us = 3.4 + (chunks > 1 ? 0.9 * chunks : 1.0) * (0.24e-3 * (double)n + 0.042e-3 * (double)nnz);
   int best = 0;
-  double best_cost = 0.0;
   for (int R : {1, 2, 4}) {
     if (!csr_restart_fits(sh, R)) continue;
-    const int units = (B + R - 1) / R;
-    const double cost = std::max(1.0, (double)units / sms) * (1.0 + R);
-    if (best == 0 || cost < best_cost) { best = R; best_cost = cost; }
+    const double rounds = std::max(1.0, (double)((B + R - 1) / R) / sms);
+    const double us = rounds * (0.35 + 0.003 * sh.slices + sh.groups * (0.0042 + 0.004 * R));
+    if (us < best_us) { best = R; best_us = us; }
   }
   return best;
 }
@@ -717,7 +318,8 @@ cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_
   RestartParams P;
   std::memset(&P, 0, sizeof(P));
   P.a = a;
-  P.ent = reinterpret_cast<const uint4*>(d.ent);
+  P.ent = d.ent;
+  P.wbits = d.shape.wbits;
   P.wstart = d.wstart;
   P.ngroups = d.ngroups;
   P.cpp = d.cpp;

@@ -118,8 +118,8 @@ cudaError_t launch_csr_res(const int32_t* rowptr, const int32_t* col, const void
 int csr_partial_rows(int64_t n, int B);
 // k_csr_restart.cu: whole runs with R restarts of the graph per CTA (state on chip between launches).
 // csr_restart_build lays the structure out (false: the graph does not fit the form: more than 20,480
-// vertices, a row longer than CSR_RESTART_MAX_DEG or a weight of more than 7
-// significant bits); csr_restart_pick
+// vertices, a row longer than CSR_RESTART_MAX_DEG or weights of more than
+// 7 significant bits and more than one magnitude); csr_restart_pick
 // gives the restarts per CTA for a run of B restarts.
 constexpr int CSR_RESTART_MAX_DEG = 256;
 constexpr int CSR_RESTART_MAX_R = 4;   // restarts per CTA: 1, 2 or 4
@@ -128,6 +128,8 @@ struct CsrRestartShape {
   uint32_t groups = 0;
   int max_groups = 0;      // groups of the longest row
   bool cp_bf16 = true;     // every c' is exact in BF16
+  bool narrow = false;     // 16-bit entries: every weight is +-w
+  uint32_t wbits = 0;      // the bits of that w as a float
 };
 struct CsrRestartHost {
   CsrRestartShape shape;
@@ -171,7 +173,7 @@ struct RestartLayout {
 bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
                        CsrRestartHost* out);
 bool csr_restart_fits(const CsrRestartShape& sh, int R);   // an instantiation exists and x fits on chip
-int csr_restart_pick(const CsrRestartShape& sh, int B, int sms);
+int csr_restart_pick(const CsrRestartShape& sh, int64_t n, int64_t nnz, int B, int sms);
 size_t csr_restart_positions(const CsrRestartShape& sh);
 cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_type, const CsrRestartRun& run, int R,
                                int sms, cudaStream_t s);

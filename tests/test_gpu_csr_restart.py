@@ -60,7 +60,7 @@ def _same(n, csr, prec, B, K, T, chunks, resident=True):
 
 @pytest.mark.parametrize("prec", [S.SBO_FP32, S.SBO_BF16, S.SBO_FP8_E4M3])
 @pytest.mark.parametrize("n,deg,B", [(1, 1, 3), (31, 3, 1), (33, 8, 7), (1025, 6, 130), (3073, 5, 9), (5121, 3, 301),
-                                     (10240, 6, 305), (10241, 4, 17), (20480, 5, 3)])
+                                     (10240, 6, 305), (10241, 4, 317), (20480, 5, 160)])
 def test_restart_resident_runs_equal_the_row_wise_ones(n, deg, B, prec):
     # 300 iterations at ybar = 1, beta = 0.025 pass through y = 0, where the perturbation rule acts
     _same(n, _graph(n, deg, n, wmax=3), prec, B, 10, 303, [303])
@@ -76,11 +76,12 @@ def test_evaluation_points_and_split_runs(K, T, chunks):
 def test_degree_and_range_limits_fall_back():
     n = 11000
     star = (np.concatenate([[0], np.full(n, 300)]), np.arange(1, 301), np.ones(300, int), np.zeros(n, int))
-    _same(n, star, S.SBO_FP32, 5, 10, 30, [30], resident=False)             # a row of 300
+    _same(n, star, S.SBO_FP32, 160, 10, 30, [30], resident=False)             # a row of 300
     heavy = _graph(n, 4, 2)
-    _same(n, (heavy[0], heavy[1], heavy[2] * 129, heavy[3]), S.SBO_FP32, 5, 10, 30, [30], resident=False)   # 8 bits
-    _same(n, (heavy[0], heavy[1], heavy[2] * 4064, heavy[3]), S.SBO_FP32, 5, 10, 30, [30])   # 127 * 32: 7 bits
+    mixed = np.where(np.arange(heavy[2].size) % 2 == 0, 1, 129) * heavy[2]
+    _same(n, (heavy[0], heavy[1], mixed, heavy[3]), S.SBO_FP32, 160, 10, 30, [30], resident=False)          # 8 bits
+    _same(n, (heavy[0], heavy[1], heavy[2] * 129, heavy[3]), S.SBO_FP32, 160, 10, 30, [30])     # one magnitude
     _same(700, _graph(700, 6, 2, wmax=127), S.SBO_BF16, 5, 10, 30, [30])
-    _same(n, (*heavy[:3], heavy[3] * 1001), S.SBO_FP32, 5, 10, 30, [30], resident=False)   # c' not exact in BF16
+    _same(n, (*heavy[:3], heavy[3] * 1001), S.SBO_FP32, 160, 10, 30, [30], resident=False)   # c' not exact in BF16
     _same(700, (*_graph(700, 4, 3)[:3], np.full(700, 1001)), S.SBO_FP32, 5, 10, 30, [30])  # small n keeps FP32 c'
-    _same(20481, _graph(20481, 3, 4), S.SBO_FP32, 2, 10, 30, [30], resident=False)
+    _same(20481, _graph(20481, 3, 4), S.SBO_FP32, 160, 10, 30, [30], resident=False)
