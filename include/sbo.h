@@ -50,7 +50,10 @@ typedef enum sbo_status {
 } sbo_status;
 
 typedef enum sbo_precision {
-  SBO_FP32 = 0,       /* A stored FP32, x operand FP32, FP32 accumulation (CUDA cores) */
+  SBO_FP32 = 0,       /* A stored FP32, x operand FP32, FP32 accumulation.  Dense problems with n >= 65
+                         and every |A_ij| <= 256 also keep A in BF16 (exact) and run on the tensor
+                         cores, x as three BF16 pieces (nearer to FP64 than the CUDA cores' FP32
+                         sums); the others run on the CUDA cores */
   SBO_BF16 = 1,       /* A stored BF16 (|A_ij| <= 256), x operand BF16 (RN from the FP32
                          master), FP32 accumulation; dense: tcgen05 tensor cores */
   SBO_FP8_E4M3 = 2    /* sparse only: weights stored E4M3 (|A_ij| <= 16), x operand BF16,
@@ -180,7 +183,8 @@ sbo_status sbo_trace(sbo_problem* p, int64_t* minF, int64_t cap, int64_t* count)
  * gradient).  L_dev (B), GX_dev, GY_dev (B*n) are device float32 outputs; any may be NULL.  A x is recomputed on every
  * call (nothing is cached between calls), with the contraction of the problem's precision.
  * stream: cudaStream_t or NULL; the call is asynchronous on it.  Scratch for the operand is kept
- * by the handle: B*n*2 bytes (dense BF16), or n*round_up(B,8)*4 (CSR FP32) or *2 (CSR BF16 /
+ * by the handle: B*n*2 bytes (dense BF16),
+ * B*n*6 (dense FP32 on the tensor cores), or n*round_up(B,8)*4 (CSR FP32) or *2 (CSR BF16 /
  * E4M3) bytes in the sparse kernels' variable-major layout.  Dense and CSR QUBO problems; not
  * Max-k-Cut. */
 sbo_status sbo_lagrangian(sbo_problem* p, int32_t B, const float* X_dev, const float* Y_dev,
@@ -220,7 +224,8 @@ sbo_status sbo_lagrangian_noalloc(sbo_problem* p, int32_t B, const float* X_dev,
  * SBO_OPT_USE_GRAPH also applies to the next sbo_gda_run of the current run, and SBO_OPT_PDL and
  * SBO_OPT_TIMEOUT_US to its directly launched kernels (replayed graphs keep the values they were
  * captured with until the next start); results depend on none of the three.
- *   SBO_OPT_KERNEL:     0 auto, 1 SIMT FP32 (plain form), 2 tcgen05 (BF16 dense),
+ *   SBO_OPT_KERNEL:     0 auto, 1 SIMT FP32 (plain form), 2 tcgen05 (BF16 dense; sbo_info reports
+ *                       it for FP32 problems on the tensor cores too),
  *                       3 tiny-n single-CTA loop (n <= 64, FP32)
  *   SBO_OPT_USE_GRAPH:  1 (default) replay blocks of K iterations from a CUDA graph; 0 launch
  *                       every kernel directly

@@ -90,6 +90,8 @@ struct sbo_problem {
   void* A = nullptr;
   int64_t lda = 0;
   int a_type = OP_F32;
+  void* A16 = nullptr;         // FP32 problems with every |A_ij| <= 256: A in BF16, for the tensor cores
+  bool tc_split = false;       // this run: FP32 problem on the tensor cores (x in three BF16 pieces)
   // CSR
   int32_t* rowptr = nullptr;
   int32_t* col = nullptr;
@@ -213,6 +215,7 @@ void free_run(sbo_problem* p) {
 void free_all(sbo_problem* p) {
   free_run(p);
   dfree(p->A, p->stream);
+  dfree(p->A16, p->stream);
   dfree(p->rowptr, p->stream);
   dfree(p->col, p->stream);
   dfree(p->val, p->stream);
@@ -266,6 +269,7 @@ EpiArgs base_args(const sbo_problem* p) {
   a.err = p->err;
   a.gkind = p->opt_g;
   a.Gd = p->Gd;
+  if (p->tc_split) a.xpiece = (int64_t)p->B * p->ld;
   if (p->single) {
     a.mu = p->mu;
     a.gpart = p->gpart;
@@ -1032,6 +1036,13 @@ struct CopyLane {
   }
 };
 
+// FP32 problems from this size on run on the tensor cores when A is exact in BF16 (k_tc SPLIT); below it
+// the single-launch kernel (n <= 64) or the CUDA cores do.
+constexpr int64_t SPLIT_MIN_N = 65;
+// ... and the Lagrangian from this size on: its two launches and the tensor maps cost more than the CUDA
+// cores take on smaller problems (n = 300, B = 64: 28.6 against 26.2 us; n = 700, B = 130: 30 against 45).
+constexpr int64_t SPLIT_LAGR_MIN_N = 400;
+
 // Dense set-up shared by the int32 and int8 entry points (q_bytes: size of one entry of Q).
 static sbo_status create_dense_impl(int64_t n, const void* Q, int q_bytes, const int32_t* c, int32_t precision,
                                     void* stream, sbo_problem** out) {
@@ -1066,6 +1077,9 @@ static sbo_status create_dense_impl(int64_t n, const void* Q, int q_bytes, const
   const size_t a_elt = p->a_type == OP_F32 ? 4 : 2;
   configure_pool_once();
   if ((e = cudaMallocAsync(&p->A, (size_t)n * p->lda * a_elt, s)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc A"));
+  if (p->a_type == OP_F32 && n >= SPLIT_MIN_N && tc_supported() &&
+      (e = cudaMallocAsync(&p->A16, (size_t)n * p->lda * 2, s)) != cudaSuccess)
+    return bail(e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation failed") : cuda_fail(e, "cudaMalloc"));
   if ((e = dalloc(&p->cp, n, s)) != cudaSuccess || (e = dalloc(&p->cp64, n, s)) != cudaSuccess ||
       (e = cudaMallocAsync(&Qd, (size_t)n * n * q_bytes, s)) != cudaSuccess || (e = dalloc(&rowsum, n, s)) != cudaSuccess ||
       (e = dalloc(&rerr, 1, s)) != cudaSuccess || (c && (e = dalloc(&cd, n, s)) != cudaSuccess))
@@ -1093,7 +1107,8 @@ static sbo_status create_dense_impl(int64_t n, const void* Q, int q_bytes, const
           return bail(cuda_fail(e, "copy Q"));
         }
       }
-      if ((e = launch_canon_dense(Qd, q_bytes, n, j0, j1, p->A, p->lda, p->a_type, rowsum, rerr, limit, s)) !=
+      if ((e = launch_canon_dense(Qd, q_bytes, n, j0, j1, p->A, p->lda, p->a_type, p->A16, rowsum, rerr, limit,
+                                   s)) !=
           cudaSuccess) {
         lane.drain();
         return bail(cuda_fail(e, "canonicalisation launch"));
@@ -1110,6 +1125,7 @@ static sbo_status create_dense_impl(int64_t n, const void* Q, int q_bytes, const
       (e = cudaStreamSynchronize(s)) != cudaSuccess)
     return bail(cuda_fail(e, "canonicalisation"));
   cleanup_tmp();
+  if (flags & 8u) dfree(p->A16, s);   // not exact in BF16: CUDA cores only
   if (flags & 1u) {
     free_all(p); delete p;
     return fail(SBO_ERANGE, precision == SBO_BF16 ? "|Q_ij + Q_ji| > 256 is not exact in BF16"
@@ -1427,15 +1443,16 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   } else if (p->prec == SBO_BF16) {
     ker = KER_TC;
   } else {
-    ker = p->n <= 64 && p->opt_dual == 0 ? KER_TINY : KER_SIMT;
+    ker = p->n <= 64 && p->opt_dual == 0 ? KER_TINY : p->A16 ? KER_TC : KER_SIMT;
   }
   if (ker == KER_TC && !tc_supported()) return fail(SBO_ECUDA, "tcgen05 path needs a compute capability 10.3 device");
   free_run(p);
   p->prm = *prm;
+  p->tc_split = ker == KER_TC && p->prec == SBO_FP32;
   p->kernel = ker;
   p->B = prm->restarts;
   p->layout = (ker == KER_CSR || ker == KER_MAXK) ? LAYOUT_NR : LAYOUT_RN;
-  p->op_type = (p->prec == SBO_FP32) ? OP_F32 : OP_BF16;
+  p->op_type = p->prec == SBO_FP32 && !p->tc_split ? OP_F32 : OP_BF16;
   p->ld = p->layout == LAYOUT_RN ? round_up(p->n, 8) : round_up(p->B, 8);
   p->t = 0;
   p->t_last_eval = 0;
@@ -1445,6 +1462,7 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   const int64_t rows = p->layout == LAYOUT_RN ? p->B : p->n;
   const size_t elems = (size_t)rows * p->ld;
   const size_t op_elt = p->op_type == OP_F32 ? 4 : 2;
+  const size_t pieces = p->tc_split ? 3 : 1;   // of the operand
   cudaError_t e = cudaSuccess;
   const bool need_master = ker == KER_TINY || ker == KER_MAXK || p->op_type != OP_F32;
   const size_t xelems = elems * (ker == KER_MAXK ? (size_t)p->kparts : 1);   // Max-k-Cut: k logits
@@ -1467,8 +1485,8 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
     al((void**)&p->Y, elems * 4);
     if (p->opt_keep_grad) al((void**)&p->Gd, elems * 4);
     if (ker != KER_TINY) {
-      al(&p->Xop[0], xelems * op_elt);
-      al(&p->Xop[1], xelems * op_elt);
+      al(&p->Xop[0], xelems * op_elt * pieces);
+      al(&p->Xop[1], xelems * op_elt * pieces);
       al(&p->bits, elems * (ker == KER_CSR ? 1 : op_elt));   // the sparse path keeps candidates as bytes
     }
     al((void**)&p->bestBits, elems);
@@ -1503,7 +1521,7 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   if (p->Y) cudaMemsetAsync(p->Y, 0, elems * 4, s);
   if (p->Gd) cudaMemsetAsync(p->Gd, 0, elems * 4, s);
   for (void* b : {p->Xop[0], p->Xop[1]})
-    if (b) cudaMemsetAsync(b, 0, xelems * op_elt, s);
+    if (b) cudaMemsetAsync(b, 0, xelems * op_elt * pieces, s);
   if (p->bits) cudaMemsetAsync(p->bits, 0, elems * (ker == KER_CSR ? 1 : op_elt), s);
   launch_fill_i64(p->bestF, p->B, LLONG_MAX, s);
   launch_fill_i64(p->bestT, p->B, -1, s);
@@ -1533,7 +1551,7 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
     }
     // the cluster split-K kernel serves problems with at most sms / 2 tiles (fewest at width 256),
     // on CTA pairs at most sms / 4 tiles of 256 x 256
-    if ((p->opt_tile_n == 0 || p->opt_tile_n >= 1000) &&
+    if ((p->tc_split || p->opt_tile_n == 0 || p->opt_tile_n >= 1000) &&
         ((int64_t)((p->n + 127) / 128) * ((p->B + 255) / 256) * 2 <= p->sms ||
          (int64_t)((p->n + 255) / 256) * ((p->B + 255) / 256) * 4 <= p->sms) &&
         (e = dalloc(&p->csk_ws, (size_t)p->sms * 256 * 128, s)) != cudaSuccess) {
@@ -1541,7 +1559,7 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
       return e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation of the cluster workspace failed")
                                             : cuda_fail(e, "cudaMalloc");
     }
-    int tn = p->opt_tile_n;
+    int tn = p->tc_split ? 1064 : p->opt_tile_n;   // (1064 falls back to 64 where it does not apply)
     std::string why;
     if (tn == 0 && p->opt_autotune) {
       sbo_status st2 = tune_tile(p, &tn);   // runs on the zeroed state, before x^0 is written
@@ -1552,8 +1570,11 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
     const int tuned_csk = tn / 10000;   // cluster size decided by the autotuner (0: none)
     tn %= 10000;
     if (tn == 512 && !tc_pair_supported(nullptr)) tn = 256;
-    e = tc_make_plan(&p->plan, p->A, p->lda, (int)p->n, p->Xop[0], p->Xop[1], p->bits, p->ld, p->B,
-                     tile_width(tn), &why);
+    e = tc_make_plan(&p->plan, p->tc_split ? p->A16 : p->A, p->lda, (int)p->n, p->Xop[0], p->Xop[1], p->bits, p->ld,
+                     p->B, tile_width(tn), &why);
+    for (int k = 0; k < 2 && e == cudaSuccess && p->tc_split; ++k)   // three pieces of every restart
+      e = tc_make_operand_map(&p->plan.mapX[k], p->Xop[k], p->ld, (int)p->n, 3 * p->B, 64, &why);
+    if (e == cudaSuccess) p->plan.split = p->tc_split;
     if (e != cudaSuccess) { free_run(p); return fail(SBO_ECUDA, "tensor-core plan: " + why); }
     p->plan.pair = tn == 512;
     p->plan.csk = 0;
@@ -1632,8 +1653,12 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
                          static_cast<float*>(p->Xop[0]), s);
   else
     e = launch_init_state((int)p->n, p->B, p->ld, p->layout, prm->seed, (float)prm->ybar, x0d, y0d, p->Xm,
-                          ker == KER_TINY ? (void*)p->Xm : p->Xop[0], ker == KER_TINY ? OP_F32 : p->op_type, p->Y,
-                          p->err, s);
+                          ker == KER_TINY || p->tc_split ? (void*)p->Xm : p->Xop[0],
+                          ker == KER_TINY || p->tc_split ? OP_F32 : p->op_type, p->Y, p->err, s);
+  if (p->tc_split && e == cudaSuccess) {
+    e = launch_to_pieces(p->Xm, (int)p->n, p->B, p->ld, p->Xop[0], p->ld, true, s);
+    ++p->launches;
+  }
   ++p->launches;
   if (x0d || y0d) { cudaStreamSynchronize(s); dfree(x0d, s); dfree(y0d, s); }
   if (e != cudaSuccess) { free_run(p); return cuda_fail(e, "init launch"); }
@@ -1730,7 +1755,8 @@ sbo_status sbo_eval(sbo_problem* p, int64_t count, const uint8_t* bits, int64_t*
     if (bits[k] > vmax) return fail(SBO_EINVAL, p->fmt == FMT_MAXK ? "parts must be < k" : "bits must be 0 or 1");
   cudaStream_t s = p->stream;
   const int layout = p->fmt == FMT_DENSE ? LAYOUT_RN : LAYOUT_NR;
-  const int op = p->fmt == FMT_CSR ? OP_U8 : p->prec == SBO_FP32 ? OP_F32 : OP_BF16;
+  const bool simt = p->fmt == FMT_DENSE && p->prec == SBO_FP32 && !p->A16;
+  const int op = p->fmt == FMT_CSR ? OP_U8 : simt || p->fmt == FMT_MAXK ? OP_F32 : OP_BF16;
   const int64_t ld = layout == LAYOUT_RN ? round_up(p->n, 8) : round_up(count, 8);
   const int64_t rows = layout == LAYOUT_RN ? count : p->n;
   uint8_t* bd = nullptr;
@@ -1768,13 +1794,13 @@ sbo_status sbo_eval(sbo_problem* p, int64_t count, const uint8_t* bits, int64_t*
       e = launch_maxk(p->rowptr, p->col, static_cast<const float*>(p->val), a, p->kparts, EPI_EVAL, s);
     } else if (p->fmt == FMT_CSR) {
       e = launch_csr(p->rowptr, p->col, p->val, p->val_type, a, op, EPI_EVAL, false, s);
-    } else if (p->prec == SBO_FP32) {
+    } else if (simt) {
       e = launch_simt(static_cast<const float*>(p->A), p->lda, a, EPI_EVAL, s);
     } else {
       TcPlan plan{};
       std::string why;
       const int tn = 64;
-      e = tc_make_plan(&plan, p->A, p->lda, (int)p->n, opd, nullptr, nullptr, ld, (int)count, tn, &why);
+      e = tc_make_plan(&plan, p->A16 ? p->A16 : p->A, p->lda, (int)p->n, opd, nullptr, nullptr, ld, (int)count, tn, &why);
       if (e != cudaSuccess) { cleanup(); return fail(SBO_ECUDA, "tensor-core plan: " + why); }
       e = launch_tc(plan, 0, nullptr, a, EPI_EVAL, timeout_ns(p), s);
     }
@@ -1952,26 +1978,32 @@ sbo_status sbo_lagrangian(sbo_problem* p, int32_t B, const float* X_dev, const f
     a.ld = ldx;
     e = launch_csr(p->rowptr, p->col, p->val, p->val_type, a, op, EPI_LAGR, false, s);
     p->launches += 2;
-  } else if (p->prec == SBO_FP32) {
+  } else if (p->prec == SBO_FP32 && (!p->A16 || p->n < SPLIT_LAGR_MIN_N)) {
     a.Xin = X_dev;
     e = launch_simt(static_cast<const float*>(p->A), p->lda, a, EPI_LAGR, s);
     ++p->launches;
   } else {
+    const bool split = p->prec == SBO_FP32;   // x in three BF16 pieces
     const int64_t ldx = round_up(p->n, 8);
-    const size_t need = (size_t)B * ldx * 2;
+    const size_t need = (size_t)B * ldx * (split ? 6 : 2);
     if (need > p->lag_cap) {
       if (p->lag_op) { cudaStreamSynchronize(s); cudaFree(p->lag_op); p->lag_op = nullptr; p->lag_cap = 0; }
       SBO_CUDA(cudaMalloc(&p->lag_op, need));   // used on the caller's stream: not stream-ordered
       SBO_CUDA(cudaMemsetAsync(p->lag_op, 0, need, s));
       p->lag_cap = need;
     }
-    e = launch_to_operand(X_dev, (int)p->n, B, p->n, p->lag_op, ldx, OP_BF16, s);
+    e = split ? launch_to_pieces(X_dev, (int)p->n, B, p->n, p->lag_op, ldx, false, s)
+              : launch_to_operand(X_dev, (int)p->n, B, p->n, p->lag_op, ldx, OP_BF16, s);
     if (e != cudaSuccess) return cuda_fail(e, "operand conversion");
     TcPlan plan{};
     std::string why;
-    int tn = 256;
+    int tn = split ? 64 : 256;
     while (tn > 64 && (int64_t)((p->n + 127) / 128) * ((B + tn - 1) / tn) < p->sms) tn /= 2;
-    e = tc_make_plan(&plan, p->A, p->lda, (int)p->n, p->lag_op, nullptr, nullptr, ldx, B, tn, &why);
+    e = tc_make_plan(&plan, split ? p->A16 : p->A, p->lda, (int)p->n, p->lag_op, nullptr, nullptr, ldx, B, tn, &why);
+    if (e == cudaSuccess && split) {
+      e = tc_make_operand_map(&plan.mapX[0], p->lag_op, ldx, (int)p->n, 3 * B, 64, &why);
+      plan.split = true;
+    }
     if (e != cudaSuccess) return fail(SBO_ECUDA, "tensor-core plan: " + why);
     e = launch_tc(plan, 0, nullptr, a, EPI_LAGR, timeout_ns(p), s);
     p->launches += 2;

@@ -38,6 +38,7 @@ struct EpiArgs {
   float* Y;                // y, updated in place
   const void* Xin;         // contraction operand x^t (FP32 or BF16), read by every tile
   void* Xout;              // operand x^{t+1} (ping-pong partner of Xin)
+  int64_t xpiece;          // elements between the three BF16 pieces of Xout (FP32 problems on tensor cores, split3)
   void* bits_out;          // if non-null: b = [x^{t+1} > 1/2] in the operand type (bytes for the sparse kernel)
   unsigned long long* F2;  // EPI_EVAL: 2F(b) accumulators per restart (two's complement)
   const float* Xl;         // EPI_LAGR: x (FP32)
@@ -104,6 +105,34 @@ __device__ __forceinline__ void op_store(void* p, int64_t idx, float v, int type
   if (type == OP_F32) static_cast<float*>(p)[idx] = v;
   else if (type == OP_U8) static_cast<uint8_t*>(p)[idx] = (uint8_t)v;
   else static_cast<__nv_bfloat16*>(p)[idx] = __float2bfloat16_rn(v);
+}
+
+// x as the sum of three BF16 values, for FP32 problems on the tensor cores.  The pieces lie on fixed grids
+// below the scale s = 2^e >= |x| of the restart (inv = 1 / s; s = 1 for iterates in the box): h a multiple
+// of 2^-8 s, m of 2^-16 s (both exact in BF16), l the rest in 8 bits (off by at most 2^-26 s, nothing for
+// |x| >= s / 4).  Sums of integer weights times h / s (or m / s) are then exact in an FP32 accumulator up
+// to 2^16 (2^7) in magnitude, whatever its rounding.  Infinities and NaN stay in h; values above the
+// scale (beyond 2^126) are cut into the three bytes of their mantissa.
+__device__ __forceinline__ void split3(float x, float s, float inv, __nv_bfloat16* h, __nv_bfloat16* m,
+                                       __nv_bfloat16* l) {
+  float a, b, c;
+  if (fabsf(x) <= s) {
+    a = rintf(x * inv * 256.0f) * (s * (1.0f / 256.0f));
+    const float r = x - a;                                   // exact
+    b = rintf(r * inv * 65536.0f) * (s * (1.0f / 65536.0f));
+    c = r - b;                                               // exact
+  } else if (fabsf(x) <= 3.4028234e38f) {
+    a = __uint_as_float(__float_as_uint(x) & 0xffff0000u);
+    const float r = x - a;
+    b = __uint_as_float(__float_as_uint(r) & 0xffff0000u);
+    c = r - b;
+  } else {
+    a = x;
+    b = c = 0.0f;
+  }
+  *h = __float2bfloat16_rn(a);
+  *m = __float2bfloat16_rn(b);
+  *l = __float2bfloat16_rn(c);
 }
 
 // One coordinate of Algorithm 1.  d is dL/dx at (x, y) and gx = g(x); returns x^{t+1}, writes

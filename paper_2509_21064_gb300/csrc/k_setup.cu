@@ -18,8 +18,9 @@ __device__ __forceinline__ int64_t tri(int64_t J) { return J * (J + 1) / 2; }   
 
 template <typename TQ>   // int32_t or int8_t entries of Q
 __global__ void __launch_bounds__(256) k_canon_dense(const TQ* __restrict__ Q, int64_t n, int64_t j0, void* A,
-                                                     int64_t lda, int a_type, unsigned long long* rowsum,
-                                                     uint32_t* range_err, int64_t a_limit) {
+                                                     int64_t lda, int a_type, __nv_bfloat16* A16,
+                                                     unsigned long long* rowsum, uint32_t* range_err,
+                                                     int64_t a_limit) {
   __shared__ int32_t s1[CANON_T][CANON_T + 1];   // Q(I, J)
   __shared__ int32_t s2[CANON_T][CANON_T + 1];   // Q(J, I)
   // pair index -> (I, J): q = tri(J) + I with 0 <= I <= J
@@ -44,7 +45,7 @@ __global__ void __launch_bounds__(256) k_canon_dense(const TQ* __restrict__ Q, i
     }
   }
   __syncthreads();
-  bool over = false;
+  bool over = false, over16 = false;
   // A(I, J)[r][q] = s1[r][q] + s2[q][r];  A(J, I)[r][q] = s2[r][q] + s1[q][r]
 #pragma unroll 2
   for (int e = tid; e < CANON_T * CANON_T / 4; e += 256) {
@@ -60,6 +61,15 @@ __global__ void __launch_bounds__(256) k_canon_dense(const TQ* __restrict__ Q, i
         v[u] = side ? (int64_t)s2[r][q + u] + s1[q + u][r] : (int64_t)s1[r][q + u] + s2[q + u][r];
         if (gi == gj0 + u) v[u] = 0;
         over |= (v[u] < 0 ? -v[u] : v[u]) > a_limit;
+        over16 |= (v[u] < 0 ? -v[u] : v[u]) > 256;
+      }
+      if (A16) {   // an FP32 problem's copy for the tensor cores
+        __nv_bfloat162 lo = __floats2bfloat162_rn((float)v[0], (float)v[1]);
+        __nv_bfloat162 hi = __floats2bfloat162_rn((float)v[2], (float)v[3]);
+        uint2 raw;
+        raw.x = *reinterpret_cast<uint32_t*>(&lo);
+        raw.y = *reinterpret_cast<uint32_t*>(&hi);
+        *reinterpret_cast<uint2*>(A16 + gi * lda + gj0) = raw;
       }
       if (a_type == OP_F32) {
         *reinterpret_cast<float4*>(static_cast<float*>(A) + gi * lda + gj0) =
@@ -75,6 +85,7 @@ __global__ void __launch_bounds__(256) k_canon_dense(const TQ* __restrict__ Q, i
     }
   }
   if (over) atomicOr(range_err, 1u);
+  if (A16 && over16) atomicOr(range_err, 8u);   // the copy is not exact
   // row sums: threads 0..63 the rows of A(I, J), threads 64..127 the rows of A(J, I)
   if (tid < 2 * CANON_T && !(tid >= CANON_T && I == J)) {
     const bool side = tid >= CANON_T;
@@ -113,19 +124,19 @@ __global__ void k_rowsum_check(const unsigned long long* rowsum, const int64_t* 
 }
 
 cudaError_t launch_canon_dense(const void* Qd, int q_bytes, int64_t n, int64_t j0, int64_t j1, void* A, int64_t lda,
-                               int a_type, unsigned long long* rowsum, uint32_t* range_err, int64_t a_limit,
-                               cudaStream_t s) {
+                               int a_type, void* A16, unsigned long long* rowsum, uint32_t* range_err,
+                               int64_t a_limit, cudaStream_t s) {
   if (lda % 4 != 0 || lda < n || j0 < 0 || j1 < j0) return cudaErrorInvalidValue;   // 4-entry stores along rows
   const int64_t pairs = j1 * (j1 + 1) / 2 - j0 * (j0 + 1) / 2;
   if (pairs == 0) return cudaSuccess;
   if (pairs > 0x7fffffffLL) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)pairs), block(256);
   if (q_bytes == 1)
-    k_canon_dense<int8_t><<<grid, block, 0, s>>>(static_cast<const int8_t*>(Qd), n, j0, A, lda, a_type, rowsum,
-                                                 range_err, a_limit);
+    k_canon_dense<int8_t><<<grid, block, 0, s>>>(static_cast<const int8_t*>(Qd), n, j0, A, lda, a_type,
+                                                 static_cast<__nv_bfloat16*>(A16), rowsum, range_err, a_limit);
   else
-    k_canon_dense<int32_t><<<grid, block, 0, s>>>(static_cast<const int32_t*>(Qd), n, j0, A, lda, a_type, rowsum,
-                                                  range_err, a_limit);
+    k_canon_dense<int32_t><<<grid, block, 0, s>>>(static_cast<const int32_t*>(Qd), n, j0, A, lda, a_type,
+                                                  static_cast<__nv_bfloat16*>(A16), rowsum, range_err, a_limit);
   return cudaGetLastError();
 }
 
@@ -194,6 +205,46 @@ cudaError_t launch_to_operand(const float* X, int n, int B, int64_t ld_in, void*
   const int64_t blocks = (total + 255) / 256;
   k_to_operand<<<(unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), 256, 0, s>>>(X, n, B, ld_in, out, ld_out,
                                                                                  op_type);
+  return cudaGetLastError();
+}
+
+// FP32 [B][n] (ld_in) -> the three BF16 pieces of split3, [piece][B][ld_out]; one block per restart at a
+// time.  unit: x lies in the box, scale 1; else the power of two above the restart's largest magnitude.
+__global__ void __launch_bounds__(256) k_to_pieces(const float* __restrict__ X, int n, int B, int64_t ld_in,
+                                                   __nv_bfloat16* out, int64_t ld_out, bool unit) {
+  __shared__ float wmax[8];
+  const int64_t piece = (int64_t)B * ld_out;
+  for (int r = blockIdx.x; r < B; r += gridDim.x) {
+    const float* x = X + r * ld_in;
+    float s = 1.0f, inv = 1.0f;
+    if (!unit) {
+      float m = 0.0f;
+      for (int i = threadIdx.x; i < n; i += 256) {
+        const float v = fabsf(x[i]);
+        if (v <= 3.4028234e38f) m = fmaxf(m, v);   // finite values only
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < 8; ++w) m = fmaxf(m, wmax[w]);
+      __syncthreads();
+      const int e = min(max(m > 0.0f ? ilogbf(m) + 1 : 0, -100), 100);
+      s = ldexpf(1.0f, e);
+      inv = ldexpf(1.0f, -e);
+    }
+    for (int i = threadIdx.x; i < n; i += 256) {
+      __nv_bfloat16* o = out + r * ld_out + i;
+      split3(x[i], s, inv, o, o + piece, o + 2 * piece);
+    }
+  }
+}
+
+cudaError_t launch_to_pieces(const float* X, int n, int B, int64_t ld_in, void* out, int64_t ld_out, bool unit,
+                             cudaStream_t s) {
+  k_to_pieces<<<(unsigned)(B < 152 * 8 ? B : 152 * 8), 256, 0, s>>>(X, n, B, ld_in, static_cast<__nv_bfloat16*>(out),
+                                                                    ld_out, unit);
   return cudaGetLastError();
 }
 

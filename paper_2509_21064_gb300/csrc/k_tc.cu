@@ -17,6 +17,12 @@
 // TMEM holds two accumulators (2 x tile_n columns) so the epilogue of one tile overlaps the
 // main loop of the next.  Tiles are visited m-major with the restart tiles of one row block
 // adjacent, so CTAs that share an A row block run together and A is read from HBM ~once.
+// SPLIT (FP32 problems whose A is exact in BF16): x comes as three BF16 pieces (split3), stacked
+// [piece][restart] in the operand, and the tile's B operand is the 3 x 64 rows of its 64 restarts, so
+// one N = 192 instruction per 16 of K forms the three products in columns of their own; the epilogue
+// adds them smallest first.  With the pieces on fixed grids each column sum is exact for the sums that
+// occur, so the result carries one or two FP32 roundings where the FP32 CUDA-core form carries one per
+// term.  It costs 3 of the tensor core's BF16 multiplications per FP32 one.
 // Every mbarrier wait is bounded by a globaltimer budget: on expiry the kernel raises
 // ERR_TIMEOUT, drains its own copies and MMAs (bounded too), frees TMEM and returns.
 #include <cudaTypedefs.h>
@@ -48,17 +54,18 @@ struct TcParams {
   int epi_variant;  // index into TcInst::epi for this launch
 };
 
-template <int BN>
+template <int BN, bool SPLIT = false>
 struct TcCfg {
+  static constexpr int BR = SPLIT ? 3 * BN : BN;   // operand rows per tile = accumulator columns
   static constexpr int A_BYTES = TC_BM * TC_BK * 2;
-  static constexpr int B_BYTES = BN * TC_BK * 2;
+  static constexpr int B_BYTES = BR * TC_BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = (TC_SMEM_BUDGET - 2048) / STAGE_BYTES > 8 ? 8 : (TC_SMEM_BUDGET - 2048) / STAGE_BYTES;
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 /* align */ + 1024 /* barriers */;
-  static constexpr int TMEM_COLS = 2 * BN;
+  static constexpr int TMEM_COLS = SPLIT ? 512 : 2 * BN;   // a power of two >= 2 BR
   // instruction descriptor: D=F32 (bit 4), A=BF16 (bits 7-9), B=BF16 (bits 10-12),
   // both K-major (bits 15, 16 clear), N>>3 at bit 17, M>>4 at bit 24
-  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BR >> 3) << 17) |
                                     ((uint32_t)(TC_BM >> 4) << 24);
 };
 
@@ -105,9 +112,9 @@ __device__ __forceinline__ bool tc_work(const TcParams& P, int j, TcWork& w) {
   return false;
 }
 
-template <int BN, int MODE, bool GROUPED>
+template <int BN, int MODE, bool GROUPED, bool SPLIT = false>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_tc(const __grid_constant__ TcParams P) {
-  using C = TcCfg<BN>;
+  using C = TcCfg<BN, SPLIT>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte aligned tile area (SWIZZLE_128B atoms), barriers after it
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -174,7 +181,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc(const __grid_constant__ Tc
           mbar_expect_tx(fb, (uint32_t)C::STAGE_BYTES);
           uint8_t* sa = tiles + stage * C::STAGE_BYTES;
           tma_load_2d(smem_u32(sa), mapA, fb, kb * TC_BK, m_tile * TC_BM);
-          tma_load_2d(smem_u32(sa + C::A_BYTES), mapX, fb, kb * TC_BK, n_tile * BN);
+          // (a piece's last tile may run into the next piece's rows: columns beyond B, never used)
+#pragma unroll
+          for (int q = 0; q < C::BR / BN; ++q)
+            tma_load_2d(smem_u32(sa + C::A_BYTES + q * BN * TC_BK * 2), mapX, fb, kb * TC_BK,
+                        (SPLIT ? q * P.epi.B : 0) + n_tile * BN);
           issued_mask |= 1u << stage;
           issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
           if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
@@ -202,7 +213,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc(const __grid_constant__ Tc
       for (int j = 0; ok && tc_work<GROUPED>(P, j, w); ++j) {
         if (!mbar_wait(smem_u32(&tempty_bar[acc]), acc_phase ^ 1u, deadline, vabort)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * C::BR);
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
           if (!mbar_wait(smem_u32(&full_bar[stage]), phase, deadline, vabort)) { ok = false; break; }
           tc_fence_after();
@@ -270,8 +281,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc(const __grid_constant__ Tc
             tc_fence_after();
             waited = true;
           }
-          tmem_ld32(tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)(acc * BN + c0), g);
-          epi_apply<MODE>(a, i, row_ok, cpi, cp2, rbase, lane, g, u, v, m_tile * 4 + wq);
+          tc_chunk<BN, SPLIT>(tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)(acc * C::BR + c0), g);
+          epi_apply<MODE, SPLIT>(a, i, row_ok, cpi, cp2, rbase, lane, g, u, v, m_tile * 4 + wq);
         }
       } else {
         ok = mbar_wait_warp(smem_u32(&tfull_bar[acc]), acc_phase, deadline, vabort, lane);
@@ -279,7 +290,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc(const __grid_constant__ Tc
           tc_fence_after();
           float* part = P.ws + (size_t)w.unit * BN * TC_BM;  // [column][row]
           for (int c0 = wg * HALF; c0 < (wg + 1) * HALF; c0 += 32) {
-            tmem_ld32(tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)(acc * BN + c0), g);
+            tc_chunk<BN, SPLIT>(tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)(acc * C::BR + c0), g);
 #pragma unroll
             for (int j = 0; j < 32; ++j) __stcg(part + (size_t)(c0 + j) * TC_BM + row, g[j]);
           }
@@ -320,7 +331,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc(const __grid_constant__ Tc
 #pragma unroll
               for (int j = 0; j < 32; ++j) g[j] += __ldcg(ps + (size_t)(c0 + j) * TC_BM + row);
             }
-            epi_apply<MODE>(a, i, row_ok, cpi, cp2, rbase, lane, g, u, v, m_tile * 4 + wq);
+            epi_apply<MODE, SPLIT>(a, i, row_ok, cpi, cp2, rbase, lane, g, u, v, m_tile * 4 + wq);
           }
         }
       }
@@ -429,6 +440,7 @@ cudaError_t tc_make_plan(TcPlan* plan, const void* A, int64_t lda, int n, const 
   plan->max_splits = 0;
   plan->pair = false;
   plan->csk = 0;
+  plan->split = false;
   const cudaError_t attr_err = ensure_attrs();
   if (attr_err != cudaSuccess) {
     if (why) *why = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(attr_err);
@@ -496,6 +508,13 @@ cudaError_t launch_tc(const TcPlan& plan, int which_x, const CUtensorMap* map_ov
   P.ws = plan.ws;
   P.counters = plan.counters;
   const int grid = sch.grid;
+  if (plan.split && mode != EPI_EVAL) {   // (candidates are 0 and 1: one piece)
+    constexpr int SM = TcCfg<64, true>::SMEM;
+    if (plan.tile_n != 64) return cudaErrorInvalidValue;
+    if (mode == EPI_UPDATE) k_tc<64, EPI_UPDATE, false, true><<<grid, TC_THREADS, SM, s>>>(P);
+    else k_tc<64, EPI_LAGR, false, true><<<grid, TC_THREADS, SM, s>>>(P);
+    return cudaGetLastError();
+  }
   switch (plan.tile_n) {
     case 64: return launch_tc_bn<64>(P, grid, mode, s);
     case 128: return launch_tc_bn<128>(P, grid, mode, s);
@@ -516,6 +535,9 @@ static cudaError_t ensure_attrs() {
     r = r == cudaSuccess ? set_attr<256, EPI_UPDATE>() : r;
     r = r == cudaSuccess ? set_attr<256, EPI_EVAL>() : r;
     r = r == cudaSuccess ? set_attr<256, EPI_LAGR>() : r;
+    for (auto k : {k_tc<64, EPI_UPDATE, false, true>, k_tc<64, EPI_LAGR, false, true>})
+      if (r == cudaSuccess)
+        r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<64, true>::SMEM);
     return r;
   });
 }

@@ -50,17 +50,20 @@ constexpr int CSK_MIN_KB = 4;      // k-blocks per CTA at least
 
 // BN restarts per tile.  PAIR: the tile is 256 rows x BN restarts on a CTA pair (cta_group::2):
 // each CTA stages its own 128 rows of A and BN / 2 restarts of x per k-block.
-template <int BN, bool PAIR>
+// SPLIT (FP32 problems, not paired): the operand is the 3 BN rows of the restarts' BF16 pieces, accumulated
+// in columns of their own and added before the partial tile goes out (see k_tc.cu).
+template <int BN, bool PAIR, bool SPLIT = false>
 struct CskCfg {
   static constexpr int H = PAIR ? 2 : 1;                  // CTAs per split
+  static constexpr int BR = SPLIT ? 3 * BN : BN;          // accumulator columns
   static constexpr int A_BYTES = TC_BM * TC_BK * 2;
-  static constexpr int B_BYTES = (BN / H) * TC_BK * 2;
+  static constexpr int B_BYTES = (BR / H) * TC_BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES =
       (CSK_SMEM_BUDGET - 2048) / STAGE_BYTES > 8 ? 8 : (CSK_SMEM_BUDGET - 2048) / STAGE_BYTES;
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 /* align */ + 1024 /* barriers */;
-  static constexpr int TMEM_COLS = BN;
-  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+  static constexpr int TMEM_COLS = SPLIT ? 256 : BN;
+  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BR >> 3) << 17) |
                                     ((uint32_t)((TC_BM * H) >> 4) << 24);
   static_assert(STAGES * STAGE_BYTES >= BN * TC_BM * 4, "the partial tile must fit in the stage buffers");
 };
@@ -111,7 +114,7 @@ constexpr int CSK_CB = 4;   // restart columns per warp whose loads are in fligh
 // The S partials of a column are summed in split order.  The state rows are padded to a multiple
 // of 8 elements, so the 16-byte loads at i0 < n stay inside the row; stores of the last, partial
 // group of four rows go element by element.
-template <int BN, int MODE, int GK, bool SINGLE>
+template <int BN, int MODE, int GK, bool SINGLE, bool SPLIT>
 __device__ __forceinline__ void csk_columns(const EpiArgs& a, void* xout, void* bits, const float* part,
                                             const float* ws_tile, int64_t split_stride, int s, int S, int row_block,
                                             int64_t r0, int c_begin, int c_end, int warp, int lane) {
@@ -220,8 +223,17 @@ __device__ __forceinline__ void csk_columns(const EpiArgs& a, void* xout, void* 
           if (a.Gd) *reinterpret_cast<float4*>(a.Gd + idx) = make_float4(dd[0], dd[1], dd[2], dd[3]);
           *reinterpret_cast<float4*>(a.Xm + idx) = make_float4(xn[0], xn[1], xn[2], xn[3]);
           if (!SINGLE) *reinterpret_cast<float4*>(a.Y + idx) = make_float4(yn[0], yn[1], yn[2], yn[3]);
-          *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(xout) + idx) =
-              make_uint2(pack_bf16x2(xn[0], xn[1]), pack_bf16x2(xn[2], xn[3]));
+          __nv_bfloat16* xo = static_cast<__nv_bfloat16*>(xout) + idx;
+          if (SPLIT) {
+            __align__(8) __nv_bfloat16 h[4], m[4], l[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) split3(xn[k], 1.0f, 1.0f, &h[k], &m[k], &l[k]);
+            *reinterpret_cast<uint2*>(xo) = *reinterpret_cast<const uint2*>(h);
+            *reinterpret_cast<uint2*>(xo + a.xpiece) = *reinterpret_cast<const uint2*>(m);
+            *reinterpret_cast<uint2*>(xo + 2 * a.xpiece) = *reinterpret_cast<const uint2*>(l);
+          } else {
+            *reinterpret_cast<uint2*>(xo) = make_uint2(pack_bf16x2(xn[0], xn[1]), pack_bf16x2(xn[2], xn[3]));
+          }
           if (bits) {
             float b[4];
 #pragma unroll
@@ -236,7 +248,9 @@ __device__ __forceinline__ void csk_columns(const EpiArgs& a, void* xout, void* 
               if (a.Gd) a.Gd[idx + k] = dd[k];
               a.Xm[idx + k] = xn[k];
               if (!SINGLE) a.Y[idx + k] = yn[k];
-              static_cast<__nv_bfloat16*>(xout)[idx + k] = __float2bfloat16_rn(xn[k]);
+              __nv_bfloat16* xo = static_cast<__nv_bfloat16*>(xout) + idx + k;
+              if (SPLIT) split3(xn[k], 1.0f, 1.0f, xo, xo + a.xpiece, xo + 2 * a.xpiece);
+              else *xo = __float2bfloat16_rn(xn[k]);
               if (bits) static_cast<__nv_bfloat16*>(bits)[idx + k] = __float2bfloat16_rn(xn[k] > 0.5f ? 1.0f : 0.0f);
             }
           }
@@ -252,12 +266,12 @@ __device__ __forceinline__ void csk_columns(const EpiArgs& a, void* xout, void* 
   }
 }
 
-template <int BN, int MODE>
+template <int BN, int MODE, bool SPLIT>
 __device__ __forceinline__ void csk_epilogue(const EpiArgs& a, void* xout, void* bits, const float* part,
                                              const float* ws_tile, int64_t split_stride, int s, int S, int row_block,
                                              int64_t r0, int c_begin, int c_end, int warp, int lane) {
 #define CSK_COLUMNS(M, G, SG)                                                                                    \
-  csk_columns<BN, M, G, SG>(a, xout, bits, part, ws_tile, split_stride, s, S, row_block, r0, c_begin, c_end, warp, \
+  csk_columns<BN, M, G, SG, SPLIT>(a, xout, bits, part, ws_tile, split_stride, s, S, row_block, r0, c_begin, c_end, warp, \
                             lane)
   if (MODE == EPI_EVAL) {
     CSK_COLUMNS(EPI_EVAL, G_QUAD, false);
@@ -271,9 +285,9 @@ __device__ __forceinline__ void csk_epilogue(const EpiArgs& a, void* xout, void*
 #undef CSK_COLUMNS
 }
 
-template <int BN, int MODE, bool PAIR>
+template <int BN, int MODE, bool PAIR, bool SPLIT = false>
 __global__ void __launch_bounds__(CSK_THREADS, 1) k_tc_csk(const __grid_constant__ CskParams P) {
-  using C = CskCfg<BN, PAIR>;
+  using C = CskCfg<BN, PAIR, SPLIT>;
   constexpr int H = C::H;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -377,7 +391,10 @@ __global__ void __launch_bounds__(CSK_THREADS, 1) k_tc_csk(const __grid_constant
             const uint32_t fb = smem_u32(&full_bar[stage]);
             mbar_expect_tx(fb, (uint32_t)C::STAGE_BYTES);
             tma_load_2d(smem_u32(sa), &P.mapA, fb, kb * TC_BK, m_tile * TC_BM);
-            tma_load_2d(smem_u32(sa + C::A_BYTES), &P.mapX[w], fb, kb * TC_BK, n_tile * BN);
+#pragma unroll
+            for (int q = 0; q < C::BR / BN; ++q)
+              tma_load_2d(smem_u32(sa + C::A_BYTES + q * BN * TC_BK * 2), &P.mapX[w], fb, kb * TC_BK,
+                          (SPLIT ? q * a.B : 0) + n_tile * BN);
           }
           issued_mask |= 1u << stage;
           issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
@@ -460,7 +477,7 @@ __global__ void __launch_bounds__(CSK_THREADS, 1) k_tc_csk(const __grid_constant
           float* mine = P.ws + (((size_t)tile * S + sp_me) * H + h) * BN * TC_BM;
           float g[32];
           for (int c0 = wg * (BN / 2); c0 < (wg + 1) * (BN / 2); c0 += 32) {
-            tmem_ld32(tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)c0, g);
+            tc_chunk<BN, SPLIT>(tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)c0, g);
             float* dst = (c0 >= c_begin && c0 < c_end) ? part : mine;
 #pragma unroll
             for (int j = 0; j < 32; ++j) dst[(c0 + j) * TC_BM + row] = g[j];
@@ -500,7 +517,7 @@ __global__ void __launch_bounds__(CSK_THREADS, 1) k_tc_csk(const __grid_constant
     // from shared memory and L2, not TMEM, so any warp may take any columns.  No CTA reads
     // another's shared memory from here on: the next cluster barrier is the next iteration's.
     void* bits = it + 1 == P.iters ? P.bits_last : nullptr;
-    csk_epilogue<BN, MODE>(a, P.xop[w ^ 1], bits, reinterpret_cast<const float*>(tiles),
+    csk_epilogue<BN, MODE, SPLIT>(a, P.xop[w ^ 1], bits, reinterpret_cast<const float*>(tiles),
                            P.ws + ((size_t)tile * S * H + h) * BN * TC_BM, (int64_t)H * BN * TC_BM, sp_me, S, mb,
                            (int64_t)n_tile * BN, c_begin, c_end, warp, lane);
     if (it + 1 == P.iters) break;
@@ -535,10 +552,10 @@ __global__ void __launch_bounds__(CSK_THREADS, 1) k_tc_csk(const __grid_constant
   }
 }
 
-template <int BN, int MODE, bool PAIR>
+template <int BN, int MODE, bool PAIR, bool SPLIT = false>
 cudaError_t csk_set_attr() {
-  return cudaFuncSetAttribute(k_tc_csk<BN, MODE, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              CskCfg<BN, PAIR>::SMEM);
+  return cudaFuncSetAttribute(k_tc_csk<BN, MODE, PAIR, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              CskCfg<BN, PAIR, SPLIT>::SMEM);
 }
 
 template <int BN, bool PAIR>
@@ -548,12 +565,12 @@ cudaError_t csk_set_attrs() {
 }
 
 // cluster: CTAs per cluster (S, or 2 S for pairs)
-template <int BN, bool PAIR>
+template <int BN, bool PAIR, bool SPLIT = false>
 cudaLaunchConfig_t csk_config(int grid, int cluster, cudaLaunchAttribute* attr, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(CSK_THREADS);
-  cfg.dynamicSmemBytes = CskCfg<BN, PAIR>::SMEM;
+  cfg.dynamicSmemBytes = CskCfg<BN, PAIR, SPLIT>::SMEM;
   cfg.stream = s;
   attr->id = cudaLaunchAttributeClusterDimension;
   attr->val.clusterDim.x = (unsigned)cluster;
@@ -621,11 +638,11 @@ void coop_record(int dev, int ok) {
 // together with clusters is remembered and launched plainly (the launch is one wave of clusters
 // either way).  The first attempt is never made during stream capture, where a refused launch
 // would end the capture.
-template <int BN, int MODE, bool PAIR>
+template <int BN, int MODE, bool PAIR, bool SPLIT = false>
 cudaError_t csk_launch(const CskParams& P, int tiles, cudaStream_t s) {
   const int cluster = P.S * (PAIR ? 2 : 1);
   cudaLaunchAttribute attrs[2];
-  cudaLaunchConfig_t cfg = csk_config<BN, PAIR>(tiles * cluster, cluster, &attrs[0], s);
+  cudaLaunchConfig_t cfg = csk_config<BN, PAIR, SPLIT>(tiles * cluster, cluster, &attrs[0], s);
   if (P.iters > 1) {
     int dev = 0;
     cudaGetDevice(&dev);
@@ -638,14 +655,14 @@ cudaError_t csk_launch(const CskParams& P, int tiles, cudaStream_t s) {
       attrs[1].id = cudaLaunchAttributeCooperative;
       attrs[1].val.cooperative = 1;
       cfg.numAttrs = 2;
-      const cudaError_t e = cudaLaunchKernelEx(&cfg, k_tc_csk<BN, MODE, PAIR>, P);
+      const cudaError_t e = cudaLaunchKernelEx(&cfg, k_tc_csk<BN, MODE, PAIR, SPLIT>, P);
       if (known < 0) coop_record(dev, e == cudaSuccess ? 1 : 0);
       if (e == cudaSuccess || known > 0) return e;
       cudaGetLastError();
       cfg.numAttrs = 1;
     }
   }
-  return cudaLaunchKernelEx(&cfg, k_tc_csk<BN, MODE, PAIR>, P);
+  return cudaLaunchKernelEx(&cfg, k_tc_csk<BN, MODE, PAIR, SPLIT>, P);
 }
 
 }  // namespace
@@ -698,6 +715,7 @@ cudaError_t launch_tc_csk(const TcPlan& plan, int which_x, const EpiArgs& a, int
     r = r == cudaSuccess ? csk_set_attrs<256, false>() : r;
     r = r == cudaSuccess ? csk_set_attrs<128, true>() : r;
     r = r == cudaSuccess ? csk_set_attrs<256, true>() : r;
+    r = r == cudaSuccess ? csk_set_attr<64, EPI_UPDATE, false, true>() : r;
     return r;
   });
   if (attr_err != cudaSuccess) return attr_err;
@@ -736,6 +754,7 @@ cudaError_t launch_tc_csk(const TcPlan& plan, int which_x, const EpiArgs& a, int
   const int tiles = ((a.n + TC_BM - 1) / TC_BM) * P.n_tiles;
   switch (plan.tile_n) {
     case 64:
+      if (plan.split && mode == EPI_UPDATE) return csk_launch<64, EPI_UPDATE, false, true>(P, tiles, s);
       return mode == EPI_UPDATE ? csk_launch<64, EPI_UPDATE, false>(P, tiles, s) : csk_launch<64, EPI_EVAL, false>(P, tiles, s);
     case 128:
       return mode == EPI_UPDATE ? csk_launch<128, EPI_UPDATE, false>(P, tiles, s)

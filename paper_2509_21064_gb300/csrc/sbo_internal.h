@@ -46,8 +46,8 @@ enum Layout : int { LAYOUT_RN = 0 /* [r][i] */, LAYOUT_NR = 1 /* [i][r] */ };
 // canonical A for the 64 x 64 tile pairs (I, J), I <= J, of tile columns [j0, j1) (rows of Q up
 // to tile j1 must be present); c' = c + diag Q once all of Q is present
 cudaError_t launch_canon_dense(const void* Qd, int q_bytes, int64_t n, int64_t j0, int64_t j1, void* A, int64_t lda,
-                               int a_type, unsigned long long* rowsum, uint32_t* range_err, int64_t a_limit,
-                               cudaStream_t s);
+                               int a_type, void* A16, unsigned long long* rowsum, uint32_t* range_err,
+                               int64_t a_limit, cudaStream_t s);
 cudaError_t launch_canon_linear(const void* Qd, int q_bytes, const int32_t* cd, int64_t n, float* cp, int64_t* cp64,
                                 cudaStream_t s);
 cudaError_t launch_rowsum_check(const unsigned long long* rowsum, const int64_t* cp64, int64_t n,
@@ -57,6 +57,8 @@ cudaError_t launch_init_state(int n, int B, int64_t ld, int layout, uint64_t see
                               uint32_t* err, cudaStream_t s);
 cudaError_t launch_to_operand(const float* X, int n, int B, int64_t ld_in, void* out, int64_t ld_out,
                               int op_type, cudaStream_t s);
+cudaError_t launch_to_pieces(const float* X, int n, int B, int64_t ld_in, void* out, int64_t ld_out, bool unit,
+                             cudaStream_t s);
 cudaError_t launch_to_operand_t(const float* X, int n, int B, int64_t ld_in, void* out, int64_t ld_out,
                                 int op_type, cudaStream_t s);
 cudaError_t launch_bits_to_operand(const uint8_t* bits, int n, int count, void* out, int64_t ld_out,
@@ -225,6 +227,7 @@ struct TcPlan {
   float* ws;               // >= sms * tile_n * 128 floats
   int* counters;           // >= sms * 8 ints, zero before the first launch
   int max_splits;
+  bool split;              // FP32 problem: the operands are three BF16 pieces, [3 B][ld] (tile_n 64)
   bool pair;               // CTA-pair kernel (k_tc2.cu): 256 x 256 tiles; tile_n is then 128
   int csk;                 // >= 2: split-K over a cluster of csk CTAs (csk_pair: CTA pairs) per tile (k_tc3.cu)
   bool csk_pair;           // csk on CTA pairs: tiles of 256 rows x 2 tile_n restarts

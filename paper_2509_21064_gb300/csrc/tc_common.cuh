@@ -101,6 +101,23 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+// Accumulator chunk of 32 restarts: SPLIT adds the three pieces' columns, smallest first.
+template <int BN, bool SPLIT>
+__device__ __forceinline__ void tc_chunk(uint32_t taddr, float (&g)[32]) {
+  if (!SPLIT) {
+    tmem_ld32(taddr, g);
+    return;
+  }
+  float t[32];
+  tmem_ld32(taddr + 2 * BN, g);
+  tmem_ld32(taddr + BN, t);
+#pragma unroll
+  for (int j = 0; j < 32; ++j) g[j] += t[j];
+  tmem_ld32(taddr, t);
+#pragma unroll
+  for (int j = 0; j < 32; ++j) g[j] += t[j];
+}
+
 // ---- CTA pairs and clusters (tcgen05 cta_group::2) ----------------------------------------------
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -212,11 +229,19 @@ __device__ __forceinline__ void epi_load(const EpiArgs& a, int64_t i, bool row_o
   }
 }
 
+template <bool SPLIT>
+__device__ __forceinline__ void epi_store_operand(const EpiArgs& a, int64_t idx, float x) {
+  __nv_bfloat16* xp = static_cast<__nv_bfloat16*>(a.Xout) + idx;
+  if (SPLIT) split3(x, 1.0f, 1.0f, xp, xp + a.xpiece, xp + 2 * a.xpiece);
+  else *xp = __float2bfloat16_rn(x);
+}
+
 // One chunk of the PDBO update for a compile-time constraint function GK, with one dual per
 // coordinate (SINGLE false) or per restart (SINGLE true: the warp's 32 rows also add up g(x^t) per
 // restart into row `prow` of the partial sums).  The kind and the form are uniform per launch, so
 // epi_apply picks one specialisation per chunk instead of testing them per element.
-template <int GK, bool SINGLE>
+// SPLIT: x^{t+1} goes out as the three BF16 pieces of split3.
+template <int GK, bool SINGLE, bool SPLIT = false>
 __device__ __forceinline__ void epi_update(const EpiArgs& a, int64_t i, bool row_ok, float cpi, int64_t rbase,
                                            int lane, const float (&g)[32], const float (&u)[32], const float (&v)[32],
                                            int prow) {
@@ -235,7 +260,7 @@ __device__ __forceinline__ void epi_update(const EpiArgs& a, int64_t i, bool row
         const float xn = pdbo_update(x, y, d, gx, a.alpha, a.beta, a.delta, a.grad_tol, &yn);
         if (a.Gd) a.Gd[idx] = d;
         a.Xm[idx] = xn;
-        static_cast<__nv_bfloat16*>(a.Xout)[idx] = __float2bfloat16_rn(xn);
+        epi_store_operand<SPLIT>(a, idx, xn);
         if (a.bits_out)
           static_cast<__nv_bfloat16*>(a.bits_out)[idx] = __float2bfloat16_rn(xn > 0.5f ? 1.0f : 0.0f);
         gv[j] = gx;
@@ -256,7 +281,7 @@ __device__ __forceinline__ void epi_update(const EpiArgs& a, int64_t i, bool row
         if (a.Gd) a.Gd[idx] = d;
         a.Xm[idx] = xn;
         a.Y[idx] = yn;
-        static_cast<__nv_bfloat16*>(a.Xout)[idx] = __float2bfloat16_rn(xn);
+        epi_store_operand<SPLIT>(a, idx, xn);
         if (a.bits_out)
           static_cast<__nv_bfloat16*>(a.bits_out)[idx] = __float2bfloat16_rn(xn > 0.5f ? 1.0f : 0.0f);
       }
@@ -267,17 +292,17 @@ __device__ __forceinline__ void epi_update(const EpiArgs& a, int64_t i, bool row
 // One chunk of the epilogue given the accumulator values g (= (A x_r)_i for 32 restarts r).  In
 // the single-constraint form (a.mu set) the warp's 32 rows also add up g(x^t) per restart into
 // row `prow` of the partial sums.
-template <int MODE>
+template <int MODE, bool SPLIT = false>
 __device__ __forceinline__ void epi_apply(const EpiArgs& a, int64_t i, bool row_ok, float cpi, long long cp2,
                                           int64_t rbase, int lane, const float (&g)[32], const float (&u)[32],
                                           const float (&v)[32], int prow = 0) {
   if (MODE == EPI_UPDATE) {
     if (a.gkind == G_ENTROPY) {
-      if (a.mu) epi_update<G_ENTROPY, true>(a, i, row_ok, cpi, rbase, lane, g, u, v, prow);
-      else epi_update<G_ENTROPY, false>(a, i, row_ok, cpi, rbase, lane, g, u, v, prow);
+      if (a.mu) epi_update<G_ENTROPY, true, SPLIT>(a, i, row_ok, cpi, rbase, lane, g, u, v, prow);
+      else epi_update<G_ENTROPY, false, SPLIT>(a, i, row_ok, cpi, rbase, lane, g, u, v, prow);
     } else {
-      if (a.mu) epi_update<G_QUAD, true>(a, i, row_ok, cpi, rbase, lane, g, u, v, prow);
-      else epi_update<G_QUAD, false>(a, i, row_ok, cpi, rbase, lane, g, u, v, prow);
+      if (a.mu) epi_update<G_QUAD, true, SPLIT>(a, i, row_ok, cpi, rbase, lane, g, u, v, prow);
+      else epi_update<G_QUAD, false, SPLIT>(a, i, row_ok, cpi, rbase, lane, g, u, v, prow);
     }
   } else if (MODE == EPI_EVAL) {
 #pragma unroll

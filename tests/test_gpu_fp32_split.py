@@ -1,0 +1,94 @@
+"""FP32 dense problems on the tensor cores (A exact in BF16, x as three BF16 pieces): at least as exact as
+the FP32 CUDA-core form, at the edges of its 128 x 64 tiles and 64-wide k-blocks.  Bounds: the
+trajectory within the FP32 tolerance 1e-5 of the FP64 oracle; A x against FP64 no further off than the
+CUDA-core form on the same inputs."""
+import numpy as np
+import pytest
+
+import oracle as O
+import workloads as W
+from paper_2509_21064_gb300 import sbo as S
+from paper_2509_21064_gb300.build import build as build_lib
+from _helpers import gpu_trajectory, normwise, oracle_trajectory, to_gda_params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build_lib()
+    S.lib()
+
+
+@pytest.mark.parametrize("n,B", [(65, 1), (128, 64), (129, 65), (640, 130), (1001, 37)])
+def test_split_trajectory_and_evaluations(n, B):
+    Q, c = W.dense_qubo(n, seed=n)
+    p = W.dense_params(Q, restarts=B, iters=60, eval_every=10, seed=7)
+    prm = to_gda_params(p)
+    with S.Problem.dense(Q, c, precision=S.SBO_FP32) as P:
+        gx, gy = gpu_trajectory(P, prm, 50)
+        assert P.info()["kernel"] == S.KERNEL_TC
+        ox, oy, _ = oracle_trajectory(Q, c, p, 50)
+        assert normwise(gx, ox).max() <= 1e-5 and normwise(gy, oy).max() <= 1e-5
+        trace = P.trace()
+        for e, F in enumerate(trace):
+            assert int(O.objective_batch(Q, c, O.round_bits(gx[10 * (e + 1)])).min()) == int(F)
+        P.gda(prm)
+        x, F, _, _ = P.best()
+        bits = (np.random.default_rng(0).random((70, n)) > 0.5).astype(np.uint8)
+        assert np.array_equal(P.eval(bits), O.objective_batch(Q, c, bits))
+    assert O.objective(Q, c, x) == F
+
+
+def _gradient(fn, P, X):
+    import torch
+    Xt = torch.tensor(X, dtype=torch.float32, device="cuda")
+    GX = torch.empty_like(Xt)
+    fn(P.h, X.shape[0], Xt.data_ptr(), torch.zeros_like(Xt).data_ptr(), None, None, GX.data_ptr(), None,
+       torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    return GX.cpu().numpy().astype(np.float64)
+
+
+@pytest.mark.parametrize("n,B,values", [(400, 3, "unit"), (513, 64, "unit"), (1500, 130, "unit"), (3000, 70, "unit"),
+                                        (1500, 66, "tiny"), (1500, 66, "large"), (1500, 66, "small"),
+                                        (700, 65, "binary")])
+def test_split_is_no_further_from_fp64_than_the_cuda_cores(n, B, values):
+    """dL/dx at y = 0 is A x + c'.  sbo_lagrangian takes the split form, sbo_lagrangian_noalloc the CUDA cores."""
+    Q, c = W.dense_qubo(n, seed=n + 1)
+    rng = np.random.default_rng(n)
+    X = {"unit": lambda: rng.random((B, n)), "tiny": lambda: rng.random((B, n)) * 2.0**-rng.integers(0, 40, (B, n)),
+         "large": lambda: rng.normal(size=(B, n)) * 10.0**rng.integers(-3, 6, (B, n)),
+         "small": lambda: rng.normal(size=(B, n)) * 1e-20,
+         "binary": lambda: rng.integers(0, 2, (B, n)).astype(float)}[values]().astype(np.float32).astype(np.float64)
+    A, cp = O.canonicalize(Q, c)
+    if values == "small":
+        cp = 0.0 * cp   # below FP32 beside c'
+    want = X @ A + cp
+    with S.Problem.dense(Q, c * (values != "small"), precision=S.SBO_FP32) as P:
+        split = np.linalg.norm(_gradient(S.sbo_lagrangian, P, X) - want) / np.linalg.norm(want)
+        simt = np.linalg.norm(_gradient(S.sbo_lagrangian_noalloc, P, X) - want) / np.linalg.norm(want)
+    # 6e-8: half an FP32 ulp, the rounding of the result itself
+    assert split <= max(simt, 6e-8), (split, simt)
+
+
+def test_split_keeps_infinities_and_nan():
+    n, B = 500, 6
+    Q, c = W.dense_qubo(n, seed=3)
+    X = np.random.default_rng(1).random((B, n))
+    X[1, 5], X[2, 7], X[3, 9], X[4, 11] = np.inf, -np.inf, np.nan, 3.4e38
+    with S.Problem.dense(Q, c, precision=S.SBO_FP32) as P:
+        split, simt = (_gradient(f, P, X) for f in (S.sbo_lagrangian, S.sbo_lagrangian_noalloc))
+    assert np.array_equal(np.isnan(split), np.isnan(simt))
+    assert np.array_equal(np.isposinf(split), np.isposinf(simt)) and np.array_equal(np.isneginf(split), np.isneginf(simt))
+
+
+def test_entries_beyond_bf16_stay_on_the_cuda_cores():
+    n = 130
+    Q = np.random.default_rng(2).integers(-400, 401, (n, n)).astype(np.int32)
+    p = W.dense_params(Q, restarts=9, iters=20, eval_every=10, seed=1)
+    with S.Problem.dense(Q, None, precision=S.SBO_FP32) as P:
+        P.gda(to_gda_params(p))
+        assert P.info()["kernel"] == S.KERNEL_SIMT
+        x, F, _, _ = P.best()
+    assert O.objective(Q, np.zeros(n, np.int32), x) == F
