@@ -1958,8 +1958,14 @@ sbo_status sbo_lagrangian(sbo_problem* p, int32_t B, const float* X_dev, const f
   a.gout = gout_dev;
   a.err = p->err;
   a.gkind = p->opt_g;
-  if (L_dev) SBO_CUDA(cudaMemsetAsync(L_dev, 0, sizeof(float) * B, s));
   cudaError_t e;
+  if (p->fmt == FMT_CSR && p->rst_buf) {
+    e = launch_csr_lagr(p->rst, a, p->prec == SBO_FP32 ? OP_F32 : OP_BF16, p->sms, s);
+    ++p->launches;
+    if (e != cudaSuccess) return cuda_fail(e, "Lagrangian launch");
+    return SBO_OK;
+  }
+  if (L_dev) SBO_CUDA(cudaMemsetAsync(L_dev, 0, sizeof(float) * B, s));
   if (p->fmt == FMT_CSR) {
     // sparse form: x goes to the variable-major operand of the sparse kernel (FP32, or BF16 for
     // BF16 / E4M3 weights), the epilogue reads the caller's FP32 x and y

@@ -34,7 +34,7 @@
 namespace sbo {
 
 constexpr int RST_THREADS = 1024;
-constexpr int RST_SPARE = 2;   // groups a warp reads ahead of their use
+constexpr int RST_SPARE = 4;   // spare groups at the end of the streams: warps read up to four ahead of their use
 constexpr int RST_WARPS = RST_THREADS / 32;
 constexpr int RST_PAD = 32;     // positions after the last one whose x is 0
 constexpr size_t RST_SMEM_MAX = 225 * 1024;   // dynamic; the static arrays take up to 1.2 KB of the 227
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
     xs[npos * R + k] = xs[(nx_pos + npos) * R + k] = 0.0f;
   if (threadIdx.x < RST_PAD) bb[npos + threadIdx.x] = 0;
   for (int k = threadIdx.x; k < P.slices; k += RST_THREADS) ngr[k] = P.ngroups[k];
-  constexpr int AHEAD = ONE || (NARROW && Q <= 10) ? RST_SPARE : 1;   // groups in flight per warp (registers allowing)
+  constexpr int AHEAD = ONE || (NARROW && Q <= 10) ? 2 : 1;   // groups in flight per warp (registers allowing)
   const uint32_t stream0 = P.wstart[warp] * 32 + lane;
   constexpr int NC = PACK ? (Q + 1) / 2 : Q;
   float cps[PACK ? 1 : NC];
@@ -456,6 +456,11 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
   }
 }
 
+}  // namespace
+
+#ifdef RST_PICK
+namespace {
+
 template <int Q, int R, bool PACK>
 RestartKernel kernel_of(bool bf16, bool one) {
   constexpr bool N = RST_NARROW;
@@ -480,5 +485,6 @@ RestartKernel RST_PICK(const CsrRestartShape& sh, int R, bool bf16) {
     default: return nullptr;
   }
 }
+#endif
 
 }  // namespace sbo

@@ -1,0 +1,108 @@
+// Lagrangian value and gradients (section 3.1) of sparse problems, restart by restart, on the structure
+// of the restart-resident runs (csr_restart.cuh).
+//
+// The caller's x, y and the gradients are restart-major ([r][i]), which suits a CTA that takes one restart
+// at a time: x goes to shared memory by position, each thread sums its vertices' neighbours from there,
+// the sums go back to shared memory by vertex, and one pass along i reads y and writes the gradients
+// coalesced and adds up L.  Every input is read and every output written once; L[r] has one owner and
+// needs no atomics.
+//
+// What bounds it: the shared-memory gathers (as in the runs) and the latency of the load and store
+// phases, one CTA per SM.  The row-wise kernel (k_csr EPI_LAGR) after a transposing conversion moved 32
+// bytes per 4 of x, y and the gradients (a lane's neighbours along i lie n apart): 4-regular n = 20,000,
+// B = 512 170 -> 66 us for L alone and 280 -> 103 us for both gradients (12 and 37 us of bytes).
+#include <algorithm>
+
+#include "csr_restart.cuh"
+
+namespace sbo {
+namespace {
+
+template <bool BF16, bool NARROW, int BASE>
+__global__ void __launch_bounds__(RST_THREADS, 1) k_csr_lagr(CsrRestartDev D, EpiArgs a) {
+  using G = typename Group<NARROW>::T;
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int npos = D.shape.slices * 32, n = a.n;
+  float* xs = reinterpret_cast<float*>(smem);   // x by position, zeros beyond
+  float* gs = xs + npos + RST_PAD;              // A x by vertex
+  uint8_t* ngr = reinterpret_cast<uint8_t*>(gs + npos);   // groups of each slice
+  __shared__ float red[RST_WARPS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int p = n + threadIdx.x; p < npos + RST_PAD; p += RST_THREADS) xs[p] = 0.0f;
+  for (int s = threadIdx.x; s < D.shape.slices; s += RST_THREADS) ngr[s] = D.ngroups[s];
+  for (int64_t r = blockIdx.x; r < a.B; r += gridDim.x) {
+    const float* x = a.Xl + r * n;
+    const float* y = a.Yl + r * n;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n; i += RST_THREADS) xs[__ldg(D.pos + i)] = __ldg(x + i);
+    __syncthreads();
+    const G* st = reinterpret_cast<const G*>(D.ent) + D.wstart[warp] * 32 + lane;
+    G nx[RST_SPARE];   // groups read ahead (the streams end in spare ones)
+#pragma unroll
+    for (int d = 0; d < RST_SPARE; ++d, st += 32) nx[d] = __ldg(st);
+    int v = warp * 32 + lane < n ? __ldg(D.perm + warp * 32 + lane) : 0;   // vertex, a slice ahead
+    for (int s = warp; s < D.shape.slices; s += RST_WARPS) {
+      const int ng = ngr[s], p = s * 32 + lane, i = v;
+      if (p + RST_THREADS < n) v = __ldg(D.perm + p + RST_THREADS);
+      float acc[1] = {0.0f};
+      for (int g = 0; g < ng; ++g) {
+        const G e = nx[0];
+#pragma unroll
+        for (int d = 0; d + 1 < RST_SPARE; ++d) nx[d] = nx[d + 1];
+        nx[RST_SPARE - 1] = __ldg(st);
+        st += 32;
+        gather4<1, BF16, BASE>(xs, e, D.shape.wbits, acc);
+      }
+      if (p < n) gs[i] = acc[0];
+    }
+    __syncthreads();
+    const float sc = a.gout ? a.gout[r] : 1.0f;
+    float l = 0.0f;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += RST_THREADS) {
+      const float xi = __ldg(x + i), yi = __ldg(y + i), g = gs[i], c = __ldg(a.cp + i);
+      const float gx = g_val(xi, a.gkind);
+      if (a.GX) a.GX[r * n + i] = sc * (g + c + yi * g_der(xi, a.gkind));
+      if (a.GY) a.GY[r * n + i] = sc * gx;
+      l += 0.5f * xi * g + c * xi + yi * gx;
+    }
+    if (a.L) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (lane == 0) red[warp] = l;
+      __syncthreads();
+      if (warp == 0) {
+        l = red[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) a.L[r] = l;
+      }
+    }
+    __syncthreads();   // gs and red are free again
+  }
+}
+
+using LagrKernel = void (*)(CsrRestartDev, EpiArgs);
+template <bool BF16, bool NARROW>
+LagrKernel lagr_of(bool base1) {
+  return base1 ? (LagrKernel)k_csr_lagr<BF16, NARROW, 1> : (LagrKernel)k_csr_lagr<BF16, NARROW, 2>;
+}
+
+size_t lagr_smem(const CsrRestartShape& sh) { return ((size_t)sh.slices * 64 + RST_PAD) * sizeof(float) + (size_t)sh.slices; }
+
+}  // namespace
+
+cudaError_t launch_csr_lagr(const CsrRestartDev& d, const EpiArgs& a, int op_type, int sms, cudaStream_t s) {
+  const bool base1 = (d.shape.slices + RST_WARPS - 1) / RST_WARPS > 10;   // see k_csr_restart: BASE
+  const bool bf16 = op_type == OP_BF16;
+  LagrKernel k = d.shape.narrow ? (bf16 ? lagr_of<true, true>(base1) : lagr_of<false, true>(base1))
+                                : (bf16 ? lagr_of<true, false>(base1) : lagr_of<false, false>(base1));
+  const size_t sm = lagr_smem(d.shape);
+  if (sm > RST_SMEM_MAX) return cudaErrorInvalidValue;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RST_SMEM_MAX);
+  if (e != cudaSuccess) return e;
+  k<<<(unsigned)std::min(a.B, 4 * sms), RST_THREADS, sm, s>>>(d, a);
+  return cudaGetLastError();
+}
+
+}  // namespace sbo

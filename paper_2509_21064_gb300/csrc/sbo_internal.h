@@ -186,6 +186,8 @@ cudaError_t launch_restart_gather(const CsrRestartDev& d, const float* src, int 
 cudaError_t launch_restart_best_row(const CsrRestartDev& d, const uint8_t* best, int n, int R, int64_t r, uint8_t* dst,
                                     cudaStream_t s);
 cudaError_t launch_restart_convert(const CsrRestartDev& d, RestartLayout L, bool to_rows, cudaStream_t s);
+// k_csr_lagr.cu: sbo_lagrangian of a sparse problem on the same structure (Xl, Yl, L, GX, GY, gout of a).
+cudaError_t launch_csr_lagr(const CsrRestartDev& d, const EpiArgs& a, int op_type, int sms, cudaStream_t s);
 // k_csr_staged.cu: the update with every row's operands staged in shared memory by bulk copies
 // (CSR_FORM_STAGED); max_deg is the largest row length of A.  csr_staged_shape reports its stage
 // layout and false when it does not apply (fewer than four stages fit).

@@ -85,3 +85,42 @@ def test_degree_and_range_limits_fall_back():
     _same(n, (*heavy[:3], heavy[3] * 1001), S.SBO_FP32, 160, 10, 30, [30], resident=False)   # c' not exact in BF16
     _same(700, (*_graph(700, 4, 3)[:3], np.full(700, 1001)), S.SBO_FP32, 5, 10, 30, [30])  # small n keeps FP32 c'
     _same(20481, _graph(20481, 3, 4), S.SBO_FP32, 160, 10, 30, [30], resident=False)
+
+
+@pytest.mark.parametrize("prec", [S.SBO_FP32, S.SBO_BF16])
+@pytest.mark.parametrize("n,deg,B,wmax,g", [(1, 1, 3, 1, 0), (33, 6, 5, 1, 0), (1025, 5, 17, 3, 1), (10240, 4, 3, 3, 0),
+                                           (10241, 4, 3, 1, 0), (20480, 3, 2, 7, 0), (200, 8, 700, 1, 0)])
+def test_sparse_lagrangian_restart_by_restart(n, deg, B, wmax, g, prec):
+    """Value and gradients on the same structure against FP64 numpy (BF16: of the rounded operand), more
+    restarts than CTAs included.  dL/dx sums at most ~30 terms and dL/dy = g(x) two: 1e-6 normwise; L sums n
+    terms in FP32: 1e-5."""
+    import torch
+    from _helpers import bf16_round
+    rowptr, col, val, c = _graph(n, deg, n + B, wmax)
+    rng = np.random.default_rng(n)
+    X = rng.random((B, n)).astype(np.float32)
+    Y = rng.normal(size=(B, n)).astype(np.float32)
+    gout = rng.random(B).astype(np.float32)
+    rows = np.repeat(np.arange(n), np.diff(rowptr))
+    Xc = (bf16_round(X) if prec == S.SBO_BF16 else X.astype(np.float64)).reshape(B, n)
+    G = np.zeros((n, B))
+    np.add.at(G, rows, (val[:, None] * Xc[:, col].T))
+    np.add.at(G, col, (val[:, None] * Xc[:, rows].T))
+    G, Xd, Yd = G.T, X.astype(np.float64), Y.astype(np.float64)
+    if g == S.G_ENTROPY:
+        u = np.clip(Xd, 1e-6, 1 - 1e-6)
+        gv, gd = Xd * np.log(Xd) + (1 - Xd) * np.log1p(-Xd), np.log(u / (1 - u))
+    else:
+        gv, gd = Xd * Xd - Xd, 2 * Xd - 1
+    want = {"L": 0.5 * (Xd * G).sum(1) + Xd @ c + (Yd * gv).sum(1), "GX": gout[:, None] * (G + c + Yd * gd),
+            "GY": gout[:, None] * gv}
+    with S.Problem.csr(n, rowptr, col, val, c, precision=prec) as P:
+        P.set_option(S.SBO_OPT_G, g)
+        Xt, Yt, gt = (torch.tensor(v, device="cuda") for v in (X, Y, gout))
+        L, GX, GY = torch.full((B,), 7.0, device="cuda"), torch.empty_like(Xt), torch.empty_like(Xt)
+        S.sbo_lagrangian(P.h, B, Xt.data_ptr(), Yt.data_ptr(), gt.data_ptr(), L.data_ptr(), GX.data_ptr(), GY.data_ptr(),
+                         torch.cuda.current_stream())
+        torch.cuda.synchronize()
+    for name, got, tol in (("L", L, 1e-5), ("GX", GX, 1e-6), ("GY", GY, 1e-6)):
+        got = got.cpu().numpy().astype(np.float64)
+        assert np.linalg.norm(got - want[name]) <= tol * max(np.linalg.norm(want[name]), 1e-3), name
