@@ -596,30 +596,33 @@ CsrRestartRun restart_run_args(const sbo_problem* p) {
   return r;
 }
 
+// Evaluation counters after `steps` more iterations: the evaluation points are the multiples of K, and T.
+void evals_after(const sbo_problem* p, int64_t steps, long long* n_evals, long long* t_last) {
+  const int64_t K = p->prm.eval_every, T = p->prm.iters, t0 = p->t, t1 = t0 + steps;
+  const bool at_T = T > t0 && T <= t1;
+  *n_evals = p->n_evals_host + t1 / K - t0 / K + (at_T && T % K != 0 ? 1 : 0);
+  *t_last = p->t_last_eval;
+  if (t1 / K > t0 / K) *t_last = t1 / K * K;
+  if (at_T) *t_last = std::max<long long>(*t_last, T);
+}
+
 sbo_status run_restart(sbo_problem* p, int64_t iters) {
   sbo_status st = to_units(p);
   if (st != SBO_OK) return st;
   const int64_t per = p->opt_steps_per_launch == 0 ? 4096 : p->opt_steps_per_launch;
-  const int64_t K = p->prm.eval_every, T = p->prm.iters;
   for (int64_t done = 0; done < iters;) {
     const int64_t chunk = std::min(per, iters - done);
-    const int64_t t0 = p->t, t1 = p->t + chunk;
     CsrRestartRun r = restart_run_args(p);
-    r.t0 = t0;
-    r.K = K;
-    r.T = T;
+    r.t0 = p->t;
+    r.K = p->prm.eval_every;
+    r.T = p->prm.iters;
     r.e0 = p->n_evals_host;
     r.iters = (int)chunk;
-    // evaluation points in (t0, t1]: the multiples of K, and T
-    const bool at_T = T > t0 && T <= t1;
-    r.n_evals_new = p->n_evals_host + t1 / K - t0 / K + (at_T && T % K != 0 ? 1 : 0);
-    r.t_last_new = p->t_last_eval;
-    if (t1 / K > t0 / K) r.t_last_new = t1 / K * K;
-    if (at_T) r.t_last_new = std::max<int64_t>(r.t_last_new, T);
+    evals_after(p, chunk, &r.n_evals_new, &r.t_last_new);
     cudaError_t e = launch_csr_restart(p->rst, base_args(p), p->op_type, r, p->rst_R, p->sms, p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "restart-resident launch");
     ++p->launches;
-    p->t = t1;
+    p->t += chunk;
     p->n_evals_host = r.n_evals_new;
     p->t_last_eval = r.t_last_new;
     done += chunk;
@@ -660,20 +663,16 @@ sbo_status run_tiny(sbo_problem* p, int64_t steps) {
   a.trace = p->trace;
   a.e0 = p->n_evals_host;
   a.trace_cap = p->trace_cap;
-  a.evalF = p->evalF;
+  a.n_evals = p->n_evals;
+  a.t_last = p->t_last;
+  evals_after(p, steps, &a.n_evals_new, &a.t_last_new);
   a.G = p->Gd;
   cudaError_t e = launch_tiny(a, p->stream);
   ++p->launches;
   if (e != cudaSuccess) return cuda_fail(e, "tiny-n launch");
-  int64_t ne = 0;
-  for (int64_t t = p->t + 1; t <= p->t + steps; ++t)
-    if (t % p->prm.eval_every == 0 || t == p->prm.iters) { ++ne; p->t_last_eval = t; }
-  p->n_evals_host += ne;
+  p->n_evals_host = a.n_evals_new;
+  p->t_last_eval = a.t_last_new;
   p->t += steps;
-  long long ne_dev = (long long)p->n_evals_host, tl = (long long)p->t_last_eval;
-  SBO_CUDA(cudaMemcpyAsync(p->n_evals, &ne_dev, sizeof(long long), cudaMemcpyHostToDevice, p->stream));
-  SBO_CUDA(cudaMemcpyAsync(p->t_last, &tl, sizeof(long long), cudaMemcpyHostToDevice, p->stream));
-  SBO_CUDA(cudaStreamSynchronize(p->stream));  // the host values above must outlive the copies
   return SBO_OK;
 }
 

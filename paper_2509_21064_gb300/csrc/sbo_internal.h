@@ -86,7 +86,8 @@ struct TinyArgs {
   uint8_t* bestBits;       // [B][ld]
   long long* trace;        // min_r F per evaluation, written at trace[e0 + e]
   int64_t e0, trace_cap;
-  long long* evalF;        // scratch [B], F of the current evaluation
+  long long *n_evals, *t_last;         // set to the values below by the launch
+  long long n_evals_new, t_last_new;
   float* G;                // if non-null: dL/dx of the latest iteration, [B][ld]
 };
 cudaError_t launch_tiny(const TinyArgs& a, cudaStream_t s);
