@@ -502,7 +502,8 @@ bool restart_wanted(const sbo_problem* p) {
          (p->opt_steps_per_launch == 0 || p->opt_steps_per_launch >= RESTART_MIN_ITERS);
 }
 bool restart_runs(const sbo_problem* p, int64_t iters) {
-  return p->kernel == KER_CSR && p->rst_R > 0 && iters >= RESTART_MIN_ITERS && restart_wanted(p);
+  return (p->kernel == KER_CSR || p->kernel == KER_MAXK) && p->rst_R > 0 && iters >= RESTART_MIN_ITERS &&
+         restart_wanted(p);
 }
 
 // Buffers of the restart-resident runs, for any number of restarts per CTA.
@@ -607,7 +608,8 @@ void evals_after(const sbo_problem* p, int64_t steps, long long* n_evals, long l
 }
 
 sbo_status run_restart(sbo_problem* p, int64_t iters) {
-  sbo_status st = to_units(p);
+  const bool maxk = p->kernel == KER_MAXK;   // (its kernel works on the row-wise arrays)
+  sbo_status st = maxk ? flush_pending(p) : to_units(p);
   if (st != SBO_OK) return st;
   const int64_t per = p->opt_steps_per_launch == 0 ? 4096 : p->opt_steps_per_launch;
   for (int64_t done = 0; done < iters;) {
@@ -619,7 +621,10 @@ sbo_status run_restart(sbo_problem* p, int64_t iters) {
     r.e0 = p->n_evals_host;
     r.iters = (int)chunk;
     evals_after(p, chunk, &r.n_evals_new, &r.t_last_new);
-    cudaError_t e = launch_csr_restart(p->rst, base_args(p), p->op_type, r, p->rst_R, p->sms, p->stream);
+    EpiArgs a = base_args(p);
+    a.Xout = p->Xop[p->cur];
+    cudaError_t e = maxk ? launch_maxk_restart(p->rst, a, p->kparts, p->bestBits, r, p->stream)
+                         : launch_csr_restart(p->rst, a, p->op_type, r, p->rst_R, p->sms, p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "restart-resident launch");
     ++p->launches;
     p->t += chunk;
@@ -1146,6 +1151,41 @@ sbo_status sbo_create_dense_i8(int64_t n, const int8_t* Q, const int32_t* c, int
   return create_dense_impl(n, Q, 1, c, precision, stream, out);
 }
 
+// The restart-resident structure in one device buffer: group streams (16-byte groups), c' exact, then the
+// 4-byte tables and the group counts.
+static sbo_status upload_restart(sbo_problem* p, const CsrRestartHost& rh) {
+  const size_t b_ent = rh.ent.size() * 4, b_c64 = rh.cpp64.size() * 8, b_ws = rh.wstart.size() * 4,
+               b_perm = rh.perm.size() * 4, b_pos = rh.pos.size() * 4, b_cp = rh.cpp.size() * 4,
+               b_w = rh.ngroups.size();
+  std::vector<uint8_t> img(b_ent + b_c64 + b_ws + b_perm + b_pos + b_cp + b_w);
+  size_t off = 0;
+  auto put = [&](const void* src, size_t bytes) {
+    std::memcpy(img.data() + off, src, bytes);
+    off += bytes;
+    return off - bytes;
+  };
+  const size_t o_ent = put(rh.ent.data(), b_ent), o_c64 = put(rh.cpp64.data(), b_c64),
+               o_ws = put(rh.wstart.data(), b_ws), o_perm = put(rh.perm.data(), b_perm),
+               o_pos = put(rh.pos.data(), b_pos), o_cp = put(rh.cpp.data(), b_cp), o_w = put(rh.ngroups.data(), b_w);
+  uint8_t* dev = nullptr;
+  cudaError_t e = dalloc(&dev, img.size(), p->stream);
+  if (e != cudaSuccess)
+    return e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation failed") : cuda_fail(e, "cudaMalloc");
+  p->rst_buf = dev;
+  if ((e = cudaStreamSynchronize(p->stream)) != cudaSuccess ||
+      (e = cudaMemcpy(dev, img.data(), img.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+    return cuda_fail(e, "upload of the graph");
+  p->rst.shape = rh.shape;
+  p->rst.ent = reinterpret_cast<uint32_t*>(dev + o_ent);
+  p->rst.cpp64 = reinterpret_cast<int64_t*>(dev + o_c64);
+  p->rst.wstart = reinterpret_cast<uint32_t*>(dev + o_ws);
+  p->rst.perm = reinterpret_cast<int32_t*>(dev + o_perm);
+  p->rst.pos = reinterpret_cast<int32_t*>(dev + o_pos);
+  p->rst.cpp = reinterpret_cast<float*>(dev + o_cp);
+  p->rst.ngroups = dev + o_w;
+  return SBO_OK;
+}
+
 sbo_status sbo_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col, const int32_t* val,
                           const int32_t* c, int32_t precision, void* stream, sbo_problem** out) {
   g_last_error.clear();
@@ -1255,35 +1295,10 @@ sbo_status sbo_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const i
       (e = cudaMemcpy(p->cp64, cp.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice)) != cudaSuccess)
     return bail(cuda_fail(e, "upload CSR"));
   CsrRestartHost rh;
-  if (csr_restart_build(n, rp.data(), cc.data(), vv.data(), cp.data(), &rh)) {
-    // one buffer: group streams (16-byte groups), c' exact, then the 4-byte tables and the group counts
-    const size_t b_ent = rh.ent.size() * 4, b_c64 = rh.cpp64.size() * 8, b_ws = rh.wstart.size() * 4,
-                 b_perm = rh.perm.size() * 4, b_pos = rh.pos.size() * 4, b_cp = rh.cpp.size() * 4, b_w = rh.ngroups.size();
-    std::vector<uint8_t> img(b_ent + b_c64 + b_ws + b_perm + b_pos + b_cp + b_w);
-    size_t off = 0;
-    auto put = [&](const void* src, size_t bytes) {
-      std::memcpy(img.data() + off, src, bytes);
-      off += bytes;
-      return off - bytes;
-    };
-    const size_t o_ent = put(rh.ent.data(), b_ent), o_c64 = put(rh.cpp64.data(), b_c64),
-                 o_ws = put(rh.wstart.data(), b_ws), o_perm = put(rh.perm.data(), b_perm), o_pos = put(rh.pos.data(), b_pos),
-                 o_cp = put(rh.cpp.data(), b_cp), o_w = put(rh.ngroups.data(), b_w);
-    uint8_t* dev = nullptr;
-    if ((e = dalloc(&dev, img.size(), cs)) != cudaSuccess)
-      return bail(e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation failed") : cuda_fail(e, "cudaMalloc"));
-    p->rst_buf = dev;
-    if ((e = cudaStreamSynchronize(cs)) != cudaSuccess ||
-        (e = cudaMemcpy(dev, img.data(), img.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
-      return bail(cuda_fail(e, "upload CSR"));
-    p->rst.shape = rh.shape;
-    p->rst.ent = reinterpret_cast<uint32_t*>(dev + o_ent);
-    p->rst.cpp64 = reinterpret_cast<int64_t*>(dev + o_c64);
-    p->rst.wstart = reinterpret_cast<uint32_t*>(dev + o_ws);
-    p->rst.perm = reinterpret_cast<int32_t*>(dev + o_perm);
-    p->rst.pos = reinterpret_cast<int32_t*>(dev + o_pos);
-    p->rst.cpp = reinterpret_cast<float*>(dev + o_cp);
-    p->rst.ngroups = dev + o_w;
+  if (csr_restart_build(n, rp.data(), cc.data(), vv.data(), cp.data(), CSR_RESTART_WARPS, csr_restart_bank_lanes(n),
+                        csr_restart_shift(n), &rh)) {
+    st = upload_restart(p, rh);
+    if (st != SBO_OK) return bail(st);
   }
   *out = p;
   return SBO_OK;
@@ -1354,6 +1369,16 @@ sbo_status sbo_create_maxkcut(int64_t n, int64_t m, const int32_t* ei, const int
       (e = cudaMemset(p->cp, 0, sizeof(float) * n)) != cudaSuccess ||
       (e = cudaMemset(p->cp64, 0, sizeof(int64_t) * n)) != cudaSuccess)
     return bail(cuda_fail(e, "upload graph"));
+  if (n <= maxk_restart_limit(k)) {
+    std::vector<int64_t> wi(vv.size()), zero((size_t)n, 0);
+    for (size_t q = 0; q < vv.size(); ++q) wi[q] = (int64_t)vv[q];   // (integers below 2^24)
+    CsrRestartHost rh;
+    if (csr_restart_build(n, rp.data(), cc.data(), wi.data(), zero.data(), MAXK_RESTART_WARPS,
+                          k % 4 == 0 ? 8 : k % 2 == 0 ? 16 : 32, 2, &rh)) {
+      st = upload_restart(p, rh);
+      if (st != SBO_OK) return bail(st);
+    }
+  }
   *out = p;
   return SBO_OK;
 }
@@ -1479,6 +1504,8 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
       ker == KER_CSR && !p->single && p->opt_csr_form == 0 && !p->opt_keep_grad && restart_wanted(p);
   if (try_restart) p->rst_R = csr_restart_pick(p->rst.shape, p->n, p->nnz, p->B, p->sms);
   const bool home = p->rst_R > 0;
+  if (ker == KER_MAXK && restart_wanted(p) && maxk_restart_pays(p->rst.shape, p->n, p->nnz, p->kparts, p->B, p->sms))
+    p->rst_R = 1;
   if (!home) {
     if (need_master) al((void**)&p->Xm, xelems * 4);
     al((void**)&p->Y, elems * 4);

@@ -36,6 +36,7 @@ namespace sbo {
 constexpr int RST_THREADS = 1024;
 constexpr int RST_SPARE = 4;   // spare groups at the end of the streams: warps read up to four ahead of their use
 constexpr int RST_WARPS = RST_THREADS / 32;
+static_assert(RST_WARPS == CSR_RESTART_WARPS, "the streams are laid out for this many warps");
 constexpr int RST_PAD = 32;     // positions after the last one whose x is 0
 constexpr size_t RST_SMEM_MAX = 225 * 1024;   // dynamic; the static arrays take up to 1.2 KB of the 227
 
@@ -102,7 +103,7 @@ template <> struct Group<true> { using T = uint2; };
 // Byte offset for R restarts of a position's x, from its offset for BASE restarts.
 template <int R, int BASE>
 __device__ __forceinline__ uint32_t scale_offset(uint32_t o) {
-  return R == BASE ? o : R < BASE ? o >> 1 : R == 2 * BASE ? o << 1 : o << 2;
+  return R == BASE ? o : R < BASE ? o >> 1 : R == 2 * BASE ? o << 1 : R == 4 * BASE ? o << 2 : o << 3;
 }
 // The k-th entry of a group: byte offset of the neighbour's x for R restarts, and its weight.
 template <int R, int BASE>
@@ -114,7 +115,7 @@ __device__ __forceinline__ void entry(const uint4& c, int k, uint32_t, uint32_t&
 template <int R, int BASE>
 __device__ __forceinline__ void entry(const uint2& c, int k, uint32_t wbits, uint32_t& off, float& w) {
   const uint32_t e = k < 2 ? c.x : c.y;
-  constexpr int S = R == 1 ? 2 : R == 2 ? 3 : 4;
+  constexpr int S = R == 1 ? 2 : R == 2 ? 3 : R == 4 ? 4 : 5;
   if (k & 1) {
     off = (e >> (16 - S)) & (0x7fffu << S);
     w = __uint_as_float((e & 0x80000000u) ^ wbits);

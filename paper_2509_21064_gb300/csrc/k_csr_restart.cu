@@ -132,12 +132,12 @@ RestartKernel pick_kernel(const CsrRestartShape& sh, int R, bool bf16) {
 // vertices gives each the free lane of its slice that adds least to the squares of the bank loads of
 // the gathers it takes part in, its own lane where that is as good (a torus in natural order has no
 // conflicts and stays as it is).  Two restarts per CTA (graphs up to 10,240 vertices) gather 8 bytes
-// per lane in two half warps over 16 pairs of banks: there the vertices move within half slices.
+// per lane in two half warps over 16 pairs of banks: there the vertices move within half slices (BK =
+// 16; quarter slices, BK = 8, for the 16-byte gathers of Max-k-Cut).
 // Random 4-regular graph: 3.51 -> 2.05 wavefronts per 4-byte gather (n = 20,000, 3 ms of host time),
 // 6.15 -> 4.10 per 8-byte gather (n = 10,000, 1 ms).
-static void place_lanes(int64_t n, const int32_t* rp, const int32_t* col, std::vector<int32_t>& perm,
-                 std::vector<int32_t>& pos) {
-  const int BK = n > 10 * RST_THREADS ? 32 : 16;
+static void place_lanes(int64_t n, const int32_t* rp, const int32_t* col, int BK, std::vector<int32_t>& perm,
+                        std::vector<int32_t>& pos) {
   const int64_t slices = (n + 31) / 32;
   std::vector<int64_t> first((size_t)slices + 1, 0);   // gather sets (neighbour slots) before each slice
   for (int64_t s = 0; s < slices; ++s) {
@@ -181,7 +181,7 @@ static void place_lanes(int64_t n, const int32_t* rp, const int32_t* col, std::v
 }
 
 bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
-                       CsrRestartHost* out) {
+                       int warps, int bank_lanes, int shift, CsrRestartHost* out) {
   if (n < 1 || n > 20 * RST_THREADS) return false;
   int maxd = 0;
   for (int64_t i = 0; i < n; ++i) maxd = std::max(maxd, rp[i + 1] - rp[i]);
@@ -201,7 +201,6 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
     if (bits_of((float)val[e]) & ~ENT_W) return false;
   // positions by descending degree, equal degrees in vertex order
   const int slices = (int)((n + 31) / 32);
-  const int shift = n > 10 * RST_THREADS ? 2 : 3;   // see k_csr_restart: BASE
   std::vector<int32_t> first((size_t)maxd + 2, 0), perm((size_t)n), pos((size_t)n);
   for (int64_t i = 0; i < n; ++i) ++first[(size_t)(maxd - (rp[i + 1] - rp[i])) + 1];
   for (int d = 0; d <= maxd; ++d) first[(size_t)d + 1] += first[(size_t)d];
@@ -210,7 +209,7 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
     perm[(size_t)p] = (int32_t)i;
     pos[(size_t)i] = p;
   }
-  place_lanes(n, rp, col, perm, pos);
+  place_lanes(n, rp, col, bank_lanes, perm, pos);
   out->ngroups.assign((size_t)slices, 0);
   // The kernel's ONE form walks exactly one group per slice, so with no row above four neighbours slices of isolated vertices hold one (padding) too.
   for (int s = 0; s < slices; ++s) {
@@ -220,17 +219,17 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
     out->ngroups[(size_t)s] = (uint8_t)std::max((width + 3) / 4, maxd <= 4 ? 1 : 0);
   }
   uint32_t groups = 0;
-  out->wstart.assign(RST_WARPS + 1, 0);
-  for (int w = 0; w < RST_WARPS; ++w) {
+  out->wstart.assign(warps + 1, 0);
+  for (int w = 0; w < warps; ++w) {
     out->wstart[(size_t)w] = groups;
-    for (int s = w; s < slices; s += RST_WARPS) groups += out->ngroups[(size_t)s];
+    for (int s = w; s < slices; s += warps) groups += out->ngroups[(size_t)s];
   }
-  out->wstart[RST_WARPS] = groups;
+  out->wstart[warps] = groups;
   const size_t words = narrow ? 64 : 128;   // of a group
   out->ent.assign(((size_t)groups + RST_SPARE) * words, narrow ? (uint32_t)slices * 32u * 0x10001u : 0u);
-  for (int w = 0; w < RST_WARPS; ++w) {
+  for (int w = 0; w < warps; ++w) {
     size_t g = out->wstart[(size_t)w];
-    for (int s = w; s < slices; s += RST_WARPS) {
+    for (int s = w; s < slices; s += warps) {
       const int gr = out->ngroups[(size_t)s];
       for (int l = 0; l < 32; ++l) {
         const int64_t p = (int64_t)s * 32 + l;

@@ -1,0 +1,336 @@
+// Max-k-Cut runs restart by restart: a CTA owns one restart of the whole graph and runs many iterations of
+// the GDA of k_maxk.cu on it without leaving the SM (the idea and the structure of csr_restart.cuh).
+//
+// X of every vertex (KP values) lies in shared memory by position, the logits
+// Z in the registers of the thread that owns the vertex, y beside X.  An iteration gathers the neighbours' X,
+// updates Z and y in place, and, after a barrier, writes X = softmax(Z): no second copy of X is needed.
+// Evaluations (argmax parts, exact cut, best record) stay in the CTA.  The state is read from and
+// written back to the variable-major arrays of k_maxk.cu once per launch.  Same arithmetic in the same
+// order as k_maxk: bit-identical.
+//
+// What bounds it: instruction issue (the exponentials and the division among it) and, with 32 warps, the
+// length of each warp's chain through the two phases.  With 512 threads and y in registers too the
+// unrolled code of 20 vertices per thread was slower (torus n = 10,000, k = 3, B = 100: 8.6 us per
+// iteration, 10.4 with two vertices interleaved); this form takes 7.4, the row-wise kernel 13.7.
+#include <algorithm>
+#include <cstring>
+
+#include "csr_restart.cuh"
+
+namespace sbo {
+namespace {
+
+constexpr int MKR_WARPS = MAXK_RESTART_WARPS;
+constexpr int MKR_THREADS = 32 * MKR_WARPS;
+
+struct MaxkParams {
+  CsrRestartDev D;
+  EpiArgs a;               // Xm: Z; Xout: X of the current iterate; Y
+  uint8_t* bestBits;
+  int64_t t0, K, T, e0;
+  int iters, ent_in_smem;
+  long long *bestF, *bestT, *evalF, *trace, *n_evals, *t_last;
+  long long trace_cap, t_last_new, n_evals_new;
+};
+
+constexpr int maxk_vec(int kp) { return kp % 4 == 0 ? 4 : kp % 2 == 0 ? 2 : 1; }     // floats per shared-memory access
+constexpr int maxk_slots(int kp) { return kp <= 3 ? 10 : 32 / kp; }                  // vertices per thread
+
+// Slots per thread Q: Q KP registers of logits, at most 32 of 64.
+template <int KP, bool NARROW>
+__global__ void __launch_bounds__(MKR_THREADS, 1) k_maxk_restart(const __grid_constant__ MaxkParams P) {
+  constexpr int Q = maxk_slots(KP), V = maxk_vec(KP);
+  using G = typename Group<NARROW>::T;
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int npos = P.D.shape.slices * 32;
+  float* xs = reinterpret_cast<float*>(smem);                  // [npos + RST_PAD][KP], zeros beyond npos
+  float* ys = xs + (size_t)(npos + RST_PAD) * KP;              // y by position
+  G* ent_s = reinterpret_cast<G*>(ys + npos);                  // group streams (when they fit)
+  const uint32_t words = P.ent_in_smem ? (P.D.wstart[MKR_WARPS] + RST_SPARE) * 32 : 0;
+  uint8_t* part = reinterpret_cast<uint8_t*>(ent_s + words);
+  uint8_t* best = part + npos + RST_PAD;
+  uint8_t* ngr = best + npos;
+  __shared__ long long red[MKR_WARPS];
+  __shared__ int s_any;
+  const EpiArgs& a = P.a;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = a.n, slices = P.D.shape.slices;
+  const int64_t r = blockIdx.x;
+  const int p0 = threadIdx.x;
+  const uint32_t wbits = P.D.shape.wbits;
+
+  for (int s = threadIdx.x; s < slices; s += MKR_THREADS) ngr[s] = P.D.ngroups[s];
+  const G* ent_g = static_cast<const G*>(static_cast<const void*>(P.D.ent));
+  for (uint32_t k = threadIdx.x; k < words; k += MKR_THREADS) ent_s[k] = ent_g[k];
+  for (int k = threadIdx.x; k < RST_PAD * KP; k += MKR_THREADS) xs[(size_t)npos * KP + k] = 0.0f;
+  if (threadIdx.x < RST_PAD) part[npos + threadIdx.x] = 0;
+  if (threadIdx.x == 0) s_any = 0;
+
+  // X = softmax(Z) of slot q's vertex into shared memory (k_maxk's arithmetic); its argmax part
+  float z[Q][KP];
+  auto publish = [&](int p, const float (&zv)[KP]) {
+    float zmax = -INFINITY;
+#pragma unroll
+    for (int j = 0; j < KP; ++j) zmax = fmaxf(zmax, zv[j]);
+    float den = 0.0f, e[KP];
+#pragma unroll
+    for (int j = 0; j < KP; ++j) {
+      e[j] = expf(zv[j] - zmax);
+      den += e[j];
+    }
+    const float inv = 1.0f / den;
+#pragma unroll
+    for (int j = 0; j < KP; ++j) e[j] *= inv;
+    float* o = xs + p * KP;
+#pragma unroll
+    for (int j = 0; j < KP; j += V) {
+      if (V == 4) *reinterpret_cast<float4*>(o + j) = make_float4(e[j], e[(j + 1) % KP], e[(j + 2) % KP], e[(j + 3) % KP]);
+      else if (V == 2) *reinterpret_cast<float2*>(o + j) = make_float2(e[j], e[(j + 1) % KP]);
+      else o[j] = e[j];
+    }
+  };
+  auto load_x = [&](const float* p, float (&x)[KP]) {
+#pragma unroll
+    for (int j = 0; j < KP; j += V) {
+      if (V == 4) {
+        const float4 t = *reinterpret_cast<const float4*>(p + j);
+        x[j] = t.x;
+        x[(j + 1) % KP] = t.y;
+        x[(j + 2) % KP] = t.z;
+        x[(j + 3) % KP] = t.w;
+      } else if (V == 2) {
+        const float2 t = *reinterpret_cast<const float2*>(p + j);
+        x[j] = t.x;
+        x[(j + 1) % KP] = t.y;
+      } else {
+        x[j] = p[j];
+      }
+    }
+  };
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int p = p0 + q * MKR_THREADS;
+#pragma unroll
+    for (int j = 0; j < KP; ++j) z[q][j] = 0.0f;
+    if (warp + q * MKR_WARPS < slices) {
+      ys[p] = p < n ? a.Y[(int64_t)P.D.perm[p] * a.ld + r] : 0.0f;
+      if (p < n) {
+        const int64_t i = P.D.perm[p];
+#pragma unroll
+        for (int j = 0; j < KP; ++j) z[q][j] = a.Xm[(i * KP + j) * a.ld + r];
+      }
+      publish(p, z[q]);
+    }
+  }
+  __syncthreads();
+
+  long long bestF = P.bestF[r], bestT = P.bestT[r];   // (every thread keeps the record)
+  const uint32_t stream0 = P.D.wstart[warp] * 32 + lane;
+  int64_t t = P.t0, e_idx = P.e0;
+  const int64_t t_end = P.t0 + P.iters;
+  while (t < t_end) {   // stretches of iterations up to an evaluation point or the end
+    int64_t next = (t / P.K + 1) * P.K;
+    if (P.T > t && P.T < next) next = P.T;
+    const int64_t stop = next < t_end ? next : t_end;
+    for (int left = (int)(stop - t); left > 0; --left) {
+      const G* st = (P.ent_in_smem ? ent_s : ent_g) + stream0;
+      G nx[2] = {st[0], st[32]};   // groups read ahead (the streams end in spare ones)
+      st += 64;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        if (warp + q * MKR_WARPS >= slices) break;   // no later slice either
+        const int p = p0 + q * MKR_THREADS;
+        float acc[KP];
+#pragma unroll
+        for (int j = 0; j < KP; ++j) acc[j] = 0.0f;
+        const int ng = ngr[warp + q * MKR_WARPS];
+        for (int g = 0; g < ng; ++g) {
+          const G c = nx[0];
+          nx[0] = nx[1];
+          nx[1] = *st;
+          st += 32;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            uint32_t off;
+            float w, v[KP];
+            entry<1, 1>(c, k, wbits, off, w);   // 4 x position
+            off *= KP;
+            load_x(reinterpret_cast<const float*>(reinterpret_cast<const char*>(xs) + off), v);
+#pragma unroll
+            for (int j = 0; j < KP; ++j) acc[j] = fmaf(w, v[j], acc[j]);
+          }
+        }
+        float s[KP], h[KP], dot = 0.0f, ss = 0.0f;
+        const float y = ys[p];
+        load_x(xs + p * KP, s);
+#pragma unroll
+        for (int j = 0; j < KP; ++j) {
+          h[j] = 2.0f * (acc[j] + y * s[j]);
+          dot = fmaf(s[j], h[j], dot);
+          ss = fmaf(s[j], s[j], ss);
+        }
+#pragma unroll
+        for (int j = 0; j < KP; ++j) z[q][j] = z[q][j] - a.alpha * (s[j] * (h[j] - dot));
+        ys[p] = y + a.beta * (ss - 1.0f);
+      }
+      __syncthreads();   // every gather of x^t is done
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        if (warp + q * MKR_WARPS >= slices) break;
+        publish(p0 + q * MKR_THREADS, z[q]);
+      }
+      __syncthreads();
+    }
+    t = stop;
+    if (t != next) break;
+    // candidates: the argmax part of every vertex, ties to the smallest
+    for (int p = p0; p < npos; p += MKR_THREADS) {
+      float x[KP];
+      load_x(xs + p * KP, x);
+      int b = 0;
+      float bx = -1.0f;
+#pragma unroll
+      for (int j = 0; j < KP; ++j)
+        if (x[j] > bx) { bx = x[j]; b = j; }
+      part[p] = (uint8_t)b;
+    }
+    __syncthreads();
+    // 2F = -sum over the stored entries of w [parts differ]; a row's sum is exact in FP32 (below 2^24)
+    long long f2 = 0;
+    const G* st = (P.ent_in_smem ? ent_s : ent_g) + stream0;
+    for (int s = warp; s < slices; s += MKR_WARPS) {
+      const int ng = ngr[s], p = s * 32 + lane;
+      const uint8_t mine = part[p];
+      float acc = 0.0f;
+      for (int g = 0; g < ng; ++g, st += 32) {
+        const G c = *st;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          uint32_t off;
+          float w;
+          entry<1, 1>(c, k, wbits, off, w);
+          const uint32_t l = off / 4;
+          // (padding: weight 0, or the zero position beyond npos)
+          if (l < (uint32_t)npos && part[l] != mine) acc += w;
+        }
+      }
+      if (p < n) f2 -= (long long)acc;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) f2 += __shfl_xor_sync(0xffffffffu, f2, o);
+    if (lane == 0) red[warp] = f2;
+    __syncthreads();
+    f2 = 0;
+#pragma unroll
+    for (int w = 0; w < MKR_WARPS; ++w) f2 += red[w];
+    const long long F = f2 / 2;
+    if (threadIdx.x == 0) {
+      P.evalF[r] = F;
+      if (e_idx < P.trace_cap) atomicMin(&P.trace[e_idx], F);
+      if (F < bestF) s_any = 1;
+    }
+    if (F < bestF) {   // strict: equal values keep the earliest t (the same decision in every thread)
+      bestF = F;
+      bestT = t;
+      for (int p = p0; p < npos; p += MKR_THREADS) best[p] = part[p];
+    }
+    ++e_idx;
+    __syncthreads();   // red and part are free again
+  }
+  __syncthreads();
+
+  const bool any = s_any != 0;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int p = p0 + q * MKR_THREADS;
+    if (warp + q * MKR_WARPS >= slices) break;
+    if (p >= n) continue;
+    const int64_t i = P.D.perm[p];
+    float x[KP];
+    load_x(xs + p * KP, x);
+#pragma unroll
+    for (int j = 0; j < KP; ++j) {
+      a.Xm[(i * KP + j) * a.ld + r] = z[q][j];
+      static_cast<float*>(a.Xout)[(i * KP + j) * a.ld + r] = x[j];
+    }
+    a.Y[i * a.ld + r] = ys[p];
+    if (any) P.bestBits[i * a.ld + r] = best[p];
+  }
+  if (threadIdx.x == 0 && any) {
+    P.bestF[r] = bestF;
+    P.bestT[r] = bestT;
+  }
+  if (r == 0 && threadIdx.x == 0) {
+    *P.n_evals = P.n_evals_new;
+    *P.t_last = P.t_last_new;
+  }
+}
+
+using MaxkKernel = void (*)(MaxkParams);
+template <int KP>
+MaxkKernel maxk_of(bool narrow) {
+  return narrow ? (MaxkKernel)k_maxk_restart<KP, true> : (MaxkKernel)k_maxk_restart<KP, false>;
+}
+
+size_t maxk_smem(const CsrRestartShape& sh, int kp, bool ent) {
+  const size_t npos = (size_t)sh.slices * 32;
+  return (npos + RST_PAD) * kp * 4 + npos * 4 + 2 * npos + RST_PAD + (size_t)sh.slices +
+         (ent ? ((size_t)sh.groups + RST_SPARE) * (sh.narrow ? 256 : 512) : 0);
+}
+
+}  // namespace
+
+int64_t maxk_restart_limit(int kp) { return (int64_t)maxk_slots(kp) * MKR_THREADS; }
+
+// Whether a run goes restart by restart.  Both sides' time per iteration (us) from fits to measurements on
+// GB300 (n 300-10,000, k 2-8, mean degree 4-6, B 8-512; within about 20 %): a restart's slices and groups
+// times k, in rounds over the SMs, against the row-wise kernel's rows and gathers per 128 restarts
+// (torus n = 10,000, k = 3, B = 100: 7.4 here, 13.7 row-wise; ER n = 4,096, k = 8, B = 512: 57 and 91).
+bool maxk_restart_pays(const CsrRestartShape& sh, int64_t n, int64_t nnz, int kp, int B, int sms) {
+  if (n > maxk_restart_limit(kp) || maxk_smem(sh, kp, false) > RST_SMEM_MAX) return false;
+  const double here = (double)((B + sms - 1) / sms) * (0.5 + kp * (0.003 * sh.slices + 0.005 * sh.groups));
+  const double rows = 4.5 + (double)((B + 127) / 128) * kp * (4.7e-5 * (double)n + 6.5e-5 * (double)nnz);
+  return here < rows;
+}
+
+cudaError_t launch_maxk_restart(const CsrRestartDev& d, const EpiArgs& a, int kp, uint8_t* bestBits,
+                                const CsrRestartRun& run, cudaStream_t s) {
+  MaxkParams P{};
+  P.D = d;   // streams laid out with entries of 4 x position
+  P.a = a;
+  P.bestBits = bestBits;
+  P.t0 = run.t0;
+  P.K = run.K;
+  P.T = run.T;
+  P.e0 = run.e0;
+  P.iters = run.iters;
+  P.bestF = run.bestF;
+  P.bestT = run.bestT;
+  P.evalF = run.evalF;
+  P.trace = run.trace;
+  P.trace_cap = run.trace_cap;
+  P.n_evals = run.n_evals;
+  P.t_last = run.t_last;
+  P.n_evals_new = run.n_evals_new;
+  P.t_last_new = run.t_last_new;
+  MaxkKernel k = nullptr;
+  switch (kp) {
+    case 2: k = maxk_of<2>(d.shape.narrow); break;
+    case 3: k = maxk_of<3>(d.shape.narrow); break;
+    case 4: k = maxk_of<4>(d.shape.narrow); break;
+    case 5: k = maxk_of<5>(d.shape.narrow); break;
+    case 6: k = maxk_of<6>(d.shape.narrow); break;
+    case 7: k = maxk_of<7>(d.shape.narrow); break;
+    case 8: k = maxk_of<8>(d.shape.narrow); break;
+    default: return cudaErrorInvalidValue;
+  }
+  P.ent_in_smem = maxk_smem(d.shape, kp, true) <= RST_SMEM_MAX;
+  const size_t sm = maxk_smem(d.shape, kp, P.ent_in_smem != 0);
+  if (a.n > maxk_restart_limit(kp) || sm > RST_SMEM_MAX) return cudaErrorInvalidValue;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RST_SMEM_MAX);
+  if (e != cudaSuccess) return e;
+  k<<<(unsigned)a.B, MKR_THREADS, sm, s>>>(P);
+  return cudaGetLastError();
+}
+
+}  // namespace sbo

@@ -173,8 +173,13 @@ struct RestartLayout {
   void* Xop;
   uint8_t* bestBits;
 };
+// warps: of the CTA that will walk the streams; bank_lanes: lanes whose gathers share a pass over the banks
+// (place_lanes in k_csr_restart.cu); shift: wide entries hold position << shift.
+constexpr int CSR_RESTART_WARPS = 32;
+inline int csr_restart_bank_lanes(int64_t n) { return n > 10240 ? 32 : 16; }   // one restart per CTA, or two
+inline int csr_restart_shift(int64_t n) { return n > 10240 ? 2 : 3; }          // bytes of one restart's x, or two's
 bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
-                       CsrRestartHost* out);
+                       int warps, int bank_lanes, int shift, CsrRestartHost* out);
 bool csr_restart_fits(const CsrRestartShape& sh, int R);   // an instantiation exists and x fits on chip
 int csr_restart_pick(const CsrRestartShape& sh, int64_t n, int64_t nnz, int B, int sms);
 size_t csr_restart_positions(const CsrRestartShape& sh);
@@ -196,6 +201,13 @@ bool csr_staged_shape(int64_t ld, int op_type, int max_deg, int* D, int* S, int*
 cudaError_t launch_csr_staged(const int32_t* rowptr, const int32_t* col, const void* val, int val_type,
                               const EpiArgs& a, int op_type, int max_deg, int sms, bool pdl, uint64_t timeout_ns,
                               cudaStream_t s);
+// k_maxk_restart.cu: whole Max-k-Cut runs with one restart per CTA (the state's arrays as in k_maxk.cu, read
+// and written once per launch).  run.X, .Y, .best and .sched are not used.
+constexpr int MAXK_RESTART_WARPS = 32;
+int64_t maxk_restart_limit(int kp);                          // largest n
+bool maxk_restart_pays(const CsrRestartShape& sh, int64_t n, int64_t nnz, int kp, int B, int sms);
+cudaError_t launch_maxk_restart(const CsrRestartDev& d, const EpiArgs& a, int kp, uint8_t* bestBits,
+                                const CsrRestartRun& run, cudaStream_t s);
 // k_maxk.cu  (Max-k-Cut: Z, X as [(i k + j) ld + r], y and parts as [i ld + r]; Z in EpiArgs::Xm)
 cudaError_t launch_maxk(const int32_t* rowptr, const int32_t* col, const float* w, const EpiArgs& a, int kp, int mode,
                         cudaStream_t s);

@@ -1,0 +1,46 @@
+"""Max-k-Cut runs restart by restart against the row-wise kernel (SBO_OPT_EVAL_MODE = 2 keeps it), which the
+oracle parity tests hold: iterates, records, traces and best candidates equal bit for bit, at the edges of
+slices (32 vertices), of 1,024 vertices per register slot and of every k's slots, with split runs."""
+import numpy as np
+import pytest
+
+from paper_2509_21064_gb300 import sbo as S
+from paper_2509_21064_gb300.build import build as build_lib
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build_lib()
+    S.lib()
+
+
+def _run(n, edges, k, prm, chunks, mode):
+    with S.Problem.maxkcut(n, *edges, k) as P:
+        P.set_option(S.SBO_OPT_EVAL_MODE, mode)
+        P.start(prm)
+        n0 = P.launch_count()
+        for c in chunks:
+            P.run(c)
+        P.sync()
+        launches = P.launch_count() - n0
+        return launches, (*P.state(), *P.restart_best(), P.trace(), *P.best())
+
+
+@pytest.mark.parametrize("n,k,deg,B,wmax,chunks", [
+    (1, 2, 0, 3, 1, [40]), (31, 3, 3, 2, 1, [40]), (33, 8, 8, 5, 3, [40]), (1025, 3, 4, 9, 1, [9, 3, 12, 16]),
+    (1024, 5, 6, 3, 100, [40]), (4096, 8, 3, 2, 1, [40]), (5120, 6, 3, 2, 2, [40]), (8192, 4, 3, 2, 1, [40]),
+    (10240, 2, 5, 200, 1, [40]), (10240, 3, 4, 160, 7, [25, 15]), (4096, 7, 3, 2, 1, [13, 27])])
+def test_maxk_restart_runs_equal_the_row_wise_ones(n, k, deg, B, wmax, chunks):
+    rng = np.random.default_rng(n + k)
+    m = n * deg // 2
+    a, b = rng.integers(0, n, m), rng.integers(0, n, m)
+    keep = (a != b) & (a % 13 != 5) & (b % 13 != 5)      # some isolated vertices
+    edges = (a[keep], b[keep], rng.integers(1, wmax + 1, int(keep.sum())) * rng.choice([-1, 1], int(keep.sum())))
+    prm = S.params(B, 35, 0.1, 0.01, 1.0, eval_every=7, seed=3)   # evaluations at 7, .., 35 and past T at 42, ..
+    lr, rows = _run(n, edges, k, prm, chunks, S.EVAL_MODE_BESIDE)
+    lo, own = _run(n, edges, k, prm, chunks, S.EVAL_MODE_RULE)
+    for x, y in zip(own, rows):
+        assert np.array_equal(x, y)
+    assert lo < lr
