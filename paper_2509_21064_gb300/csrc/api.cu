@@ -75,6 +75,11 @@ void dfree(T*& p, cudaStream_t s) {
 
 }  // namespace
 
+// Blocks of K iterations a call must still have before it for a graph to be captured: capture and
+// instantiation take 100-200 us of host time, a directly launched block of ten grouped launches 25 us, and
+// the host stays ahead of the device either way.
+constexpr int64_t GRAPH_MIN_BLOCKS = 6;
+
 struct sbo_problem {
   int64_t n = 0;
   int fmt = FMT_DENSE;
@@ -1151,13 +1156,35 @@ sbo_status sbo_create_dense_i8(int64_t n, const int8_t* Q, const int32_t* c, int
   return create_dense_impl(n, Q, 1, c, precision, stream, out);
 }
 
+// Entries (i, j) of a sparse matrix by row, then column: counted into rows, then each (short) row sorted.
+struct Trip { int32_t i, j; int64_t v; };
+static void sort_by_row(int64_t n, std::vector<Trip>& tr) try {
+  std::vector<size_t> at((size_t)n + 1, 0);
+  for (const Trip& t : tr) ++at[(size_t)t.i + 1];
+  for (int64_t i = 0; i < n; ++i) at[(size_t)i + 1] += at[(size_t)i];
+  std::vector<size_t> next(at.begin(), at.end() - 1);
+  std::vector<Trip> out(tr.size());
+  for (const Trip& t : tr) out[next[(size_t)t.i]++] = t;
+  for (int64_t i = 0; i < n; ++i)
+    std::sort(out.begin() + (int64_t)at[(size_t)i], out.begin() + (int64_t)at[(size_t)i + 1],
+              [](const Trip& a, const Trip& b) { return a.j < b.j; });
+  tr.swap(out);
+} catch (const std::bad_alloc&) {   // no room for the copy: in place
+  std::sort(tr.begin(), tr.end(), [](const Trip& a, const Trip& b) { return a.i != b.i ? a.i < b.i : a.j < b.j; });
+}
+
 // The restart-resident structure in one device buffer: group streams (16-byte groups), c' exact, then the
 // 4-byte tables and the group counts.
 static sbo_status upload_restart(sbo_problem* p, const CsrRestartHost& rh) {
   const size_t b_ent = rh.ent.size() * 4, b_c64 = rh.cpp64.size() * 8, b_ws = rh.wstart.size() * 4,
                b_perm = rh.perm.size() * 4, b_pos = rh.pos.size() * 4, b_cp = rh.cpp.size() * 4,
                b_w = rh.ngroups.size();
-  std::vector<uint8_t> img(b_ent + b_c64 + b_ws + b_perm + b_pos + b_cp + b_w);
+  std::vector<uint8_t> img;
+  try {
+    img.resize(b_ent + b_c64 + b_ws + b_perm + b_pos + b_cp + b_w);
+  } catch (const std::bad_alloc&) {
+    return fail(SBO_ENOMEM, "host allocation failed");
+  }
   size_t off = 0;
   auto put = [&](const void* src, size_t bytes) {
     std::memcpy(img.data() + off, src, bytes);
@@ -1203,7 +1230,6 @@ sbo_status sbo_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const i
   std::vector<int64_t> cp(n, 0);
   if (c)
     for (int64_t i = 0; i < n; ++i) cp[i] = c[i];
-  struct Trip { int32_t i, j; int64_t v; };
   std::vector<Trip> tr;
   tr.reserve((size_t)2 * nnz);
   for (int64_t i = 0; i < n; ++i)
@@ -1214,7 +1240,7 @@ sbo_status sbo_create_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const i
       tr.push_back({(int32_t)i, j, (int64_t)val[e]});
       tr.push_back({j, (int32_t)i, (int64_t)val[e]});
     }
-  std::sort(tr.begin(), tr.end(), [](const Trip& a, const Trip& b) { return a.i != b.i ? a.i < b.i : a.j < b.j; });
+  sort_by_row(n, tr);
   std::vector<int32_t> rp(n + 1, 0), cc;
   std::vector<int64_t> vv;
   cc.reserve(tr.size());
@@ -1313,7 +1339,6 @@ sbo_status sbo_create_maxkcut(int64_t n, int64_t m, const int32_t* ei, const int
   if (m < 0 || (m > 0 && (!ei || !ej || !w))) return fail(SBO_EINVAL, "m must be >= 0 and the edge arrays non-NULL");
   if (k < 2 || k > 8) return fail(SBO_EINVAL, "k must be in [2, 8]");
   // W symmetric: both directions of every edge, duplicates summed, zero sums dropped
-  struct Trip { int32_t i, j; int64_t v; };
   std::vector<Trip> tr;
   tr.reserve((size_t)2 * m);
   for (int64_t e = 0; e < m; ++e) {
@@ -1323,7 +1348,7 @@ sbo_status sbo_create_maxkcut(int64_t n, int64_t m, const int32_t* ei, const int
     tr.push_back({a, b, (int64_t)w[e]});
     tr.push_back({b, a, (int64_t)w[e]});
   }
-  std::sort(tr.begin(), tr.end(), [](const Trip& x, const Trip& y) { return x.i != y.i ? x.i < y.i : x.j < y.j; });
+  sort_by_row(n, tr);
   std::vector<int32_t> rp(n + 1, 0), cc;
   std::vector<float> vv;
   std::vector<int64_t> rowabs(n, 0);
@@ -2262,9 +2287,7 @@ sbo_status group_start_tile(sbo_group* g, const sbo_gda_params* prms, int tile_n
       return fail(SBO_EINVAL, "members of a group share iters and eval_every");
   }
   group_free_graphs(g);
-  if (g->d_insts || g->d_commit) cudaStreamSynchronize(g->stream);
-  if (g->d_insts) { cudaFree(g->d_insts); g->d_insts = nullptr; }
-  if (g->d_commit) { cudaFree(g->d_commit); g->d_commit = nullptr; }
+  if (g->d_insts || g->d_commit) cudaStreamSynchronize(g->stream);   // the tables are rewritten below
   g->started = false;
   // start every member on the group's tile width, then build the instance table
   for (size_t k = 0; k < cnt; ++k) {
@@ -2275,7 +2298,7 @@ sbo_status group_start_tile(sbo_group* g, const sbo_gda_params* prms, int tile_n
     p->opt_split_k = 0;
     sbo_status st = sbo_gda_start(p, &prms[k], nullptr);
     if (st != SBO_OK) return st;
-    SBO_CUDA(cudaStreamSynchronize(p->stream));
+    if (p->stream != g->stream) SBO_CUDA(cudaStreamSynchronize(p->stream));
   }
   g->order.resize(cnt);
   for (size_t k = 0; k < cnt; ++k) g->order[k] = (int)k;
@@ -2307,7 +2330,7 @@ sbo_status group_start_tile(sbo_group* g, const sbo_gda_params* prms, int tile_n
   }
   g->num_tiles = tiles;
   g->tile_n = tile_n;
-  SBO_CUDA(cudaMalloc(&g->d_insts, sizeof(TcInst) * cnt));
+  if (!g->d_insts) SBO_CUDA(cudaMalloc(&g->d_insts, sizeof(TcInst) * cnt));
   SBO_CUDA(cudaMemcpy(g->d_insts, tab.data(), sizeof(TcInst) * cnt, cudaMemcpyHostToDevice));
   std::vector<CommitArgs> ctab(cnt);
   g->max_n = g->max_B = 0;
@@ -2316,7 +2339,7 @@ sbo_status group_start_tile(sbo_group* g, const sbo_gda_params* prms, int tile_n
     g->max_n = std::max<int64_t>(g->max_n, g->members[k]->n);
     g->max_B = std::max<int64_t>(g->max_B, g->members[k]->B);
   }
-  SBO_CUDA(cudaMalloc(&g->d_commit, sizeof(CommitArgs) * cnt));
+  if (!g->d_commit) SBO_CUDA(cudaMalloc(&g->d_commit, sizeof(CommitArgs) * cnt));
   SBO_CUDA(cudaMemcpy(g->d_commit, ctab.data(), sizeof(CommitArgs) * cnt, cudaMemcpyHostToDevice));
   g->T = prms[0].iters;
   g->K = prms[0].eval_every;
@@ -2355,13 +2378,31 @@ sbo_status sbo_group_create(int32_t count, sbo_problem* const* problems, void* s
 }
 
 // Tile width of a group: the one given, or (0) the fastest of the candidates, each timed on the
-// group's own instance table over a few grouped update launches.
+// group's own instance table over a few grouped update launches.  The decision is kept per device and
+// member sizes like the others, so that a later start does not start every member four times (8
+// members, n 500-3,000: 3.3 of 4.9 ms of a 30-iteration run).
 sbo_status sbo_group_start(sbo_group* g, const sbo_gda_params* prms) {
   g_last_error.clear();
   if (!g || !prms) return fail(SBO_EINVAL, "group or params is NULL");
   if (g->opt_tile_n != 0) return group_start_tile(g, prms, g->opt_tile_n);
+  static std::mutex mu;
+  static std::map<std::string, int> cache;
+  std::ostringstream name;
+  name << "grp1:" << tune_device(g->members[0]);
   int max_B = 1;
-  for (size_t k = 0; k < g->members.size(); ++k) max_B = std::max(max_B, prms[k].restarts);
+  for (size_t k = 0; k < g->members.size(); ++k) {
+    max_B = std::max(max_B, prms[k].restarts);
+    name << ":" << g->members[k]->n << "x" << prms[k].restarts;
+  }
+  const std::string key = name.str();
+  int known = 0;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find(key);
+    if (it != cache.end()) known = it->second;
+    else if (tune_cache_lookup(key, &known, [](int v) { return v == 64 || v == 128 || v == 256; })) cache[key] = known;
+  }
+  if (known) return group_start_tile(g, prms, known);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   SBO_CUDA(cudaEventCreate(&e0));
   SBO_CUDA(cudaEventCreate(&e1));
@@ -2388,6 +2429,11 @@ sbo_status sbo_group_start(sbo_group* g, const sbo_gda_params* prms) {
   if (st != SBO_OK) return st;
   st = read_err(g->members[0]);
   if (st != SBO_OK) return st;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    cache[key] = best;
+    tune_cache_store(key, best);
+  }
   return group_start_tile(g, prms, best);   // fresh state on the chosen width
 }
 
@@ -2403,7 +2449,9 @@ sbo_status sbo_group_run(sbo_group* g, int64_t iters) {
     const int64_t stop = std::min(nx, t_end);
     const int64_t steps = stop - g->t;
     const bool eval_here = stop == nx;
-    if (g->opt_graph && eval_here && steps == g->K && g->t % g->K == 0 && g->t_last_eval == g->t) {
+    // (capturing a block costs about as much as launching five: worth it only when more are to come)
+    if (g->opt_graph && eval_here && steps == g->K && g->t % g->K == 0 && g->t_last_eval == g->t &&
+        (g->gexec[g->cur] || (t_end - g->t) / g->K > GRAPH_MIN_BLOCKS)) {
       const int par = g->cur;
       if (!g->gexec[par]) {
         sbo_status st = group_capture(g, par);

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <new>
 
 namespace sbo {
 namespace {
@@ -180,7 +181,7 @@ static void place_lanes(int64_t n, const int32_t* rp, const int32_t* col, int BK
   }
 }
 
-bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
+static bool build_layout(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
                        int warps, int bank_lanes, int shift, CsrRestartHost* out) {
   if (n < 1 || n > 20 * RST_THREADS) return false;
   int maxd = 0;
@@ -266,6 +267,15 @@ bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const i
   out->shape.groups = groups;
   out->shape.max_groups = std::max(1, (maxd + 3) / 4);
   return true;
+}
+
+bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
+                       int warps, int bank_lanes, int shift, CsrRestartHost* out) {
+  try {
+    return build_layout(n, rp, col, val, cp, warps, bank_lanes, shift, out);
+  } catch (const std::bad_alloc&) {
+    return false;   // the row-wise kernels need no layout
+  }
 }
 
 bool csr_restart_fits(const CsrRestartShape& sh, int R) {
