@@ -11,6 +11,8 @@
 #include <map>
 #include <mutex>
 #include <sstream>
+#include <system_error>
+#include <thread>
 #include <tuple>
 #include <cmath>
 #include <cstring>
@@ -71,6 +73,92 @@ template <typename T>
 void dfree(T*& p, cudaStream_t s) {
   if (p) cudaFreeAsync(p, s);
   p = nullptr;
+}
+
+// Small results come back through pinned memory, so that several of them and the error word share one
+// synchronisation (each copy into pageable memory is one of its own, 8-10 us).  Buffers are borrowed from
+// a pool of the process: at most eight are kept, any thread may take one, and one that does not fit or
+// cannot be had leaves the caller to copy directly.
+class PinnedLoan {
+ public:
+  static constexpr size_t BYTES = 64 << 10;
+  explicit PinnedLoan(size_t need) {
+    if (need > BYTES) return;
+    {
+      std::lock_guard<std::mutex> lock(mu());
+      if (!kept().empty()) {
+        mem_ = kept().back();
+        kept().pop_back();
+      }
+    }
+    if (!mem_ && cudaHostAlloc(&mem_, BYTES, cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      mem_ = nullptr;
+    }
+  }
+  ~PinnedLoan() {
+    if (!mem_) return;
+    {
+      std::lock_guard<std::mutex> lock(mu());
+      if (kept().size() < 8) {
+        kept().push_back(mem_);   // (within the capacity reserved below)
+        return;
+      }
+    }
+    cudaFreeHost(mem_);
+  }
+  PinnedLoan(const PinnedLoan&) = delete;
+  PinnedLoan& operator=(const PinnedLoan&) = delete;
+  // copies [src, src + bytes) of the device on s; *at gets its place here (valid after synchronising s)
+  cudaError_t fetch(const void* src, size_t bytes, cudaStream_t s, const void** at) {
+    void* dst = static_cast<char*>(mem_) + used_;
+    used_ += (bytes + 15) / 16 * 16;
+    *at = dst;
+    return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s);
+  }
+  explicit operator bool() const { return mem_ != nullptr; }
+
+ private:
+  static std::mutex& mu() {
+    static std::mutex m;
+    return m;
+  }
+  static std::vector<void*>& kept() {
+    static std::vector<void*>* v = [] {
+      auto* w = new std::vector<void*>();   // never freed: outlives every thread's last loan
+      w->reserve(8);
+      return w;
+    }();
+    return *v;
+  }
+  void* mem_ = nullptr;
+  size_t used_ = 0;
+};
+
+// Faults in the pages of a large output buffer with several threads while the device prepares its
+// contents: a copy into freshly mapped memory otherwise stops at every page (41 MB of iterates: 18 ms of
+// a 20 ms call).  The contents are left as they are.
+void touch_pages(void* dst, size_t bytes) {
+  constexpr size_t PAGE = 4096, SHARE = 1 << 20, LEAST = 16 << 20;   // (5 MB: the threads cost more than the faults)
+  const size_t threads = std::min<size_t>({8, bytes / (2 * SHARE), std::thread::hardware_concurrency()});
+  cudaPointerAttributes attr;
+  if (bytes < LEAST || threads < 2 || cudaPointerGetAttributes(&attr, dst) != cudaSuccess || attr.type != cudaMemoryTypeUnregistered) {
+    cudaGetLastError();   // small, or not plain host memory
+    return;
+  }
+  auto touch = [=](size_t k) {
+    volatile char* p = static_cast<volatile char*>(dst);
+    const size_t end = bytes / threads * (k + 1);
+    for (size_t at = bytes / threads * k; at < end; at += PAGE) p[at] = p[at];
+  };
+  std::thread pool[8];
+  size_t started = 1;
+  try {
+    for (; started < threads; ++started) pool[started] = std::thread(touch, started);
+  } catch (const std::system_error&) {   // no more threads: the copy faults in the rest itself
+  }
+  touch(0);
+  for (size_t k = 1; k < started; ++k) pool[k].join();
 }
 
 }  // namespace
@@ -989,9 +1077,8 @@ sbo_status check_params(const sbo_gda_params* q) {
   return SBO_OK;
 }
 
-sbo_status read_err(sbo_problem* p) {
-  uint32_t w = 0;
-  SBO_CUDA(cudaMemcpy(&w, p->err, sizeof(w), cudaMemcpyDeviceToHost));
+// The status of error word w (cleared on the device when raised).
+sbo_status report_err(sbo_problem* p, uint32_t w) {
   if (w) {
     SBO_CUDA(cudaMemset(p->err, 0, sizeof(uint32_t)));
     // a launch that gave up may have left the grid barrier's words raised
@@ -1000,6 +1087,45 @@ sbo_status read_err(sbo_problem* p) {
     return fail(SBO_EDEVICE, "a device-side bounds check failed (input out of range)");
   }
   return SBO_OK;
+}
+
+sbo_status read_err(sbo_problem* p) {
+  uint32_t w = 0;
+  SBO_CUDA(cudaMemcpy(&w, p->err, sizeof(w), cudaMemcpyDeviceToHost));
+  return report_err(p, w);
+}
+
+// Up to three small device arrays into host buffers (null: skipped), ordered after the work on the
+// problem's stream, with the error word: one synchronisation where pinned memory is to be had.
+struct Fetch { void* dst; const void* src; size_t bytes; };
+sbo_status fetch_results(sbo_problem* p, std::initializer_list<Fetch> list) {
+  cudaStream_t s = p->stream;
+  size_t need = 16;
+  for (const Fetch& f : list) need += f.dst ? f.bytes + 16 : 0;
+  PinnedLoan pin(need);
+  if (!pin) {
+    SBO_CUDA(cudaStreamSynchronize(s));
+    for (const Fetch& f : list)
+      if (f.dst && f.bytes) SBO_CUDA(cudaMemcpy(f.dst, f.src, f.bytes, cudaMemcpyDeviceToHost));
+    return read_err(p);
+  }
+  const void *w = nullptr, *at[3] = {};
+  cudaError_t e = cudaSuccess;
+  int k = 0;
+  for (const Fetch& f : list) {
+    if (e == cudaSuccess && f.dst && f.bytes) e = pin.fetch(f.src, f.bytes, s, &at[k]);
+    ++k;
+  }
+  if (e == cudaSuccess) e = pin.fetch(p->err, sizeof(uint32_t), s, &w);
+  const cudaError_t e2 = cudaStreamSynchronize(s);   // also before the buffer is given back
+  if (e == cudaSuccess) e = e2;
+  if (e != cudaSuccess) return cuda_fail(e, "read-back");
+  k = 0;
+  for (const Fetch& f : list) {
+    if (at[k]) std::memcpy(f.dst, at[k], f.bytes);
+    ++k;
+  }
+  return report_err(p, *static_cast<const uint32_t*>(w));
 }
 
 }  // namespace
@@ -1783,8 +1909,7 @@ sbo_status sbo_sync(sbo_problem* p) {
   if (!p) return fail(SBO_EINVAL, "problem is NULL");
   sbo_status st = flush_pending(p);
   if (st != SBO_OK) return st;
-  SBO_CUDA(cudaStreamSynchronize(p->stream));
-  return read_err(p);
+  return fetch_results(p, {});
 }
 
 sbo_status sbo_gda(sbo_problem* p, const sbo_gda_params* prm) {
@@ -1880,9 +2005,7 @@ sbo_status sbo_best(sbo_problem* p, uint8_t* x_out, int64_t* F_out, int64_t* ite
   ++p->launches;
   if (e != cudaSuccess) return cuda_fail(e, "best selection");
   long long h[3];
-  SBO_CUDA(cudaMemcpyAsync(h, p->sel, sizeof(h), cudaMemcpyDeviceToHost, s));
-  SBO_CUDA(cudaStreamSynchronize(s));
-  sbo_status st = read_err(p);
+  sbo_status st = fetch_results(p, {{h, p->sel, sizeof(h)}});
   if (st != SBO_OK) return st;
   if (h[1] < 0 || h[2] < 0 || h[2] >= p->B) return fail(SBO_EDEVICE, "inconsistent best record");
   if (F_out) *F_out = h[0];
@@ -1914,10 +2037,7 @@ sbo_status sbo_restart_best(sbo_problem* p, int64_t* F, int64_t* t) {
   if (!p->started) return fail(SBO_ENOTREADY, "sbo_gda_start has not been called");
   sbo_status st = flush_pending(p);
   if (st != SBO_OK) return st;
-  SBO_CUDA(cudaStreamSynchronize(p->stream));
-  if (F) SBO_CUDA(cudaMemcpy(F, p->bestF, sizeof(int64_t) * p->B, cudaMemcpyDeviceToHost));
-  if (t) SBO_CUDA(cudaMemcpy(t, p->bestT, sizeof(int64_t) * p->B, cudaMemcpyDeviceToHost));
-  return read_err(p);
+  return fetch_results(p, {{F, p->bestF, sizeof(int64_t) * p->B}, {t, p->bestT, sizeof(int64_t) * p->B}});
 }
 
 sbo_status sbo_state(sbo_problem* p, float* X, float* Y) {
@@ -1925,33 +2045,37 @@ sbo_status sbo_state(sbo_problem* p, float* X, float* Y) {
   if (!p) return fail(SBO_EINVAL, "problem is NULL");
   if (!p->started) return fail(SBO_ENOTREADY, "sbo_gda_start has not been called");
   cudaStream_t s = p->stream;
-  float* tmp = nullptr;
   const int kx = p->kernel == KER_MAXK ? p->kparts : 1;   // Max-k-Cut: X_:,i has k entries
-  SBO_CUDA(dalloc(&tmp, (size_t)p->B * p->n * kx, s));
+  const size_t nx = X ? (size_t)p->B * p->n * kx : 0, ny = Y && !p->single ? (size_t)p->B * p->n : 0;
+  float* tmp = nullptr;
+  SBO_CUDA(dalloc(&tmp, nx + ny, s));
   cudaError_t e = cudaSuccess;
-  if (X) {
-    if (p->kernel == KER_MAXK)
-      e = launch_maxk_gather(static_cast<const float*>(p->Xop[p->cur]), (int)p->n, kx, p->B, p->ld, tmp, s);
-    else
-      e = gather_x(p, tmp, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(X, tmp, sizeof(float) * p->B * p->n * kx, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (nx)
+    e = p->kernel == KER_MAXK
+            ? launch_maxk_gather(static_cast<const float*>(p->Xop[p->cur]), (int)p->n, kx, p->B, p->ld, tmp, s)
+            : gather_x(p, tmp, s);
+  if (ny && e == cudaSuccess)
+    e = p->rst_home ? launch_restart_gather(p->rst, p->rY, (int)p->n, p->B, p->rst_R, tmp + nx, s)
+                    : launch_gather_state(p->Y, (int)p->n, p->B, p->ld, p->layout, tmp + nx, s);
+  if (e == cudaSuccess) {   // while the kernels run
+    if (nx) touch_pages(X, sizeof(float) * nx);
+    if (ny) touch_pages(Y, sizeof(float) * ny);
   }
-  if (Y && e == cudaSuccess && p->single) {
+  if (nx && e == cudaSuccess) e = cudaMemcpyAsync(X, tmp, sizeof(float) * nx, cudaMemcpyDeviceToHost, s);
+  if (ny && e == cudaSuccess) e = cudaMemcpyAsync(Y, tmp + nx, sizeof(float) * ny, cudaMemcpyDeviceToHost, s);
+  std::vector<float> mu;
+  if (Y && p->single && e == cudaSuccess) {
     // one dual per restart: every coordinate of restart r reports mu_r
-    std::vector<float> mu((size_t)p->B);
+    mu.resize((size_t)p->B);
     e = cudaMemcpyAsync(mu.data(), p->mu, sizeof(float) * p->B, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (int64_t r = 0; r < p->B && e == cudaSuccess; ++r) std::fill(Y + r * p->n, Y + (r + 1) * p->n, mu[r]);
-  } else if (Y && e == cudaSuccess) {
-    e = p->rst_home ? launch_restart_gather(p->rst, p->rY, (int)p->n, p->B, p->rst_R, tmp, s)
-                    : launch_gather_state(p->Y, (int)p->n, p->B, p->ld, p->layout, tmp, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(Y, tmp, sizeof(float) * p->B * p->n, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
+  sbo_status st = SBO_OK;
+  if (e == cudaSuccess) st = fetch_results(p, {});   // synchronises
+  else cudaStreamSynchronize(s);
   dfree(tmp, s);
   if (e != cudaSuccess) return cuda_fail(e, "state read-back");
-  return read_err(p);
+  for (size_t r = 0; r < mu.size() && st == SBO_OK; ++r) std::fill(Y + r * p->n, Y + (r + 1) * p->n, mu[r]);
+  return st;
 }
 
 sbo_status sbo_gradient(sbo_problem* p, float* G) {
@@ -1978,13 +2102,11 @@ sbo_status sbo_trace(sbo_problem* p, int64_t* minF, int64_t cap, int64_t* count)
   if (!p->started) return fail(SBO_ENOTREADY, "sbo_gda_start has not been called");
   sbo_status st = flush_pending(p);
   if (st != SBO_OK) return st;
-  SBO_CUDA(cudaStreamSynchronize(p->stream));
+  const int64_t m = std::max<int64_t>(0, std::min<int64_t>(std::min<int64_t>(p->n_evals_host, cap), p->trace_cap));
   long long ne = 0;
-  SBO_CUDA(cudaMemcpy(&ne, p->n_evals, sizeof(ne), cudaMemcpyDeviceToHost));
+  st = fetch_results(p, {{&ne, p->n_evals, sizeof(ne)}, {m > 0 ? minF : nullptr, p->trace, sizeof(int64_t) * m}});
   if (count) *count = ne;
-  const int64_t m = std::min<int64_t>(std::min<int64_t>(ne, cap), p->trace_cap);
-  if (minF && m > 0) SBO_CUDA(cudaMemcpy(minF, p->trace, sizeof(int64_t) * m, cudaMemcpyDeviceToHost));
-  return read_err(p);
+  return st;
 }
 
 sbo_status sbo_lagrangian(sbo_problem* p, int32_t B, const float* X_dev, const float* Y_dev, const float* gout_dev,
