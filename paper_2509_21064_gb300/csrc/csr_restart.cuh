@@ -29,6 +29,8 @@
 // n = 2,000, B = 256 5.5 -> 1.9 us; 100 x 100 torus, E4M3, B = 512 16.5 -> 8.2 us; 4-regular n = 20,000,
 // B = 512 38.6 -> 20.4 us.
 #pragma once
+#include <type_traits>
+
 #include "sbo_internal.h"
 
 namespace sbo {
@@ -179,8 +181,10 @@ __device__ __forceinline__ void add_bits4(const uint8_t* bb, const G& c, uint32_
   }
 }
 
-// One iteration's work on one vertex after its neighbour sums: update of R restarts.
-template <int R>
+// One iteration's work on one vertex after its neighbour sums: update of R restarts.  CHECK false: no y of
+// the CTA can reach 0 in this stretch of iterations, so the perturbation rule (which needs y <= 0)
+// cannot apply and its test is left out.
+template <int R, bool CHECK>
 __device__ __forceinline__ void update(const EpiArgs& a, const float* xc, float* xn, const float (&acc)[R], float cp,
                                        float (&y)[R]) {
   float xo[R], xv[R];
@@ -199,9 +203,11 @@ __device__ __forceinline__ void update(const EpiArgs& a, const float* xc, float*
     const float gx = g_val(x, G_QUAD);
     const float d = acc[r] + cp + y[r] * g_der(x, G_QUAD);
     // pdbo_update (common.cuh) with the projection as a saturation: the same value
-    const bool stagnating = fabsf(x - 0.5f) <= a.delta && fabsf(d) <= a.grad_tol && y[r] <= 0.0f;
     xv[r] = __saturatef(x - a.alpha * d);
-    if (stagnating) xv[r] = x <= 0.5f ? 0.5f - a.delta : 0.5f + a.delta;
+    if (CHECK) {
+      const bool stagnating = fabsf(x - 0.5f) <= a.delta && fabsf(d) <= a.grad_tol && y[r] <= 0.0f;
+      if (stagnating) xv[r] = x <= 0.5f ? 0.5f - a.delta : 0.5f + a.delta;
+    }
     y[r] = y[r] + a.beta * gx;
   }
   st_vec<R>(xn, xv);
@@ -227,6 +233,8 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
   __shared__ long long red[RST_WARPS][R];
   __shared__ long long s_bestF[R], s_bestT[R];
   __shared__ uint32_t s_improved, s_any;
+  __shared__ float ymin_w[RST_WARPS];
+  __shared__ volatile float s_ymin;   // a lower bound of this unit's y
   __shared__ int s_ticket;
   // progress of the chunk, kept here and not in registers, which the state needs: t done and t at its end
   __shared__ volatile int64_t s_t, s_end;
@@ -295,6 +303,7 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
     }
     if (threadIdx.x == 0) {
       s_any = 0u;
+      s_ymin = -1.0f;
       s_ticket = c * P.units + u;
       s_t = P.t0 + (int64_t)c * P.chunk_len;
       s_end = P.t0 + min((int64_t)(c + 1) * P.chunk_len, (int64_t)P.iters);
@@ -323,38 +332,70 @@ __global__ void __launch_bounds__(RST_THREADS, 1) k_csr_restart(const __grid_con
     const float* xc = xs;
     float* xn = xs + nx_pos * R;
     while (s_t < s_end) {   // stretches of iterations that end at an evaluation point or with the chunk
-      for (int left = (int)min(until_eval(s_t), (int64_t)(s_end - s_t)); left > 0; --left) {
-        const G* st = (P.ent_in_smem ? ent_s : ent_g) + stream0;
-        G nx[AHEAD];   // groups read ahead (the streams end in RST_SPARE spare groups)
+      const int stretch = (int)min(until_eval(s_t), (int64_t)(s_end - s_t));
+      auto iterate = [&](auto check) {
+        for (int left = stretch; left > 0; --left) {
+          const G* st = (P.ent_in_smem ? ent_s : ent_g) + stream0;
+          G nx[AHEAD];   // groups read ahead (the streams end in RST_SPARE spare groups)
 #pragma unroll
-        for (int d = 0; d < AHEAD; ++d, st += 32) nx[d] = *st;
+          for (int d = 0; d < AHEAD; ++d, st += 32) nx[d] = *st;
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          if (warp + q * RST_WARPS >= P.slices) break;   // no later slice either
-          const int p = p0 + q * RST_THREADS;
-          float acc[R];
+          for (int q = 0; q < Q; ++q) {
+            if (warp + q * RST_WARPS >= P.slices) break;   // no later slice either
+            const int p = p0 + q * RST_THREADS;
+            float acc[R];
 #pragma unroll
-          for (int r = 0; r < R; ++r) acc[r] = 0.0f;
-          const int ng = ONE ? 1 : ngr[warp + q * RST_WARPS];
-          for (int g = 0; g < ng; ++g) {
-            const G e = nx[0];
+            for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+            const int ng = ONE ? 1 : ngr[warp + q * RST_WARPS];
+            for (int g = 0; g < ng; ++g) {
+              const G e = nx[0];
 #pragma unroll
-            for (int d = 0; d + 1 < AHEAD; ++d) nx[d] = nx[d + 1];
-            nx[AHEAD - 1] = *st;
-            st += 32;
-            gather4<R, BF16, BASE>(xc, e, P.wbits, acc);
+              for (int d = 0; d + 1 < AHEAD; ++d) nx[d] = nx[d + 1];
+              nx[AHEAD - 1] = *st;
+              st += 32;
+              gather4<R, BF16, BASE>(xc, e, P.wbits, acc);
+            }
+            const float cp = !PACK ? cps[PACK ? 0 : q]
+                                   : __uint_as_float((q & 1) ? cpk[PACK ? q / 2 : 0] & 0xffff0000u : cpk[PACK ? q / 2 : 0] << 16);
+            update<R, decltype(check)::value>(a, xc + p * R, xn + p * R, acc, cp, y[q]);
           }
-          const float cp = !PACK ? cps[PACK ? 0 : q]
-                                 : __uint_as_float((q & 1) ? cpk[PACK ? q / 2 : 0] & 0xffff0000u : cpk[PACK ? q / 2 : 0] << 16);
-          update<R>(a, xc + p * R, xn + p * R, acc, cp, y[q]);
+          {
+            float* t = const_cast<float*>(xc);
+            xc = xn;
+            xn = t;
+          }
+          __syncthreads();
         }
-        {
-          float* t = const_cast<float*>(xc);
-          xc = xn;
-          xn = t;
+      };
+      // y falls by at most beta / 4 and a rounding of y an iteration (g >= -1/4): while a lower bound of the
+      // CTA's y stays above 0 for the whole stretch the perturbation rule is out of reach
+      auto after = [&](float ymin) { return ymin - (float)stretch * (0.2501f * a.beta + 1.2e-7f * fabsf(ymin)); };
+      if (!(after(s_ymin) > 0.0f)) {   // near 0, or not known yet: the actual minimum
+        float m = 3.4e38f;
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+          if (warp + q * RST_WARPS < P.slices && p0 + q * RST_THREADS < n)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+              if (s_ticket % P.units * R + r < a.B) m = fminf(m, y[q][r]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) ymin_w[warp] = m;
+        __syncthreads();
+        if (warp == 0) {
+          m = ymin_w[lane];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+          if (lane == 0) s_ymin = m;
         }
         __syncthreads();
       }
+      const float left_y = after(s_ymin);
+      const bool clear = left_y > 0.0f;
+      __syncthreads();   // every thread has read s_ymin
+      if (threadIdx.x == 0) s_ymin = left_y;
+      if (clear) iterate(std::false_type());
+      else iterate(std::true_type());
       const int64_t t = min(s_t + until_eval(s_t), (int64_t)s_end);
       const bool is_eval = t - s_t == until_eval(s_t);
       __syncthreads();   // every thread has read s_t
