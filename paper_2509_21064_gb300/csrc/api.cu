@@ -11,8 +11,6 @@
 #include <map>
 #include <mutex>
 #include <sstream>
-#include <system_error>
-#include <thread>
 #include <tuple>
 #include <cmath>
 #include <cstring>
@@ -134,32 +132,6 @@ class PinnedLoan {
   void* mem_ = nullptr;
   size_t used_ = 0;
 };
-
-// Faults in the pages of a large output buffer with several threads while the device prepares its
-// contents: a copy into freshly mapped memory otherwise stops at every page (41 MB of iterates: 18 ms of
-// a 20 ms call).  The contents are left as they are.
-void touch_pages(void* dst, size_t bytes) {
-  constexpr size_t PAGE = 4096, SHARE = 1 << 20, LEAST = 16 << 20;   // (5 MB: the threads cost more than the faults)
-  const size_t threads = std::min<size_t>({8, bytes / (2 * SHARE), std::thread::hardware_concurrency()});
-  cudaPointerAttributes attr;
-  if (bytes < LEAST || threads < 2 || cudaPointerGetAttributes(&attr, dst) != cudaSuccess || attr.type != cudaMemoryTypeUnregistered) {
-    cudaGetLastError();   // small, or not plain host memory
-    return;
-  }
-  auto touch = [=](size_t k) {
-    volatile char* p = static_cast<volatile char*>(dst);
-    const size_t end = bytes / threads * (k + 1);
-    for (size_t at = bytes / threads * k; at < end; at += PAGE) p[at] = p[at];
-  };
-  std::thread pool[8];
-  size_t started = 1;
-  try {
-    for (; started < threads; ++started) pool[started] = std::thread(touch, started);
-  } catch (const std::system_error&) {   // no more threads: the copy faults in the rest itself
-  }
-  touch(0);
-  for (size_t k = 1; k < started; ++k) pool[k].join();
-}
 
 }  // namespace
 
@@ -2057,10 +2029,6 @@ sbo_status sbo_state(sbo_problem* p, float* X, float* Y) {
   if (ny && e == cudaSuccess)
     e = p->rst_home ? launch_restart_gather(p->rst, p->rY, (int)p->n, p->B, p->rst_R, tmp + nx, s)
                     : launch_gather_state(p->Y, (int)p->n, p->B, p->ld, p->layout, tmp + nx, s);
-  if (e == cudaSuccess) {   // while the kernels run
-    if (nx) touch_pages(X, sizeof(float) * nx);
-    if (ny) touch_pages(Y, sizeof(float) * ny);
-  }
   if (nx && e == cudaSuccess) e = cudaMemcpyAsync(X, tmp, sizeof(float) * nx, cudaMemcpyDeviceToHost, s);
   if (ny && e == cudaSuccess) e = cudaMemcpyAsync(Y, tmp + nx, sizeof(float) * ny, cudaMemcpyDeviceToHost, s);
   std::vector<float> mu;
