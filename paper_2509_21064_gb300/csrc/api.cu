@@ -69,7 +69,7 @@ cudaError_t dalloc(T** p, size_t count, cudaStream_t s) {
 }
 template <typename T>
 void dfree(T*& p, cudaStream_t s) {
-  if (p) cudaFreeAsync(p, s);
+  if (p) cudaFreeAsync((void*)p, s);
   p = nullptr;
 }
 
@@ -181,7 +181,10 @@ struct sbo_problem {
   int opt_eval_mode = 0;      // SBO_OPT_EVAL_MODE: 0 the rule (beside), 1 in line, 2 beside
   int64_t opt_timeout_us = 4000000;
   int64_t opt_steps_per_launch = 0;   // cluster split-K iterations per launch (0: 4,096)
-  // run
+  // run: the state of a run lies in one block, kept for the next start while it is large enough and not
+  // more than twice what is needed
+  char* arena = nullptr;
+  size_t arena_bytes = 0;
   bool started = false;
   sbo_gda_params prm{};
   int kernel = KER_AUTO, layout = LAYOUT_RN, op_type = OP_F32, tile_n = 0;
@@ -246,39 +249,25 @@ void free_run(sbo_problem* p) {
       if (set[k]) { cudaGraphExecDestroy(set[k]); set[k] = nullptr; }
   p->eval_pending = false;
   p->eval_fused = false;
-  dfree(p->Xm, p->stream);
-  dfree(p->Y, p->stream);
-  dfree(p->Gd, p->stream);
-  dfree(p->Xop[0], p->stream);
-  dfree(p->Xop[1], p->stream);
-  dfree(p->bits, p->stream);
-  dfree(p->bestF, p->stream);
-  dfree(p->bestT, p->stream);
-  dfree(p->evalF, p->stream);
-  dfree(p->trace, p->stream);
-  dfree(p->n_evals, p->stream);
-  dfree(p->t_last, p->stream);
-  dfree(p->sel, p->stream);
-  dfree(p->F2, p->stream);
-  dfree(p->bestBits, p->stream);
-  dfree(p->commit_ctr, p->stream);
-  dfree(p->mu, p->stream);
-  dfree(p->gpart, p->stream);
+  auto drop = [&](auto*& q) {   // parts of the block stay with it
+    const char* c = reinterpret_cast<const char*>(q);
+    if (c && p->arena && c >= p->arena && c < p->arena + p->arena_bytes) q = nullptr;
+    else dfree(q, p->stream);
+  };
+  drop(p->Xm); drop(p->Y); drop(p->Gd); drop(p->Xop[0]); drop(p->Xop[1]); drop(p->bits); drop(p->bestBits);
+  drop(p->bestF); drop(p->bestT); drop(p->evalF); drop(p->trace); drop(p->n_evals); drop(p->t_last); drop(p->sel);
+  drop(p->F2); drop(p->commit_ctr); drop(p->mu); drop(p->gpart);
+  drop(p->tc_ws); drop(p->tc_ctr); drop(p->tc_gbar); drop(p->csk_ws);
+  drop(p->rX); drop(p->rY); drop(p->rBest); drop(p->rst_sched);
   p->single = false;
-  dfree(p->tc_ws, p->stream);
-  dfree(p->tc_ctr, p->stream);
-  dfree(p->tc_gbar, p->stream);
-  dfree(p->csk_ws, p->stream);
-  dfree(p->rX, p->stream);
-  dfree(p->rY, p->stream);
-  dfree(p->rBest, p->stream);
-  dfree(p->rst_sched, p->stream);
   p->rst_home = false;
   p->started = false;
 }
 
 void free_all(sbo_problem* p) {
   free_run(p);
+  dfree(p->arena, p->stream);
+  p->arena_bytes = 0;
   dfree(p->A, p->stream);
   dfree(p->A16, p->stream);
   dfree(p->rowptr, p->stream);
@@ -1616,9 +1605,12 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   // min-F trace: one entry per evaluation up to T, plus slack for runs continued beyond T
   const int64_t evals_T = prm->iters / prm->eval_every + 2;
   p->trace_cap = std::min<int64_t>(evals_T, 1 << 20) + 4096;
-  auto al = [&](void** q, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMallocAsync(q, bytes ? bytes : 1, p->stream);
-  };
+  // The parts of the run's block: zeroed ones (padding never holds stale values) come first, so that one
+  // memset covers them.
+  struct Part { void** at; size_t bytes; bool zero; };
+  Part parts[32];
+  int n_parts = 0;
+  auto al = [&](void** q, size_t bytes, bool zero) { parts[n_parts++] = {q, (bytes + 255) / 256 * 256, zero}; };
   // A sparse run that goes restart by restart starts in that layout: the row-wise arrays are allocated
   // (and the row-wise form left to its rule or an earlier decision) only if a later call needs them.
   p->rst_R = 0;
@@ -1630,84 +1622,85 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   if (ker == KER_MAXK && restart_wanted(p) && maxk_restart_pays(p->rst.shape, p->n, p->nnz, p->kparts, p->B, p->sms))
     p->rst_R = 1;
   if (!home) {
-    if (need_master) al((void**)&p->Xm, xelems * 4);
-    al((void**)&p->Y, elems * 4);
-    if (p->opt_keep_grad) al((void**)&p->Gd, elems * 4);
+    if (need_master) al((void**)&p->Xm, xelems * 4, true);
+    al((void**)&p->Y, elems * 4, true);
+    if (p->opt_keep_grad) al((void**)&p->Gd, elems * 4, true);
     if (ker != KER_TINY) {
-      al(&p->Xop[0], xelems * op_elt * pieces);
-      al(&p->Xop[1], xelems * op_elt * pieces);
-      al(&p->bits, elems * (ker == KER_CSR ? 1 : op_elt));   // the sparse path keeps candidates as bytes
+      al(&p->Xop[0], xelems * op_elt * pieces, true);
+      al(&p->Xop[1], xelems * op_elt * pieces, true);
+      al(&p->bits, elems * (ker == KER_CSR ? 1 : op_elt), true);   // the sparse path keeps candidates as bytes
     }
-    al((void**)&p->bestBits, elems);
+    al((void**)&p->bestBits, elems, true);
+  } else {
+    const size_t npos = csr_restart_positions(p->rst.shape), rows = (size_t)p->B + CSR_RESTART_MAX_R - 1;
+    al((void**)&p->rX, rows * npos * 4, false);
+    al((void**)&p->rY, rows * npos * 4, false);
+    al((void**)&p->rBest, (size_t)p->B * npos, true);
+    al((void**)&p->rst_sched, ((size_t)p->B + 2) * 4, false);
   }
-  if (e == cudaSuccess && home) e = alloc_units(p);
-  al((void**)&p->bestF, sizeof(long long) * p->B);
-  al((void**)&p->bestT, sizeof(long long) * p->B);
-  al((void**)&p->evalF, sizeof(long long) * p->B);
-  al((void**)&p->F2, sizeof(unsigned long long) * p->B);
-  al((void**)&p->commit_ctr, sizeof(unsigned int));
+  al((void**)&p->F2, sizeof(unsigned long long) * p->B, true);
+  al((void**)&p->commit_ctr, sizeof(unsigned int), true);
+  al((void**)&p->n_evals, sizeof(long long), true);
+  al((void**)&p->t_last, sizeof(long long), true);
+  al((void**)&p->bestF, sizeof(long long) * p->B, false);
+  al((void**)&p->bestT, sizeof(long long) * p->B, false);
+  al((void**)&p->evalF, sizeof(long long) * p->B, false);
+  al((void**)&p->trace, sizeof(long long) * p->trace_cap, false);
+  al((void**)&p->sel, sizeof(long long) * 3, false);
   if (p->single) {
     // rows of partial sums the update kernel writes: 4 per 128 variables (tcgen05 kernels; CTA
     // pairs round up to 256), 1 per 64 variables (SIMT), 1 per block along the rows (CSR)
     p->gpart_rows = ker == KER_TC ? (p->n + 255) / 256 * 8 : ker == KER_SIMT ? (p->n + 63) / 64
                                                                              : csr_partial_rows(p->n, p->B);
     p->gpart_ld = round_up(p->B, 8);
-    al((void**)&p->mu, sizeof(float) * p->gpart_ld);
-    al((void**)&p->gpart, sizeof(float) * p->gpart_rows * p->gpart_ld);
+    al((void**)&p->mu, sizeof(float) * p->gpart_ld, false);
+    al((void**)&p->gpart, sizeof(float) * p->gpart_rows * p->gpart_ld, false);
   }
-  al((void**)&p->trace, sizeof(long long) * p->trace_cap);
-  al((void**)&p->n_evals, sizeof(long long));
-  al((void**)&p->t_last, sizeof(long long));
-  al((void**)&p->sel, sizeof(long long) * 3);
-  if (e != cudaSuccess) {
-    free_run(p);
-    return e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation of the run state failed")
-                                          : cuda_fail(e, "cudaMalloc");
-  }
-  cudaStream_t s = p->stream;
-  // zero every buffer so padding never holds stale values; sentinels for bests and trace
-  if (p->Xm) cudaMemsetAsync(p->Xm, 0, xelems * 4, s);
-  if (p->Y) cudaMemsetAsync(p->Y, 0, elems * 4, s);
-  if (p->Gd) cudaMemsetAsync(p->Gd, 0, elems * 4, s);
-  for (void* b : {p->Xop[0], p->Xop[1]})
-    if (b) cudaMemsetAsync(b, 0, xelems * op_elt * pieces, s);
-  if (p->bits) cudaMemsetAsync(p->bits, 0, elems * (ker == KER_CSR ? 1 : op_elt), s);
-  launch_fill_i64(p->bestF, p->B, LLONG_MAX, s);
-  launch_fill_i64(p->bestT, p->B, -1, s);
-  launch_fill_i64(p->trace, p->trace_cap, LLONG_MAX, s);
-  p->launches += 3;
-  cudaMemsetAsync(p->F2, 0, sizeof(unsigned long long) * p->B, s);
-  cudaMemsetAsync(p->commit_ctr, 0, sizeof(unsigned int), s);
-  if (p->bestBits) cudaMemsetAsync(p->bestBits, 0, elems, s);
-  cudaMemsetAsync(p->n_evals, 0, sizeof(long long), s);
-  cudaMemsetAsync(p->t_last, 0, sizeof(long long), s);
   if (ker == KER_TC) {
     // split-K workspace (sized for the widest tile): one partial tile per CTA, arrival counters
     // per tail tile slice
     if (p->opt_split_k >= 2) {
-      if ((e = dalloc(&p->tc_ws, (size_t)p->sms * 256 * 128, s)) != cudaSuccess ||
-          (e = dalloc(&p->tc_ctr, (size_t)p->sms * TC_WS_COUNTERS_PER_TILE, s)) != cudaSuccess) {
-        free_run(p);
-        return e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation of the split-K workspace failed")
-                                              : cuda_fail(e, "cudaMalloc");
-      }
-      cudaMemsetAsync(p->tc_ctr, 0, sizeof(int) * p->sms * TC_WS_COUNTERS_PER_TILE, s);
-    }
-    if ((e = dalloc(&p->tc_gbar, 3, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(p->tc_gbar, 0, 3 * sizeof(unsigned int), s)) != cudaSuccess) {
-      free_run(p);
-      return cuda_fail(e, "grid barrier words");
+      al((void**)&p->tc_ws, (size_t)p->sms * 256 * 128 * 4, false);
+      al((void**)&p->tc_ctr, sizeof(int) * p->sms * TC_WS_COUNTERS_PER_TILE, true);
     }
     // the cluster split-K kernel serves problems with at most sms / 2 tiles (fewest at width 256),
     // on CTA pairs at most sms / 4 tiles of 256 x 256
     if ((p->tc_split || p->opt_tile_n == 0 || p->opt_tile_n >= 1000) &&
         ((int64_t)((p->n + 127) / 128) * ((p->B + 255) / 256) * 2 <= p->sms ||
-         (int64_t)((p->n + 255) / 256) * ((p->B + 255) / 256) * 4 <= p->sms) &&
-        (e = dalloc(&p->csk_ws, (size_t)p->sms * 256 * 128, s)) != cudaSuccess) {
-      free_run(p);
-      return e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation of the cluster workspace failed")
-                                            : cuda_fail(e, "cudaMalloc");
-    }
+         (int64_t)((p->n + 255) / 256) * ((p->B + 255) / 256) * 4 <= p->sms))
+      al((void**)&p->csk_ws, (size_t)p->sms * 256 * 128 * 4, false);
+  }
+  // grid barrier words of the cluster kernels and the resident sparse form
+  if (ker == KER_TC || (ker == KER_CSR && !p->single)) al((void**)&p->tc_gbar, 3 * sizeof(unsigned int), true);
+  size_t zero_bytes = 0, bytes = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int k = 0; k < n_parts; ++k)
+      if (parts[k].zero == (pass == 0)) bytes += parts[k].bytes;
+    if (pass == 0) zero_bytes = bytes;
+  }
+  cudaStream_t s = p->stream;
+  if (bytes > p->arena_bytes || p->arena_bytes > 2 * bytes) {
+    dfree(p->arena, s);
+    p->arena_bytes = 0;
+    if ((e = dalloc(&p->arena, bytes, s)) == cudaSuccess) p->arena_bytes = bytes;
+  }
+  if (e != cudaSuccess) {
+    free_run(p);
+    return e == cudaErrorMemoryAllocation ? fail(SBO_ENOMEM, "device allocation of the run state failed")
+                                          : cuda_fail(e, "cudaMalloc");
+  }
+  size_t off = 0;
+  for (int pass = 0; pass < 2; ++pass)
+    for (int k = 0; k < n_parts; ++k)
+      if (parts[k].zero == (pass == 0)) {
+        *parts[k].at = p->arena + off;
+        off += parts[k].bytes;
+      }
+  if ((e = cudaMemsetAsync(p->arena, 0, zero_bytes, s)) == cudaSuccess)
+    e = launch_fill_records(p->bestF, p->bestT, p->B, p->trace, p->trace_cap, s);   // sentinels
+  ++p->launches;
+  if (e != cudaSuccess) { free_run(p); return cuda_fail(e, "run state set-up"); }
+  if (ker == KER_TC) {
     int tn = p->tc_split ? 1064 : p->opt_tile_n;   // (1064 falls back to 64 where it does not apply)
     std::string why;
     if (tn == 0 && p->opt_autotune) {
@@ -1744,13 +1737,6 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   }
   p->csr_form = CSR_FORM_RULE;
   if (ker == KER_CSR && !p->single) {
-
-    // grid barrier words of the resident form (allocated before the autotuner, which times it)
-    if ((e = dalloc(&p->tc_gbar, 3, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(p->tc_gbar, 0, 3 * sizeof(unsigned int), s)) != cudaSuccess) {
-      free_run(p);
-      return cuda_fail(e, "grid barrier words");
-    }
     if (p->opt_csr_form != 0) {
       p->csr_form = p->opt_csr_form;
     } else if (p->opt_autotune) {

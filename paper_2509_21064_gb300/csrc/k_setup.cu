@@ -289,14 +289,21 @@ cudaError_t launch_bits_to_operand(const uint8_t* bits, int n, int count, void* 
   return cudaGetLastError();
 }
 
-__global__ void k_fill_i64(long long* p, int64_t count, long long v) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
-    p[e] = v;
+// No record yet: bestF and the trace hold LLONG_MAX, bestT -1.
+__global__ void k_fill_records(long long* bestF, long long* bestT, int64_t B, long long* trace, int64_t cap) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < cap || e < B; e += (int64_t)gridDim.x * blockDim.x) {
+    if (e < cap) trace[e] = 0x7fffffffffffffffll;
+    if (e < B) {
+      bestF[e] = 0x7fffffffffffffffll;
+      bestT[e] = -1;
+    }
+  }
 }
 
-cudaError_t launch_fill_i64(long long* p, int64_t count, long long v, cudaStream_t s) {
-  const int64_t blocks = (count + 255) / 256;
-  k_fill_i64<<<(unsigned)(blocks < 1024 ? (blocks > 0 ? blocks : 1) : 1024), 256, 0, s>>>(p, count, v);
+cudaError_t launch_fill_records(long long* bestF, long long* bestT, int64_t B, long long* trace, int64_t cap,
+                                cudaStream_t s) {
+  const int64_t count = B > cap ? B : cap, blocks = (count + 255) / 256;
+  k_fill_records<<<(unsigned)(blocks < 1024 ? (blocks > 0 ? blocks : 1) : 1024), 256, 0, s>>>(bestF, bestT, B, trace, cap);
   return cudaGetLastError();
 }
 

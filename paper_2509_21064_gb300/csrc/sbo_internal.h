@@ -63,7 +63,8 @@ cudaError_t launch_to_operand_t(const float* X, int n, int B, int64_t ld_in, voi
                                 int op_type, cudaStream_t s);
 cudaError_t launch_bits_to_operand(const uint8_t* bits, int n, int count, void* out, int64_t ld_out,
                                    int layout, int op_type, cudaStream_t s);
-cudaError_t launch_fill_i64(long long* p, int64_t count, long long v, cudaStream_t s);
+cudaError_t launch_fill_records(long long* bestF, long long* bestT, int64_t B, long long* trace, int64_t cap,
+                                cudaStream_t s);
 cudaError_t launch_gather_state(const float* src, int n, int B, int64_t ld, int layout, float* dst_rn,
                                 cudaStream_t s);
 // k_simt.cu  (FP32 A, restart-major state)
