@@ -46,7 +46,7 @@ namespace {
 
 constexpr int CSK_THREADS = 384;   // warp 0 TMA, warp 1 TMEM + MMA, warps 4-11 partial tile; all in the reduction
 constexpr int CSK_SMEM_BUDGET = 196 * 1024;
-constexpr int CSK_MIN_KB = 4;      // k-blocks per CTA at least
+constexpr int CSK_MIN_KB = 2;      // k-blocks per CTA at least
 
 // BN restarts per tile.  PAIR: the tile is 256 rows x BN restarts on a CTA pair (cta_group::2):
 // each CTA stages its own 128 rows of A and BN / 2 restarts of x per k-block.
