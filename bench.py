@@ -594,6 +594,9 @@ def other_configs(S, torch, dev, args, pk, hetero_jobs):
         P.start(S.params(**p.asdict()))
         form = P.info()["tile_n"]     # the sparse update's form chosen by the autotuner
         blocks = 40
+        n0 = P.launch_count()
+        P.run(K)
+        on_chip = P.launch_count() - n0 <= 2   # restart by restart: the state stays on chip within a call
         sec = _timed_blocks(torch, stream, lambda: P.run(K), blocks)
         P.sync()
         P.close()
@@ -606,7 +609,9 @@ def other_configs(S, torch, dev, args, pk, hetero_jobs):
         resident = 16 * n * B * 4 <= l2 * 3
         out[key] = {"n": n, "restarts": B, "precision": prec_name, "eval_every": K, "update_form": form,
                     "us_per_iteration": t_it * 1e6, "restart_iterations_per_s": B / t_it,
-                    "roofline": {"bound": "latency (x, y fit in L2)" if resident else "hbm",
+                    "roofline": {"bound": "instruction issue and shared memory (state on chip for the K iterations of "
+                                          "a call; the bytes are what a pass per iteration would move)" if on_chip
+                                 else "latency (x, y fit in L2)" if resident else "hbm",
                                  "achieved": bytes_it / t_it / 1e9, "peak": hbm, "unit": "GB/s",
                                  "frac": bytes_it / t_it / 1e9 / hbm, "bytes_per_iteration": bytes_it,
                                  "bytes_counted": f"{per} B per (vertex, restart) of state (x, y FP32 read and "

@@ -140,6 +140,25 @@ RestartKernel pick_kernel(const CsrRestartShape& sh, int R, bool bf16) {
 static void place_lanes(int64_t n, const int32_t* rp, const int32_t* col, int BK, std::vector<int32_t>& perm,
                         std::vector<int32_t>& pos) {
   const int64_t slices = (n + 31) / 32;
+  // nothing to do where no two gathers of a pass meet (different vertices on one bank)
+  bool clash = false;
+  for (int64_t p0 = 0; p0 < n && !clash; p0 += BK) {
+    int len = 0;
+    for (int64_t p = p0; p < std::min<int64_t>(n, p0 + BK); ++p)
+      len = std::max(len, rp[perm[(size_t)p] + 1] - rp[perm[(size_t)p]]);
+    for (int k = 0; k < len && !clash; ++k) {
+      int32_t on[32];
+      std::fill(on, on + BK, -1);
+      for (int64_t p = p0; p < std::min<int64_t>(n, p0 + BK); ++p) {
+        const int32_t i = perm[(size_t)p];
+        if (k >= rp[i + 1] - rp[i]) continue;
+        const int32_t q = pos[(size_t)col[rp[i] + k]];
+        clash |= on[q % BK] >= 0 && on[q % BK] != q;
+        on[q % BK] = q;
+      }
+    }
+  }
+  if (!clash) return;
   std::vector<int64_t> first((size_t)slices + 1, 0);   // gather sets (neighbour slots) before each slice
   for (int64_t s = 0; s < slices; ++s) {
     const int32_t i = perm[(size_t)s * 32];             // by descending degree: the longest row
