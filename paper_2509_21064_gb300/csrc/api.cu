@@ -1640,7 +1640,8 @@ sbo_status sbo_gda_start_xy(sbo_problem* p, const sbo_gda_params* prm, const flo
   p->single = p->opt_dual == 1;
   const bool try_restart =
       ker == KER_CSR && !p->single && p->opt_csr_form == 0 && !p->opt_keep_grad && restart_wanted(p);
-  if (try_restart) p->rst_R = csr_restart_pick(p->rst.shape, p->n, p->nnz, p->B, p->sms);
+  if (try_restart)
+    p->rst_R = csr_restart_pick(p->rst.shape, p->n, p->nnz, p->B, prm->iters, p->op_type == OP_BF16, p->sms);
   const bool home = p->rst_R > 0;
   if (ker == KER_MAXK && restart_wanted(p) && maxk_restart_pays(p->rst.shape, p->n, p->nnz, p->kparts, p->B, p->sms))
     p->rst_R = 1;

@@ -305,33 +305,51 @@ bool csr_restart_fits(const CsrRestartShape& sh, int R) {
 // into so that the last round of units leaves no SM idle: with u units on c CTAs, k chunks take
 // ceil(u k / c) chunk times, each a chunk's iterations and about one iteration's time for the load and
 // write-back of the state (4-regular graph n = 20,000, B = 512: 4 rounds -> 3.4).
-static int chunks_for(int units, int ctas, int iters) {
-  if (units <= ctas || units % ctas == 0) return 1;
+// cost: that time in iterations.
+static int chunks_for(int units, int ctas, int iters, double* cost_out = nullptr) {
   int best = 1;
-  double best_cost = 0.0;
-  for (int k = 1; k <= 16 && iters / k >= 16; ++k) {
+  double best_cost = (double)((units + ctas - 1) / ctas) * (iters + 1.0);
+  if (cost_out) *cost_out = best_cost;
+  if (units <= ctas || units % ctas == 0) return 1;
+  for (int k = 2; k <= 16 && iters / k >= 16; ++k) {
     const double cost = (double)(((int64_t)units * k + ctas - 1) / ctas) * ((iters + k - 1) / k + 1.0);
-    if (k == 1 || cost < best_cost) { best = k; best_cost = cost; }
+    if (cost < best_cost) { best = k; best_cost = cost; }
   }
+  if (cost_out) *cost_out = best_cost;
   return best;
 }
 
 // Restarts per CTA of a run, 0: the row-wise kernels.  Both sides' time per iteration (us) from fits to
-// measurements on GB300 (random graphs, n 300-20,000, mean degree 3-50, B 4-512; within about 20 %):
-//   here, rounds of units on the SMs x a unit's time, which grows with its groups, restarts and slices
-//   (n = 20,000, 4-regular, R = 1: 6.0 us; n = 10,000, degree 6, R = 2: 7.9; n = 4,000, degree 50: 13.6,
-//   20.2 and 35 with R = 1, 2, 4);
-//   row-wise, the kernel boundary, and per 128 restarts the rows and their gathers (n = 10,000, degree
-//   6: 8.6 us with B = 100, 21.5 with B = 512; n = 20,000, degree 16: 22 and 69).
-// The line lies near B = 152, degree 10-20 for n = 20,000 (degree 16, B = 512: 72 here, 69 row-wise).
-int csr_restart_pick(const CsrRestartShape& sh, int64_t n, int64_t nnz, int B, int sms) {
-  const int chunks = (B + 127) / 128;
-  double best_us = 3.4 + (chunks > 1 ? 0.9 * chunks : 1.0) * (0.24e-3 * (double)n + 0.042e-3 * (double)nnz);
+// measurements on GB300 (graphs of n 300-20,000, mean degree 3-100, B 16-1,024, weights of one magnitude
+// and of several; FP32 and BF16):
+//   here, rounds of units on the SMs (as chunks_for cuts the run) x a unit's time, which grows with its
+//   groups, restarts and slices (16-bit entries: n = 20,000, 4-regular, R = 1: 5.7 us; n = 10,000, degree
+//   6, R = 2: 7.7; n = 4,000, degree 50: 13.6, 20.1 and 35 with R = 1, 2, 4; 32-bit entries a tenth to a
+//   fifth more; BF16 x 2 to 6 % more, taken as 12 % since the row-wise kernels gain
+//   up to 7 % from it);
+//   row-wise, the kernel boundary and the chain of a long row, per 128 restarts the rows and their gathers,
+//   and the state beyond what L2 keeps (n = 10,000, degree 6: 8.6 us with B = 100, 21.4 with B = 512;
+//   n = 20,000, degree 6: 14.6 and 49; n = 2,000, degree 100: 20.1 with B = 100).
+// The line for n = 20,000, FP32 lies near degree 16 with up to 152 restarts (B = 100: 20.9 here, 22.4
+// row-wise) and between 10 and 16 with B = 512 (49.7 and 56.4 at 10, 70.4 and 70.0 at 16).  Short runs that
+// chunks cannot spread stay row-wise where the last round is mostly idle: n = 20,000, degree 6, BF16,
+// B = 256, a run of 50 iterations 1,375 us here, 1,300 row-wise.  Over 215 measured shapes the choice takes
+// 1.0 % longer than the better side on average; it is the slower one, by 1 to 3 %, at n = 14,000, degree 6,
+// weights of several magnitudes, B = 256 and 1,024, and n = 4,000, degree 50, B = 512.
+int csr_restart_pick(const CsrRestartShape& sh, int64_t n, int64_t nnz, int B, int64_t iters, bool bf16, int sms) {
+  const double nd = (double)n, zd = (double)nnz;
+  double best_us = 3.16 + 0.0853 * zd / std::max(nd, 1.0) +
+                   (1.0 + 0.81 * ((B + 127) / 128 - 1)) * (0.24e-3 * nd + 0.037e-3 * zd) +
+                   0.128e-6 * std::max(0.0, 16.0 * nd * B - 100e6);
   int best = 0;
+  const int span = (int)std::min<int64_t>(std::max<int64_t>(iters, 1), 4096);   // iterations of one launch at most
   for (int R : {1, 2, 4}) {
     if (!csr_restart_fits(sh, R)) continue;
-    const double rounds = std::max(1.0, (double)((B + R - 1) / R) / sms);
-    const double us = rounds * (0.35 + 0.003 * sh.slices + sh.groups * (0.0042 + 0.004 * R));
+    double cost = 0.0;
+    chunks_for((B + R - 1) / R, sms, span, &cost);
+    const double us = cost / (span + 1.0) * (bf16 ? 1.12 : 1.0) *
+                      (sh.narrow ? 0.416 + 0.00128 * sh.slices + sh.groups * (0.00351 + 0.00444 * R)
+                                 : 0.32 + 0.0008 * sh.slices + sh.groups * (0.0048 + 0.0048 * R));
     if (us < best_us) { best = R; best_us = us; }
   }
   return best;

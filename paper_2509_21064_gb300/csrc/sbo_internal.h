@@ -182,7 +182,7 @@ inline int csr_restart_shift(int64_t n) { return n > 10240 ? 2 : 3; }          /
 bool csr_restart_build(int64_t n, const int32_t* rp, const int32_t* col, const int64_t* val, const int64_t* cp,
                        int warps, int bank_lanes, int shift, CsrRestartHost* out);
 bool csr_restart_fits(const CsrRestartShape& sh, int R);   // an instantiation exists and x fits on chip
-int csr_restart_pick(const CsrRestartShape& sh, int64_t n, int64_t nnz, int B, int sms);
+int csr_restart_pick(const CsrRestartShape& sh, int64_t n, int64_t nnz, int B, int64_t iters, bool bf16, int sms);
 size_t csr_restart_positions(const CsrRestartShape& sh);
 cudaError_t launch_csr_restart(const CsrRestartDev& d, const EpiArgs& a, int op_type, const CsrRestartRun& run, int R,
                                int sms, cudaStream_t s);
