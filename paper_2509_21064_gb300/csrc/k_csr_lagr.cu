@@ -10,7 +10,7 @@
 // What bounds it: the shared-memory gathers (as in the runs) and the latency of the load and store
 // phases, one CTA per SM.  The row-wise kernel (k_csr EPI_LAGR) after a transposing conversion moved 32
 // bytes per 4 of x, y and the gradients (a lane's neighbours along i lie n apart): 4-regular n = 20,000,
-// B = 512 170 -> 66 us for L alone and 280 -> 103 us for both gradients (12 and 37 us of bytes).
+// B = 512 170 -> 66 us for L alone and 280 -> 103 us for both gradients (12 and 25 us of bytes).
 #include <algorithm>
 
 #include "csr_restart.cuh"
