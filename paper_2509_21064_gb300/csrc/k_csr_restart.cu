@@ -334,7 +334,7 @@ static int chunks_for(int units, int ctas, int iters, double* cost_out = nullptr
 // row-wise) and between 10 and 16 with B = 512 (49.7 and 56.4 at 10, 70.4 and 70.0 at 16).  Short runs that
 // chunks cannot spread stay row-wise where the last round is mostly idle: n = 20,000, degree 6, BF16,
 // B = 256, a run of 50 iterations 1,375 us here, 1,300 row-wise.  Over 215 measured shapes the choice takes
-// 1.0 % longer than the better side on average; it is the slower one, by 1 to 3 %, at n = 14,000, degree 6,
+// 1.0 % longer than the better side on average; it is the slower one, by 1 to 4 %, at n = 14,000, degree 6,
 // weights of several magnitudes, B = 256 and 1,024, and n = 4,000, degree 50, B = 512.
 int csr_restart_pick(const CsrRestartShape& sh, int64_t n, int64_t nnz, int B, int64_t iters, bool bf16, int sms) {
   const double nd = (double)n, zd = (double)nnz;
